@@ -62,6 +62,26 @@ void make_plan(int L, FftPlan* p) {
     else if (rem == 1) p->rad[p->nst++] = 2;
 }
 
+// w_L^k = exp(-2 pi i k / L), k < L, rounded to 62 fractional bits: {re high, re low, im high,
+// im low} with value high 2^-30 + low 2^-62, low signed.  Angles are reduced to the first
+// octant in integers, so the symmetries of the table hold exactly.
+void fixed_twiddles(int L, int4* out) {
+    for (int k = 0; k < L; ++k) {
+        const int oct = 8 * k / L;                                  // octant of the angle
+        int r = 8 * k - oct * L;                                     // remainder, in units of (2 pi / 8) / L
+        if (oct & 1) r = L - r;
+        const long double ang = 0.78539816339744830961566084581988L * (long double)r / (long double)L;
+        const long double c = std::cos(ang), s = std::sin(ang), one = 4611686018427387904.0L;   // 2^62
+        const long long ci = std::llround(c * one), si = std::llround(s * one);
+        const bool sw = ((oct + 1) & 2) != 0;                        // octants 1, 2, 5, 6
+        long long re = sw ? si : ci, im = sw ? ci : si;
+        if (oct >= 2 && oct < 6) re = -re;
+        if (oct < 4) im = -im;                                       // forward sign
+        const int rl = (int)(unsigned)(unsigned long long)re, il = (int)(unsigned)(unsigned long long)im;
+        out[k] = make_int4((int)((re - rl) >> 32), rl, (int)((im - il) >> 32), il);
+    }
+}
+
 static int pow2_divisor(long long v) {
     int p = 1;
     while (v % (2LL * p) == 0 && p < (1 << 20)) p *= 2;
@@ -70,7 +90,8 @@ static int pow2_divisor(long long v) {
 
 GridPlan::~GridPlan() {
     if (tw32) cudaFree(tw32);
-    if (tw64) cudaFree(tw64);
+    if (twf) cudaFree(twf);
+    if (rcp) cudaFree(rcp);
 }
 
 }  // namespace hmg
@@ -86,8 +107,10 @@ std::shared_ptr<hmg::GridPlan> hmg_ctx::plan(int N) {
     make_plan(M, &gp->pM);
     gp->pN.tw_off = 0;
     gp->pM.tw_off = N;
-    std::vector<double2> h64(N + M);
     std::vector<float2> h32(N + M);
+    std::vector<int4> hf(N + M);
+    fixed_twiddles(N, hf.data());
+    fixed_twiddles(M, hf.data() + N);
     for (int part = 0; part < 2; ++part) {
         const int L = part == 0 ? N : M;
         const int off = part == 0 ? 0 : N;
@@ -101,24 +124,29 @@ std::shared_ptr<hmg::GridPlan> hmg_ctx::plan(int N) {
                 c = (qd == 0) ? 1.0 : (qd == 2 ? -1.0 : 0.0);
                 s = (qd == 1) ? -1.0 : (qd == 3 ? 1.0 : 0.0);
             }
-            h64[off + k] = make_double2(c, s);
             h32[off + k] = make_float2((float)c, (float)s);
         }
     }
-    if (cudaMalloc(&gp->tw64, sizeof(double2) * (N + M)) != cudaSuccess ||
+    if (cudaMalloc(&gp->twf, sizeof(int4) * (N + M)) != cudaSuccess ||
+        cudaMalloc(&gp->rcp, sizeof(long long) * fx_rcp_count(N)) != cudaSuccess ||
         cudaMalloc(&gp->tw32, sizeof(float2) * (N + M)) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    cudaMemcpy(gp->tw64, h64.data(), sizeof(double2) * (N + M), cudaMemcpyHostToDevice);
+    cudaMemcpy(gp->twf, hf.data(), sizeof(int4) * (N + M), cudaMemcpyHostToDevice);
     cudaMemcpy(gp->tw32, h32.data(), sizeof(float2) * (N + M), cudaMemcpyHostToDevice);
+    fx_rcp_table(gp->rcp, N);
+    if (cudaStreamSynchronize(0) != cudaSuccess) {   // the table is read from other streams
+        cudaGetLastError();
+        return nullptr;
+    }
     plans[N] = gp;
     return gp;
 }
 
 namespace hmg {
 
-GridDesc make_desc(const GridPlan& gp, bool fp64, const double k[3], const uint8_t* phase_d,
+GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d, int* exps,
                    int nslots, int scheme, double beta) {
     GridDesc g;
     memset(&g, 0, sizeof(g));
@@ -131,7 +159,8 @@ GridDesc make_desc(const GridPlan& gp, bool fp64, const double k[3], const uint8
     g.pN = gp.pN;
     g.pM = gp.pM;
     g.tw32 = gp.tw32;
-    g.tw64 = gp.tw64;
+    g.twf = gp.twf;
+    g.rcp = gp.rcp;
     const double kmin = std::min(k[0], std::min(k[1], k[2]));
     const double kmax = std::max(k[0], std::max(k[1], k[2]));
     g.scheme = scheme;
@@ -172,20 +201,22 @@ GridDesc make_desc(const GridPlan& gp, bool fp64, const double k[3], const uint8
     for (int s = 0; s < kMaxSlots; ++s)
         for (int c = 0; c < 3; ++c) g.E[s][c] = (s == c) ? 1.0 : 0.0;
     g.nslots = nslots;
-    set_tiles(g, fp64);
+    set_tiles(g);
+    g.expA = exps;
+    g.expB = exps ? exps + 3 * (size_t)nslots * g.NN : nullptr;
     g.phase = phase_d;
     return g;
 }
 
-void set_tiles(GridDesc& g, bool fp64) {
-    const int tile = fp64 ? 1024 : 2048;        // complex values per x-pass CTA buffer
+void set_tiles(GridDesc& g) {
+    const int tile = 2048;                      // complex values per x-pass CTA buffer
     int rows = 1;
     while (rows * 2 * g.M <= tile) rows *= 2;
     rows = std::min(rows, pow2_divisor(g.NN));
     g.rows = rows;
     const int pm = pow2_divisor(g.M);
-    g.Py = std::min(fp64 ? 8 : 16, pm);
-    g.Pz = std::min(fp64 ? 4 : 8, pm);
+    g.Py = std::min(16, pm);
+    g.Pz = std::min(8, pm);
 }
 
 static float time_launches(cudaStream_t st, const std::function<void()>& f, int reps) {
@@ -373,7 +404,7 @@ size_t state_bytes(int N, bool fp64, int nslots) {
     const size_t field32 = (size_t)nslots * 3 * N3 * 4;
     size_t b = N3 + 2 * field64;                        // phase, tau64, spec64
     if (!fp64) b += 3 * field32;                        // f32, r32, spec32
-    b += (size_t)nslots * 3 * 4 * (3 * (size_t)N * N) * 8 + 4096;   // partials
+    b += (size_t)nslots * 3 * 4 * (3 * (size_t)N * N) * 8 + 4096;   // partials, FP64 exponents
     return b;
 }
 
@@ -389,17 +420,18 @@ bool SolveState::ensure(Context* c, int N_, bool fp64_, int nslots_) {
     phase = (uint8_t*)c->alloc(N3);
     tau64 = (double*)c->alloc(f64);
     spec64 = c->alloc(f64);
+    exps = (int*)c->alloc((size_t)nslots * 6 * N * N * sizeof(int));
     if (!fp64) {
         f32buf = (float*)c->alloc(f32);
         r32 = (float*)c->alloc(f32);
         spec32 = c->alloc(f32);
     }
-    const size_t np = (size_t)nslots * 4 * 3 * N * N + 64;
+    const size_t np = (size_t)nslots * 3 * 3 * N * N + 64;   // at least one double per row
     partial = (double*)c->alloc(np * sizeof(double));
     partial2 = (double*)c->alloc(np * sizeof(double));
     partial3 = (double*)c->alloc(np * sizeof(double));
     red = (double*)c->alloc(64 * sizeof(double));
-    bool ok = phase && tau64 && spec64 && partial && partial2 && partial3 && red &&
+    bool ok = phase && tau64 && spec64 && exps && partial && partial2 && partial3 && red &&
               (fp64 || (f32buf && r32 && spec32));
     if (!ok) {
         free_all(c);
@@ -409,7 +441,7 @@ bool SolveState::ensure(Context* c, int N_, bool fp64_, int nslots_) {
 }
 
 void SolveState::free_all(Context* c) {
-    for (void** p : {(void**)&phase, (void**)&tau64, &spec64, (void**)&f32buf, (void**)&r32, &spec32,
+    for (void** p : {(void**)&phase, (void**)&tau64, &spec64, (void**)&exps, (void**)&f32buf, (void**)&r32, &spec32,
                      (void**)&partial, (void**)&partial2, (void**)&partial3, (void**)&red}) {
         c->release(*p);
         *p = nullptr;

@@ -66,7 +66,7 @@ hmg_status prepare(hmg_ctx* ctx, const uint8_t* phase, int N, const double k[3],
     const size_t N3 = (size_t)N * N * N;
     hmg_status st = cuda_status(copy_in(ctx->solve.phase, phase, N3, ctx->stream), "phase copy");
     if (st != HMG_OK) return st;
-    *g = make_desc(*gp, fp64, k, ctx->solve.phase, nslots, scheme, beta);
+    *g = make_desc(*gp, k, ctx->solve.phase, ctx->solve.exps, nslots, scheme, beta);
     if (!fp64) {
         const int v = autotune_z(ctx, *g, &ctx->solve, ctx->stream);
         g->zvar = v & 1;
@@ -525,7 +525,7 @@ static hmg_status fft_common(hmg_ctx* ctx, int N, int count, hmg_precision preci
         return HMG_OUT_OF_MEMORY;
     }
     const double k[3] = {1.0, 1.0, 1.0};
-    GridDesc g = make_desc(*gp, fp64, k, ctx->solve.phase, 1);
+    GridDesc g = make_desc(*gp, k, ctx->solve.phase, ctx->solve.exps, 1);
     if (!fp64) {
         const int v = autotune_z(ctx, g, &ctx->solve, ctx->stream);
         g.zvar = v & 1;

@@ -106,7 +106,7 @@ hmg_status Engine::add(long long id, const uint8_t* phase, int N, const double k
         e->st.free_all(ctx);
         return s;
     }
-    e->g = make_desc(*e->plan, false, k, e->st.phase, 3);
+    e->g = make_desc(*e->plan, k, e->st.phase, e->st.exps, 3);
     {
         const int v = autotune_z(ctx, e->g, &e->st, st);
         e->g.zvar = v & 1;

@@ -48,9 +48,6 @@ template <typename T2> struct TwTable;
 template <> struct TwTable<float2> {
     static __device__ __forceinline__ const float2* get(const GridDesc& g) { return g.tw32; }
 };
-template <> struct TwTable<double2> {
-    static __device__ __forceinline__ const double2* get(const GridDesc& g) { return g.tw64; }
-};
 
 // Radix-R DFT in registers, forward sign exp(-2 pi i/R) or its conjugate.
 template <bool FWD, typename T2> __device__ __forceinline__ void bfly2(T2* v) {

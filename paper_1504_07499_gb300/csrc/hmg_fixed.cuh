@@ -1,0 +1,490 @@
+// FP64 transforms in block fixed point: 64-bit integers with one exponent per pencil.
+//
+// GB300 issues 2 FP64 operations per clock and SM, against 128 32-bit integer adds and 16
+// 32x32+64 multiply-adds (IMAD.WIDE): measured, 0.50 T DFMA/s and 15.8 T 64-bit adds/s.  An
+// FP64 pass is therefore bound by the FP64 pipe (97 % of a sweep; 9.7 ms per gradient at
+// 256^3), and the same butterflies on 64-bit integers cost a tenth of that.
+//
+// Numbers.  A pencil (one 1D transform) holds complex integers v with a common exponent e,
+// value v 2^e.  On load every pencil is scaled so that its largest component fills `first`
+// bits (58 to 60, what the first radix can grow without overflow), so the quantum is at
+// most 2^-58 of the pencil's largest value where FP64 arithmetic rounds each operation to
+// 2^-53 of its own size.  Before each later radix the largest magnitude actually reached
+// decides how far the values are shifted down (mostly not at all), so no bits are given up
+// to worst-case growth.  Data twiddles carry 62 fractional bits.  Errors against 80-bit
+// references are below those of the FP64 passes these replace (see the tests).
+//
+// Between passes the spectrum stays in integers, with the exponent of the pencil that wrote
+// each value in a side array, so only the field side of the x passes converts to and from
+// FP64.  Zero pencils carry a very small exponent, pencils with an infinity or a NaN a very
+// large one that marks everything computed from them as NaN.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "hmg_internal.h"
+
+namespace hmg {
+namespace fx {
+
+struct __align__(16) c64 {
+    long long x, y;
+};
+
+constexpr int kExpZero = -(1 << 20);   // exponent of a pencil that is zero
+constexpr int kExpNan = 1 << 20;       // exponent of a pencil that holds an infinity or a NaN
+#define HMG_HD __host__ __device__ __forceinline__
+
+HMG_HD bool exp_is_nan(int e) { return e > kExpNan / 2; }
+
+HMG_HD c64 mkc(long long x, long long y) { return c64{x, y}; }
+HMG_HD c64 operator+(c64 a, c64 b) { return c64{a.x + b.x, a.y + b.y}; }
+HMG_HD c64 operator-(c64 a, c64 b) { return c64{a.x - b.x, a.y - b.y}; }
+HMG_HD c64 mul_mi(c64 a) { return c64{a.y, -a.x}; }   // -i a
+HMG_HD c64 swap_ri(c64 a) { return c64{a.y, a.x}; }   // conj(a) i: turns a forward DFT into an inverse one
+
+// x = hi 2^32 + lo with lo signed
+HMG_HD int lo_s(long long x) { return (int)(unsigned)(unsigned long long)x; }
+HMG_HD int hi_s(long long x) {
+    return (int)(unsigned)((unsigned long long)x >> 32) + (int)((unsigned)(unsigned long long)x >> 31);
+}
+HMG_HD long long wide(int a, int b) { return (long long)a * (long long)b; }
+
+// x c for a constant |c| < 1/2 given as C = round(c 2^64); error below one unit
+template <long long C>
+HMG_HD long long mulq(long long x) {
+    constexpr int cl = (int)(unsigned)(unsigned long long)C;
+    constexpr int ch = (int)((C - (long long)cl) >> 32);
+    const int xl = lo_s(x), xh = hi_s(x);
+    const long long mid = wide(xh, cl) + (wide(xl, ch) + (1LL << 31));
+    return wide(xh, ch) + (mid >> 32);
+}
+// constants as round(c 2^64); those above 1/2 as 1 - c
+constexpr long long kQ1mR2 = 5402926248376769404LL;    // 1 - sqrt(1/2)
+constexpr long long kQ1mH3 = 2471395088767036514LL;    // 1 - sqrt(3)/2
+constexpr long long kQ1mC8 = 1404174782535421627LL;    // 1 - cos(pi/8)
+constexpr long long kQS8 = 7059263338087549767LL;      // sin(pi/8)
+constexpr long long kQ1mC40 = 4315718282406409839LL;   // 1 - cos(40 deg)
+constexpr long long kQ1mS40 = 6589405544070453923LL;   // 1 - sin(40 deg)
+constexpr long long kQC80 = 3203243492287910726LL;     // cos(80 deg)
+constexpr long long kQ1mS80 = 280247492088382768LL;    // 1 - sin(80 deg)
+constexpr long long kQ1mC20 = 1112474790118499113LL;   // 1 - cos(20 deg)
+constexpr long long kQS20 = 6309158051982071155LL;     // sin(20 deg)
+
+HMG_HD long long mul_r2(long long x) { return x - mulq<kQ1mR2>(x); }
+HMG_HD long long mul_h3(long long x) { return x - mulq<kQ1mH3>(x); }
+HMG_HD long long half(long long x) { return (x + 1) >> 1; }
+
+// a (c - i s) for (c, s) = (1 - C1, S) and the like
+template <long long C1, long long S>
+HMG_HD c64 rot_1c_s(c64 a) {   // c = 1 - C1, s = S
+    return c64{a.x - mulq<C1>(a.x) + mulq<S>(a.y), a.y - mulq<C1>(a.y) - mulq<S>(a.x)};
+}
+template <long long C, long long S1>
+HMG_HD c64 rot_c_1s(c64 a) {   // c = C, s = 1 - S1
+    return c64{mulq<C>(a.x) + (a.y - mulq<S1>(a.y)), mulq<C>(a.y) - (a.x - mulq<S1>(a.x))};
+}
+template <long long C1, long long S1>
+HMG_HD c64 rot_1c_1s(c64 a) {   // c = 1 - C1, s = 1 - S1
+    return c64{a.x - mulq<C1>(a.x) + (a.y - mulq<S1>(a.y)), a.y - mulq<C1>(a.y) - (a.x - mulq<S1>(a.x))};
+}
+HMG_HD c64 rot8(c64 a) { return c64{mul_r2(a.x + a.y), mul_r2(a.y - a.x)}; }   // a exp(-i pi/4)
+
+// a w / 4 for a table twiddle w = (r.h 2^-30 + r.l 2^-62) + i (...) : {r.h, r.l, i.h, i.l}
+HMG_HD c64 cmul4(c64 a, int4 w) {
+    const int xl = lo_s(a.x), xh = hi_s(a.x), yl = lo_s(a.y), yh = hi_s(a.y);
+    const int nih = -w.z, nil = -w.w;
+    const long long r = 1LL << 31;
+    const long long mr = wide(yh, nil) + (wide(xh, w.y) + (wide(yl, nih) + (wide(xl, w.x) + r)));
+    const long long mi = wide(yh, w.y) + (wide(xh, w.w) + (wide(yl, w.x) + (wide(xl, w.z) + r)));
+    return c64{wide(yh, nih) + (wide(xh, w.x) + (mr >> 32)), wide(yh, w.x) + (wide(xh, w.z) + (mi >> 32))};
+}
+HMG_HD int4 conj_tw(int4 w) {
+    w.z = -w.z;
+    w.w = -w.w;
+    return w;
+}
+HMG_HD c64 quarter(c64 a) { return c64{(a.x + 2) >> 2, (a.y + 2) >> 2}; }
+
+// v / 2^s rounded, s in [0, 64]
+HMG_HD long long shr_round(long long v, int s) { return s == 0 ? v : ((v >> (s - 1)) + 1) >> 1; }
+// v 2^sh, rounded when sh < 0
+HMG_HD long long shift(long long v, int sh) {
+    if (sh >= 0) return (long long)((unsigned long long)v << (sh < 63 ? sh : 63));
+    const int s = -sh < 64 ? -sh : 64;
+    return ((v >> (s - 1)) + 1) >> 1;
+}
+HMG_HD c64 shift(c64 v, int sh) { return c64{shift(v.x, sh), shift(v.y, sh)}; }
+HMG_HD c64 shr_round(c64 v, int s) { return c64{shr_round(v.x, s), shr_round(v.y, s)}; }
+
+// the magnitude's high word (|v| <= 2^(32 + its bit length))
+HMG_HD unsigned mag(long long v) {
+    const int h = (int)(v >> 32);
+    return (unsigned)(h ^ (h >> 31));
+}
+HMG_HD unsigned mag(c64 v) { return mag(v.x) | mag(v.y); }
+HMG_HD int clz32(unsigned v) {
+#ifdef __CUDA_ARCH__
+    return __clz((int)v);
+#else
+    return v ? __builtin_clz(v) : 32;
+#endif
+}
+HMG_HD int clz64(unsigned long long v) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)v);
+#else
+    return v ? __builtin_clzll(v) : 64;
+#endif
+}
+HMG_HD int bits_of(unsigned m) { return 64 - clz32(m); }   // of the full 64-bit magnitude
+HMG_HD unsigned long long dbits(double d) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(d);
+#else
+    unsigned long long u;
+    __builtin_memcpy(&u, &d, 8);
+    return u;
+#endif
+}
+HMG_HD double bitsd(unsigned long long u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double d;
+    __builtin_memcpy(&d, &u, 8);
+    return d;
+#endif
+}
+// smallest E with |d| < 2^E (subnormals count as zero)
+HMG_HD int key_of(double d) {
+    const int ex = (int)((dbits(d) >> 52) & 0x7ff);
+    return ex == 0 ? kExpZero : ex == 2047 ? kExpNan : ex - 1022;
+}
+// round(d 2^-e) for |d| < 2^(e + 61)
+HMG_HD long long to_fixed(double d, int e) {
+    const unsigned long long u = dbits(d);
+    const int ex = (int)((u >> 52) & 0x7ff);
+    const unsigned long long m = ex ? ((u << 10) & 0x3ffffffffffffc00ull) | (1ull << 62) : 0ull;   // 1.f at bit 62
+    int r = e + 1084 - ex;                     // one less than the right shift
+    r = r < 0 ? 0 : (r > 63 ? 63 : r);
+    const long long v = (long long)(((m >> r) + 1) >> 1);
+    const long long s = (long long)u >> 63;
+    return (v ^ s) - s;
+}
+// v 2^e as a double, rounded to nearest
+HMG_HD double from_fixed(long long v, int e) {
+    const long long s = v >> 63;
+    const unsigned long long a = (unsigned long long)((v ^ s) - s);
+    const int lz = clz64(a);
+    const unsigned long long n = a << (lz & 63);
+    const int ex = e + 1085 - lz;              // biased exponent, less one (the leading bit adds it)
+    unsigned long long b = (n >> 11) + ((n >> 10) & 1) + ((unsigned long long)(unsigned)ex << 52);
+    if (ex >= 2046) b = 0x7ff0000000000000ull;
+    if (ex < 0 || a == 0) b = 0;
+    return bitsd(b | ((unsigned long long)s & 0x8000000000000000ull));
+}
+
+// ---------------------------------------------------------------------------
+// forward DFTs of small length in registers, natural order in and out
+// ---------------------------------------------------------------------------
+template <int R> struct Dft;
+template <> struct Dft<2> {
+    HMG_HD static void run(c64* v) {
+        const c64 a = v[0];
+        v[0] = a + v[1];
+        v[1] = a - v[1];
+    }
+};
+template <> struct Dft<3> {
+    HMG_HD static void run(c64* v) {
+        const c64 t = v[1] + v[2], u = v[1] - v[2];
+        const c64 m = c64{v[0].x - half(t.x), v[0].y - half(t.y)};
+        const c64 h = c64{mul_h3(u.y), -mul_h3(u.x)};   // -i sqrt(3)/2 u
+        v[0] = v[0] + t;
+        v[1] = m + h;
+        v[2] = m - h;
+    }
+};
+template <> struct Dft<4> {
+    HMG_HD static void run(c64* v) {
+        const c64 a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = mul_mi(v[1] - v[3]);
+        v[0] = a + c;
+        v[1] = b + d;
+        v[2] = a - c;
+        v[3] = b - d;
+    }
+};
+// coprime factors: index maps without twiddles (Good 1958)
+template <> struct Dft<6> {
+    HMG_HD static void run(c64* v) {
+        c64 a[3] = {v[0], v[2], v[4]}, b[3] = {v[3], v[5], v[1]};   // n = 3 a + 2 b mod 6
+        Dft<3>::run(a);
+        Dft<3>::run(b);
+        // k = 3 q + 4 c mod 6 for (k mod 2, k mod 3) = (q, c)
+        v[0] = a[0] + b[0];
+        v[3] = a[0] - b[0];
+        v[4] = a[1] + b[1];
+        v[1] = a[1] - b[1];
+        v[2] = a[2] + b[2];
+        v[5] = a[2] - b[2];
+    }
+};
+template <> struct Dft<12> {
+    HMG_HD static void run(c64* v) {
+        // n = 3 n4 + 4 n3 mod 12, k = 9 k4 + 4 k3 mod 12
+        c64 s[3][4];
+#pragma unroll
+        for (int n3 = 0; n3 < 3; ++n3) {
+#pragma unroll
+            for (int n4 = 0; n4 < 4; ++n4) s[n3][n4] = v[(3 * n4 + 4 * n3) % 12];
+            Dft<4>::run(s[n3]);
+        }
+#pragma unroll
+        for (int k4 = 0; k4 < 4; ++k4) {
+            c64 t[3] = {s[0][k4], s[1][k4], s[2][k4]};
+            Dft<3>::run(t);
+#pragma unroll
+            for (int k3 = 0; k3 < 3; ++k3) v[(9 * k4 + 4 * k3) % 12] = t[k3];
+        }
+    }
+};
+template <> struct Dft<8> {
+    HMG_HD static void run(c64* v) {
+        c64 a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            a[r] = v[r] + v[r + 4];
+            b[r] = v[r] - v[r + 4];
+        }
+        b[1] = rot8(b[1]);
+        b[2] = mul_mi(b[2]);
+        b[3] = mul_mi(rot8(b[3]));
+        Dft<4>::run(a);
+        Dft<4>::run(b);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            v[2 * r] = a[r];
+            v[2 * r + 1] = b[r];
+        }
+    }
+};
+template <> struct Dft<9> {
+    HMG_HD static void run(c64* v) {
+        c64 s[3][3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) s[b][a] = v[3 * a + b];
+            Dft<3>::run(s[b]);
+        }
+        s[1][1] = rot_1c_1s<kQ1mC40, kQ1mS40>(s[1][1]);
+        s[1][2] = rot_c_1s<kQC80, kQ1mS80>(s[1][2]);
+        s[2][1] = rot_c_1s<kQC80, kQ1mS80>(s[2][1]);
+        {   // exp(-i 160 deg) = -exp(+i 20 deg): c = -cos 20, s = sin 20
+            const c64 a = s[2][2];
+            const c64 r = c64{a.x - mulq<kQ1mC20>(a.x), a.y - mulq<kQ1mC20>(a.y)};
+            s[2][2] = c64{mulq<kQS20>(a.y) - r.x, -r.y - mulq<kQS20>(a.x)};
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            c64 t[3] = {s[0][k], s[1][k], s[2][k]};
+            Dft<3>::run(t);
+            v[k] = t[0];
+            v[k + 3] = t[1];
+            v[k + 6] = t[2];
+        }
+    }
+};
+template <> struct Dft<16> {
+    HMG_HD static void run(c64* v) {
+        c64 s[4][4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) s[b][a] = v[4 * a + b];
+            Dft<4>::run(s[b]);
+        }
+        s[1][1] = rot_1c_s<kQ1mC8, kQS8>(s[1][1]);
+        s[1][2] = rot8(s[1][2]);
+        s[1][3] = rot_c_1s<kQS8, kQ1mC8>(s[1][3]);
+        s[2][1] = rot8(s[2][1]);
+        s[2][2] = mul_mi(s[2][2]);
+        s[2][3] = mul_mi(rot8(s[2][3]));
+        s[3][1] = rot_c_1s<kQS8, kQ1mC8>(s[3][1]);
+        s[3][2] = mul_mi(rot8(s[3][2]));
+        {   // exp(-i 9 pi/8) = -exp(-i pi/8)
+            const c64 r = rot_1c_s<kQ1mC8, kQS8>(s[3][3]);
+            s[3][3] = c64{-r.x, -r.y};
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c64 t[4] = {s[0][k], s[1][k], s[2][k], s[3][k]};
+            Dft<4>::run(t);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[k + 4 * q] = t[q];
+        }
+    }
+};
+
+// Component bits a radix may start from: R 2^(b + 1/2) < 2^63 without twiddles (`first`),
+// R 2^(b + 1/2) / 4 < 2^63 and b <= 62 behind the /4 of the twiddle product (`later`).
+constexpr int first_bits(int R) { return R >= 12 ? 58 : R >= 6 ? 59 : R >= 3 ? 60 : 61; }
+constexpr int later_bits(int R) { return R >= 12 ? 60 : R >= 6 ? 61 : 62; }
+
+// Radices of a length (first stage first, 1 = no stage) and threads per pencil: every
+// thread takes whole radix butterflies, one or two per stage.
+template <int R0_, int R1_, int R2_, int T_>
+struct PlanOf {
+    static constexpr int R0 = R0_, R1 = R1_, R2 = R2_, TPP = T_;
+    static constexpr int NS = R2_ > 1 ? 3 : R1_ > 1 ? 2 : 1;
+    static constexpr int L = R0_ * R1_ * R2_;
+    static constexpr int I0 = (L / R0_ + T_ - 1) / T_, I1 = (L / R1_ + T_ - 1) / T_, I2 = (L / R2_ + T_ - 1) / T_;
+    // the last stage: radix, butterflies per thread, product of the stages before it
+    static constexpr int RL = NS == 3 ? R2_ : NS == 2 ? R1_ : R0_;
+    static constexpr int IL = NS == 3 ? I2 : NS == 2 ? I1 : I0;
+    static constexpr int NL = L / RL;
+};
+template <int L> struct Plan;
+template <> struct Plan<4> : PlanOf<4, 1, 1, 1> {};
+template <> struct Plan<6> : PlanOf<6, 1, 1, 1> {};
+template <> struct Plan<8> : PlanOf<8, 1, 1, 1> {};
+template <> struct Plan<9> : PlanOf<9, 1, 1, 1> {};
+template <> struct Plan<12> : PlanOf<4, 3, 1, 4> {};
+template <> struct Plan<16> : PlanOf<4, 4, 1, 4> {};
+template <> struct Plan<18> : PlanOf<6, 3, 1, 6> {};
+template <> struct Plan<24> : PlanOf<6, 4, 1, 6> {};
+template <> struct Plan<27> : PlanOf<9, 3, 1, 9> {};
+template <> struct Plan<32> : PlanOf<8, 4, 1, 8> {};
+template <> struct Plan<36> : PlanOf<6, 6, 1, 6> {};
+template <> struct Plan<48> : PlanOf<8, 6, 1, 8> {};
+template <> struct Plan<54> : PlanOf<9, 6, 1, 9> {};
+template <> struct Plan<64> : PlanOf<8, 8, 1, 8> {};
+template <> struct Plan<72> : PlanOf<9, 8, 1, 9> {};
+template <> struct Plan<81> : PlanOf<9, 9, 1, 9> {};
+template <> struct Plan<96> : PlanOf<12, 8, 1, 12> {};
+template <> struct Plan<108> : PlanOf<12, 9, 1, 12> {};
+template <> struct Plan<128> : PlanOf<16, 8, 1, 8> {};
+template <> struct Plan<144> : PlanOf<12, 12, 1, 12> {};
+template <> struct Plan<162> : PlanOf<9, 6, 3, 27> {};
+template <> struct Plan<192> : PlanOf<16, 12, 1, 16> {};
+template <> struct Plan<216> : PlanOf<6, 6, 6, 36> {};
+template <> struct Plan<243> : PlanOf<9, 9, 3, 27> {};
+template <> struct Plan<256> : PlanOf<16, 16, 1, 16> {};
+template <> struct Plan<288> : PlanOf<6, 6, 8, 48> {};
+template <> struct Plan<324> : PlanOf<9, 6, 6, 54> {};
+template <> struct Plan<384> : PlanOf<8, 8, 6, 64> {};
+template <> struct Plan<432> : PlanOf<9, 8, 6, 72> {};
+template <> struct Plan<486> : PlanOf<9, 9, 6, 81> {};
+template <> struct Plan<512> : PlanOf<8, 8, 8, 64> {};
+
+// Shared-memory slots of a pencil.  Columns: NPEN pencils interleaved (index-major), so
+// neighbouring threads touch neighbouring 16-byte slots.  Rows: one pencil after another,
+// padded by one slot per R0 values where R0 is even, so that the first stage's stores (a
+// stride of R0 slots between threads) fall on distinct banks.
+template <int L, int NPEN, bool ROW>
+struct Slots {
+    static constexpr int PAD = (ROW && Plan<L>::R0 % 2 == 0) ? Plan<L>::R0 : 0;
+    static constexpr int LEN = PAD ? L + L / PAD : L;
+    static constexpr int TOTAL = LEN * NPEN;
+    HMG_HD static int at(int i, int pen) {
+        if constexpr (ROW) return pen * LEN + (PAD ? i + i / (PAD ? PAD : 1) : i);
+        else return i * NPEN + pen;
+    }
+};
+
+#ifdef __CUDACC__
+// One later stage of radix R behind stages of product NSP: read, shift, twiddle, DFT.
+template <int L, int R, int NSP, int IT, class S>
+__device__ __forceinline__ void stage_read(c64 (&v)[IT][R], int t, int pen, const c64* sm, int sh,
+                                           const int4* __restrict__ tw) {
+    constexpr int TPP = Plan<L>::TPP, J = L / R, TS = L / (NSP * R);
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        const int j = t + it * TPP;
+        if (J % TPP == 0 || j < J) {
+            const int k = j % NSP;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[it][r] = sm[S::at(j + r * J, pen)];
+            if (sh) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[it][r] = shr_round(v[it][r], sh);
+            }
+            v[it][0] = quarter(v[it][0]);
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[it][r] = cmul4(v[it][r], __ldg(&tw[k * r * TS]));
+            Dft<R>::run(v[it]);
+        }
+    }
+}
+template <int L, int R, int NSP, int IT, class F>
+__device__ __forceinline__ void stage_emit(const c64 (&v)[IT][R], int t, F f) {
+    constexpr int TPP = Plan<L>::TPP, J = L / R;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        const int j = t + it * TPP;
+        if (J % TPP == 0 || j < J) {
+            const int base = (j / NSP) * NSP * R + j % NSP;
+#pragma unroll
+            for (int r = 0; r < R; ++r) f(base + r * NSP, v[it][r]);
+        }
+    }
+}
+
+// Forward transform of one pencil by its TPP threads.  v: the first stage's inputs,
+// v[it][r] = x[t + it TPP + r L / R0], in at most first_bits(R0) bits, exponent e; the outputs
+// stay in the last stage's registers `o` (exponent e on return): last_emit<L> names their
+// indices.  `or_max`: NS - 1 zeroed words per pencil (stride npen).  The buffer must be free
+// on entry and may still be read by other threads on return.
+template <int L, class S>
+__device__ __forceinline__ void transform(c64 (&v)[Plan<L>::I0][Plan<L>::R0], c64 (&o)[Plan<L>::IL][Plan<L>::RL], int t,
+                                          int pen, c64* sm, unsigned* or_max, int npen, int& e,
+                                          const int4* __restrict__ tw) {
+    using P = Plan<L>;
+#pragma unroll
+    for (int it = 0; it < P::I0; ++it)
+        if ((L / P::R0) % P::TPP == 0 || t + it * P::TPP < L / P::R0) Dft<P::R0>::run(v[it]);
+    if constexpr (P::NS == 1) {
+#pragma unroll
+        for (int it = 0; it < P::I0; ++it)
+#pragma unroll
+            for (int r = 0; r < P::R0; ++r) o[it][r] = v[it][r];
+    } else {
+        unsigned m = 0;
+        stage_emit<L, P::R0, 1, P::I0>(v, t, [&](int k, c64 z) {
+            m |= mag(z);
+            sm[S::at(k, pen)] = z;
+        });
+        atomicOr(&or_max[pen], m);
+        __syncthreads();
+        int sh = max(0, bits_of(or_max[pen]) - later_bits(P::R1));
+        if constexpr (P::NS == 2) {
+            stage_read<L, P::R1, P::R0, P::I1, S>(o, t, pen, sm, sh, tw);
+            e += 2 + sh;
+        } else {
+            c64 u[P::I1][P::R1];
+            stage_read<L, P::R1, P::R0, P::I1, S>(u, t, pen, sm, sh, tw);
+            e += 2 + sh;
+            __syncthreads();   // every thread has read the previous stage
+            m = 0;
+            stage_emit<L, P::R1, P::R0, P::I1>(u, t, [&](int k, c64 z) {
+                m |= mag(z);
+                sm[S::at(k, pen)] = z;
+            });
+            atomicOr(&or_max[npen + pen], m);
+            __syncthreads();
+            sh = max(0, bits_of(or_max[npen + pen]) - later_bits(P::R2));
+            stage_read<L, P::R2, P::R0 * P::R1, P::I2, S>(o, t, pen, sm, sh, tw);
+            e += 2 + sh;
+        }
+    }
+}
+template <int L, class F>
+__device__ __forceinline__ void last_emit(const c64 (&o)[Plan<L>::IL][Plan<L>::RL], int t, F f) {
+    stage_emit<L, Plan<L>::RL, Plan<L>::NL, Plan<L>::IL>(o, t, f);
+}
+#endif  // __CUDACC__
+
+}  // namespace fx
+}  // namespace hmg

@@ -1,0 +1,29 @@
+// FP64 column passes in block fixed point (y passes; z passes of a plain transform).
+#include "hmg_fixed_kernels.cuh"
+
+namespace hmg {
+
+namespace {
+void col(const GridDesc& g, unsigned mask, void* spec, const fx::ColArgs& a, cudaStream_t st) {
+    fx::c64* sp = reinterpret_cast<fx::c64*>(spec);
+    switch (g.N) {
+#define X(N_)                                                                                          \
+    case N_:                                                                                           \
+        fx::launch(fx::k_fxx_col<N_>, dim3(3 * N_ * (N_ / 2 / fx::ColShape<N_>::NP), g.nslots),         \
+                   fx::ColShape<N_>::T, fx::ColShape<N_>::smem, st, g, mask, sp, a);                    \
+        break;
+        HMG_ALL_SIZES(X)
+#undef X
+    }
+}
+}  // namespace
+
+void fx_y(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st) {
+    col(g, mask, spec, fx::ColArgs{0, forward ? 0 : 1, 0, 0, g.expA, g.expB}, st);
+}
+
+void fx_z_plain(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st) {
+    col(g, mask, spec, fx::ColArgs{1, forward ? 0 : 1, forward ? 0 : 1, forward ? 1 : 0, g.expB, g.expA}, st);
+}
+
+}  // namespace hmg

@@ -11,6 +11,11 @@ constexpr int kThreads = 256;      // threads per CTA in every FFT pass
 constexpr int kMaxStages = 12;     // radix stages per 1D transform
 constexpr int kMaxSlots = 3;       // right-hand sides (unit gradients) per RVE
 
+// Every grid size N of the library: even, 2^a 3^b, 8 .. 512.
+#define HMG_ALL_SIZES(X)                                                                             \
+    X(8) X(12) X(16) X(18) X(24) X(32) X(36) X(48) X(54) X(64) X(72) X(96) X(108) X(128) X(144) X(162) \
+    X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
+
 // Mixed-radix Stockham schedule of one 1D length (radices 2, 3, 4, 8).
 struct FftPlan {
     int L;                 // transform length
@@ -27,7 +32,12 @@ struct GridDesc {
     long long NNM;         // complex entries per component spectrum: N*N*M
     FftPlan pN, pM;        // schedules for lengths N (y, z) and M (x)
     const float2* tw32;    // twiddle tables (all lengths, concatenated)
-    const double2* tw64;
+    // FP64 passes in block fixed point (hmg_fixed.cuh): twiddles w_N^k (k < N) then w_M^k
+    // (k < M), projector reciprocals, exponents of the spectrum's pencils (3 N^2 per slot each)
+    const int4* twf;
+    const long long* rcp;
+    int* expA;
+    int* expB;
     // per-phase coefficients, k0 = sqrt(min k * max k):
     double Y[3];           // (k - k0)/(k + k0): polarization factor of the sweep
     double W[3];           // k/(k + k0): flux factor, phi = W tau
@@ -97,14 +107,12 @@ void launch_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* sp
                       const float* r32, float* d32, float* r32_out, double* partial,
                       cudaStream_t st);
 
-// Tile sizes of the generic shared-memory passes (x rows per CTA, y and z columns per CTA)
-// for FP32 or FP64 elements.  FP64 launches always take the FP64 tiles, whatever the
-// descriptor says (the FP32-bulk solver runs its FP64 work on its FP32 descriptor).
-void set_tiles(GridDesc& g, bool fp64);
+// Tile sizes of the generic FP32 shared-memory passes (x rows per CTA, y and z columns per CTA).
+void set_tiles(GridDesc& g);
 int x_ctas(const GridDesc& g);   // CTAs per right-hand side of the generic x passes
 int z_ctas(const GridDesc& g);   // CTAs per right-hand side of the generic z pass
 // CTAs per right-hand side of the x / z passes that launch_* runs for precision R
-// (the register-resident FP32 kernels where one exists, else the generic ones)
+// (FP32: the register-resident kernels where one exists, else the generic ones)
 template <typename R> int x_ctas_for(const GridDesc& g);
 template <typename R> int z_ctas_for(const GridDesc& g);
 
@@ -133,6 +141,19 @@ bool fast_yxy(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec
 bool fast_take_wait_failure();
 int fast_x_ctas(const GridDesc& g);
 int fast_z_ctas(const GridDesc& g);
+
+// FP64 passes (hmg_fixed_*.cu); XI_PLAIN, XI_INPLACE, XI_INPLACE_RES and XI_DIFF.
+int fx_x_ctas(const GridDesc& g);
+int fx_z_ctas(const GridDesc& g);
+void fx_x_forward(const GridDesc& g, int mode, unsigned mask, const double* tau, void* spec, double* partial,
+                  cudaStream_t st);
+void fx_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, double* tau, float* d32, float* r32,
+                  double* partial, cudaStream_t st);
+void fx_y(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st);
+void fx_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st);
+void fx_z_plain(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st);
+inline int fx_rcp_count(int N) { return 3 * (N / 2) * (N / 2) + 1; }
+void fx_rcp_table(long long* rcp, int N);   // device table of fx_rcp_count(N) entries, on the default stream
 
 // Fused x + y passes on thread-block clusters (hmg_fused.cu, FP32); false / 0 when the
 // grid size has no fused kernels.

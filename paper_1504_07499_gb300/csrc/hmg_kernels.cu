@@ -12,7 +12,8 @@
 // e^n - e_comp^n = (tau^n - tau^{n+1}) / (2 k0), so no field but tau is stored.
 // (The basic scheme runs through the same passes on e itself, with its own Y and the
 // Green step -P; GridDesc carries the scheme's coefficients.)  These generic kernels
-// serve FP64 and the sizes without register-resident FP32 kernels (hmg_fast.cu).
+// serve the FP32 sizes without register-resident kernels (hmg_fast.cu); FP64 passes run in
+// block fixed point (hmg_fixed.cuh).
 //
 // Spectrum layout: after the x pass each row of N reals becomes N/2 complex values
 // (x-major rows, same byte size as the real field); entry kx = 0 packs the two real
@@ -125,8 +126,7 @@ k_x_forward(GridDesc g, unsigned mask, const R* __restrict__ tau, typename Cplx<
 template <typename R, int MODE>
 __global__ void __launch_bounds__(kThreads)
 k_x_inverse(GridDesc g, unsigned mask, const typename Cplx<R>::T* __restrict__ spec, R* __restrict__ tau,
-            const float* __restrict__ r32, float* __restrict__ d32, float* __restrict__ r32_out,
-            double* __restrict__ partial) {
+            const float* __restrict__ r32, double* __restrict__ partial) {
     using T2 = typename Cplx<R>::T;
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
@@ -164,8 +164,7 @@ k_x_inverse(GridDesc g, unsigned mask, const typename Cplx<R>::T* __restrict__ s
 
     const long long fbase = (long long)slot * 3 * g.N3 + row0 * N;   // element offset of the tile
     T2* out = reinterpret_cast<T2*>(tau + fbase);
-    // output step: add r (correction sweeps), read the old field for the residual,
-    // or (XI_DIFF) write d = new - old to d32 and r32_out without touching tau
+    // output step: add r (correction sweeps), read the old field for the residual
     constexpr bool kRes = MODE == XI_INPLACE_RES || MODE == XI_ADD_R_RES;
     constexpr bool kAddR = MODE == XI_ADD_R_RES || MODE == XI_ADD_R;
     const bool resid = kRes && (g.dflags ? g.resid != 0 : true);
@@ -179,15 +178,6 @@ k_x_inverse(GridDesc g, unsigned mask, const typename Cplx<R>::T* __restrict__ s
             const T2 o = out[q];
             v = mk(wn * v.x + wo * o.x, wn * v.y + wo * o.y);
         }
-        if (MODE == XI_DIFF) {
-            const T2 o = out[q];
-            const double da = (double)v.x - (double)o.x, db = (double)v.y - (double)o.y;
-            acc += da * da + db * db;
-            const float2 df = make_float2((float)da, (float)db);
-            reinterpret_cast<float2*>(r32_out + fbase)[q] = df;
-            reinterpret_cast<float2*>(d32 + fbase)[q] = df;
-            continue;
-        }
         if (addr) {
             const float2 rv = reinterpret_cast<const float2*>(r32 + fbase)[q];
             v.x += R(rv.x);
@@ -200,9 +190,9 @@ k_x_inverse(GridDesc g, unsigned mask, const typename Cplx<R>::T* __restrict__ s
         }
         out[q] = v;
     }
-    if (kRes || MODE == XI_DIFF) {   // uniform across the CTA
+    if (kRes) {   // uniform across the CTA
         double s = block_sum(acc, red);
-        if (threadIdx.x == 0 && (resid || MODE == XI_DIFF)) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
+        if (threadIdx.x == 0 && resid) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
     }
 }
 
@@ -397,22 +387,14 @@ template <> int x_ctas_for<float>(const GridDesc& g) {
     const int f = fast_x_ctas(g);
     return f ? f : x_ctas(g);
 }
-template <> int x_ctas_for<double>(const GridDesc& g) {
-    GridDesc t = g;
-    set_tiles(t, true);
-    return x_ctas(t);
-}
+template <> int x_ctas_for<double>(const GridDesc& g) { return fx_x_ctas(g); }
 template <> int z_ctas_for<float>(const GridDesc& g) {
     const int f = fast_z_ctas(g);
     return f ? f : z_ctas(g);
 }
-template <> int z_ctas_for<double>(const GridDesc& g) {
-    GridDesc t = g;
-    set_tiles(t, true);
-    return z_ctas(t);
-}
+template <> int z_ctas_for<double>(const GridDesc& g) { return fx_z_ctas(g); }
 
-template <typename R, typename K>
+template <typename K>
 static void set_smem(K kern, size_t bytes) {
     // static (2 KB) plus dynamic shared memory above 48 KB needs the opt-in
     if (bytes > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -421,106 +403,95 @@ static void set_smem(K kern, size_t bytes) {
 template <typename R>
 void launch_x_forward(const GridDesc& g, int mode, unsigned mask, const R* tau, void* spec,
                       double* partial, cudaStream_t st) {
-    using T2 = typename Cplx<R>::T;
-    if constexpr (std::is_same<R, float>::value) {
-        if (fast_x_forward(g, mode, mask, tau, spec, partial, st)) return;
-    }
-    GridDesc t = g;   // FP64 passes take the FP64 tiles
-    if constexpr (std::is_same<R, double>::value) set_tiles(t, true);
-    const size_t sm = 2ull * t.rows * t.M * sizeof(T2);
-    dim3 grid(x_ctas(t), t.nslots);
-    T2* sp = reinterpret_cast<T2*>(spec);
-    if (mode == XF_PLAIN) {
-        set_smem<R>(k_x_forward<R, XF_PLAIN>, sm);
-        k_x_forward<R, XF_PLAIN><<<grid, kThreads, sm, st>>>(t, mask, tau, sp, partial);
-    } else if (mode == XF_POLARIZE) {
-        set_smem<R>(k_x_forward<R, XF_POLARIZE>, sm);
-        k_x_forward<R, XF_POLARIZE><<<grid, kThreads, sm, st>>>(t, mask, tau, sp, partial);
+    if constexpr (std::is_same<R, double>::value) {
+        fx_x_forward(g, mode, mask, tau, spec, partial, st);
     } else {
-        set_smem<R>(k_x_forward<R, XF_FLUX>, sm);
-        k_x_forward<R, XF_FLUX><<<grid, kThreads, sm, st>>>(t, mask, tau, sp, partial);
+        using T2 = typename Cplx<R>::T;
+        if (fast_x_forward(g, mode, mask, tau, spec, partial, st)) return;
+        const size_t sm = 2ull * g.rows * g.M * sizeof(T2);
+        dim3 grid(x_ctas(g), g.nslots);
+        T2* sp = reinterpret_cast<T2*>(spec);
+        if (mode == XF_PLAIN) {
+            set_smem(k_x_forward<R, XF_PLAIN>, sm);
+            k_x_forward<R, XF_PLAIN><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
+        } else if (mode == XF_POLARIZE) {
+            set_smem(k_x_forward<R, XF_POLARIZE>, sm);
+            k_x_forward<R, XF_POLARIZE><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
+        } else {
+            set_smem(k_x_forward<R, XF_FLUX>, sm);
+            k_x_forward<R, XF_FLUX><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
+        }
     }
 }
 
 template <typename R>
 void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st) {
-    using T2 = typename Cplx<R>::T;
-    if constexpr (std::is_same<R, float>::value) {
-        if (fast_y(g, forward, mask, spec, st)) return;
-    }
-    GridDesc t = g;   // FP64 passes take the FP64 tiles
-    if constexpr (std::is_same<R, double>::value) set_tiles(t, true);
-    const size_t sm = 2ull * t.N * t.Py * sizeof(T2);
-    dim3 grid(3 * t.N * (t.M / t.Py), t.nslots);
-    T2* sp = reinterpret_cast<T2*>(spec);
-    if (forward) {
-        set_smem<R>(k_y_pass<R, true>, sm);
-        k_y_pass<R, true><<<grid, kThreads, sm, st>>>(t, mask, sp);
+    if constexpr (std::is_same<R, double>::value) {
+        fx_y(g, forward, mask, spec, st);
     } else {
-        set_smem<R>(k_y_pass<R, false>, sm);
-        k_y_pass<R, false><<<grid, kThreads, sm, st>>>(t, mask, sp);
+        using T2 = typename Cplx<R>::T;
+        if (fast_y(g, forward, mask, spec, st)) return;
+        const size_t sm = 2ull * g.N * g.Py * sizeof(T2);
+        dim3 grid(3 * g.N * (g.M / g.Py), g.nslots);
+        T2* sp = reinterpret_cast<T2*>(spec);
+        if (forward) {
+            set_smem(k_y_pass<R, true>, sm);
+            k_y_pass<R, true><<<grid, kThreads, sm, st>>>(g, mask, sp);
+        } else {
+            set_smem(k_y_pass<R, false>, sm);
+            k_y_pass<R, false><<<grid, kThreads, sm, st>>>(g, mask, sp);
+        }
     }
 }
 
 template <typename R>
 void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st) {
-    using T2 = typename Cplx<R>::T;
-    if constexpr (std::is_same<R, float>::value) {
+    if constexpr (std::is_same<R, double>::value) {
+        if (mode == Z_FWD || mode == Z_INV) fx_z_plain(g, mode == Z_FWD, mask, spec, st);
+        else fx_z(g, mode, mask, spec, partial, st);
+    } else {
+        using T2 = typename Cplx<R>::T;
         if (fast_z(g, mode, mask, spec, partial, st)) return;
-    }
-    GridDesc t = g;   // FP64 passes take the FP64 tiles
-    if constexpr (std::is_same<R, double>::value) set_tiles(t, true);
-    const size_t sm = 2ull * 3 * t.N * t.Pz * sizeof(T2);
-    dim3 grid(z_ctas(t), t.nslots);
-    T2* sp = reinterpret_cast<T2*>(spec);
-    switch (mode) {
-        case Z_FWD:
-            set_smem<R>(k_z_pass<R, Z_FWD>, sm);
-            k_z_pass<R, Z_FWD><<<grid, kThreads, sm, st>>>(t, mask, sp, partial);
-            break;
-        case Z_INV:
-            set_smem<R>(k_z_pass<R, Z_INV>, sm);
-            k_z_pass<R, Z_INV><<<grid, kThreads, sm, st>>>(t, mask, sp, partial);
-            break;
-        case Z_ITER:
-            set_smem<R>(k_z_pass<R, Z_ITER>, sm);
-            k_z_pass<R, Z_ITER><<<grid, kThreads, sm, st>>>(t, mask, sp, partial);
-            break;
-        case Z_ITER_NOB:
-            set_smem<R>(k_z_pass<R, Z_ITER_NOB>, sm);
-            k_z_pass<R, Z_ITER_NOB><<<grid, kThreads, sm, st>>>(t, mask, sp, partial);
-            break;
-        default:
-            set_smem<R>(k_z_pass<R, Z_EQ>, sm);
-            k_z_pass<R, Z_EQ><<<grid, kThreads, sm, st>>>(t, mask, sp, partial);
-            break;
+        const size_t sm = 2ull * 3 * g.N * g.Pz * sizeof(T2);
+        dim3 grid(z_ctas(g), g.nslots);
+        T2* sp = reinterpret_cast<T2*>(spec);
+#define HMG_Z(MODE_)                     \
+    set_smem(k_z_pass<R, MODE_>, sm);    \
+    k_z_pass<R, MODE_><<<grid, kThreads, sm, st>>>(g, mask, sp, partial)
+        switch (mode) {
+            case Z_FWD: HMG_Z(Z_FWD); break;
+            case Z_INV: HMG_Z(Z_INV); break;
+            case Z_ITER: HMG_Z(Z_ITER); break;
+            case Z_ITER_NOB: HMG_Z(Z_ITER_NOB); break;
+            default: HMG_Z(Z_EQ); break;
+        }
+#undef HMG_Z
     }
 }
 
 template <typename R>
 void launch_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, R* tau,
                       const float* r32, float* d32, float* r32_out, double* partial, cudaStream_t st) {
-    using T2 = typename Cplx<R>::T;
-    if constexpr (std::is_same<R, float>::value) {
+    if constexpr (std::is_same<R, double>::value) {
+        fx_x_inverse(g, mode, mask, spec, tau, d32, r32_out, partial, st);
+    } else {
+        using T2 = typename Cplx<R>::T;
         if (fast_x_inverse(g, mode, mask, spec, tau, r32, partial, st)) return;
-    }
-    GridDesc t = g;   // FP64 passes take the FP64 tiles
-    if constexpr (std::is_same<R, double>::value) set_tiles(t, true);
-    const size_t sm = 2ull * t.rows * t.M * sizeof(T2);
-    dim3 grid(x_ctas(t), t.nslots);
-    const T2* sp = reinterpret_cast<const T2*>(spec);
-#define HMG_XI(MODE_)                                                                        \
-    set_smem<R>(k_x_inverse<R, MODE_>, sm);                                                  \
-    k_x_inverse<R, MODE_><<<grid, kThreads, sm, st>>>(t, mask, sp, tau, r32, d32, r32_out, partial)
-    switch (mode) {
-        case XI_PLAIN: HMG_XI(XI_PLAIN); break;
-        case XI_INPLACE: HMG_XI(XI_INPLACE); break;
-        case XI_INPLACE_RES: HMG_XI(XI_INPLACE_RES); break;
-        case XI_ADD_R_RES: HMG_XI(XI_ADD_R_RES); break;
-        case XI_ADD_R: HMG_XI(XI_ADD_R); break;
-        default: HMG_XI(XI_DIFF); break;
-    }
+        const size_t sm = 2ull * g.rows * g.M * sizeof(T2);
+        dim3 grid(x_ctas(g), g.nslots);
+        const T2* sp = reinterpret_cast<const T2*>(spec);
+#define HMG_XI(MODE_)                      \
+    set_smem(k_x_inverse<R, MODE_>, sm);   \
+    k_x_inverse<R, MODE_><<<grid, kThreads, sm, st>>>(g, mask, sp, tau, r32, partial)
+        switch (mode) {
+            case XI_PLAIN: HMG_XI(XI_PLAIN); break;
+            case XI_INPLACE: HMG_XI(XI_INPLACE); break;
+            case XI_INPLACE_RES: HMG_XI(XI_INPLACE_RES); break;
+            case XI_ADD_R_RES: HMG_XI(XI_ADD_R_RES); break;
+            default: HMG_XI(XI_ADD_R); break;
+        }
 #undef HMG_XI
+    }
 }
 
 template <typename R>

@@ -22,10 +22,6 @@
 #include "hmg_internal.h"
 #include "hmg_runtime.h"
 
-namespace hmg {
-void make_plan(int L, FftPlan* p);
-}
-
 using namespace hmg;
 
 namespace {
@@ -39,7 +35,8 @@ static __device__ __align__(256) double g_field[3 * kMaxN3];        // e, then t
 static __device__ __align__(256) double g_spec[3 * kMaxN3];         // tau = (k + k0) e
 static __device__ __align__(256) double g_partial[2 * kMaxPartials];
 static __device__ __align__(256) double g_red[64];
-static __device__ __align__(256) double2 g_tw[kMaxN + kMaxN / 2];
+static __device__ __align__(256) int4 g_tw[kMaxN + kMaxN / 2];
+static __device__ __align__(256) int g_exp[6 * kMaxN * kMaxN];
 
 struct Addrs {
     uint8_t* phase = nullptr;
@@ -47,7 +44,8 @@ struct Addrs {
     double* spec = nullptr;
     double* partial = nullptr;
     double* red = nullptr;
-    double2* tw = nullptr;
+    int4* tw = nullptr;
+    int* exps = nullptr;
 };
 
 std::mutex g_mu;
@@ -65,7 +63,8 @@ bool symbol_address(T** out, const T& sym) {
 hmg_status lookup(Addrs* a) {
     bool ok = symbol_address(&a->phase, g_phase[0]) && symbol_address(&a->field, g_field[0]) &&
               symbol_address(&a->spec, g_spec[0]) && symbol_address(&a->partial, g_partial[0]) &&
-              symbol_address(&a->red, g_red[0]) && symbol_address(&a->tw, g_tw[0]);
+              symbol_address(&a->red, g_red[0]) && symbol_address(&a->tw, g_tw[0]) &&
+              symbol_address(&a->exps, g_exp[0]);
     if (!ok) {
         cudaError_t e = cudaGetLastError();
         set_error("cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
@@ -112,32 +111,20 @@ extern "C" hmg_status hmg_equilibrium_noalloc(const uint8_t* phase, int N, doubl
     const long long N3 = (long long)N * N * N;
     const int M = N / 2;
 
-    // FFT schedules (host only) and the twiddle table of this N in the static array
-    GridPlan gp;
+    // the fixed-point twiddles of this N (kept on the host once computed) into the static array
+    GridPlan gp;   // owns no device table
     gp.N = N;
-    make_plan(N, &gp.pN);
-    make_plan(M, &gp.pM);
-    gp.pN.tw_off = 0;
-    gp.pM.tw_off = N;
-    {
-        double2 h[kMaxN + kMaxN / 2];
-        for (int part = 0; part < 2; ++part) {
-            const int L = part == 0 ? N : M, off = part == 0 ? 0 : N;
-            for (int k = 0; k < L; ++k) {
-                const double ang = 2.0 * M_PI * (double)k / (double)L;
-                double c = std::cos(ang), sn = -std::sin(ang);
-                if ((4 * k) % L == 0) {
-                    const int qd = (4 * k) / L;
-                    c = (qd == 0) ? 1.0 : (qd == 2 ? -1.0 : 0.0);
-                    sn = (qd == 1) ? -1.0 : (qd == 3 ? 1.0 : 0.0);
-                }
-                h[off + k] = make_double2(c, sn);
-            }
-        }
-        // pageable source: the copy has read h when the call returns
-        ce = cudaMemcpyAsync(a->tw, h, sizeof(double2) * (N + M), cudaMemcpyHostToDevice, s);
-        if (ce != cudaSuccess) return cuda_fail(ce, "twiddle upload");
+    static int4 tables[kMaxN / 2 + 1][kMaxN + kMaxN / 2];
+    static bool ready[kMaxN / 2 + 1];
+    int4* h_tw = tables[M];
+    if (!ready[M]) {
+        fixed_twiddles(N, h_tw);
+        fixed_twiddles(M, h_tw + N);
+        ready[M] = true;
     }
+    // pageable source: the copy has read the table when the call returns
+    ce = cudaMemcpyAsync(a->tw, h_tw, sizeof(int4) * (N + M), cudaMemcpyHostToDevice, s);
+    if (ce != cudaSuccess) return cuda_fail(ce, "twiddle upload");
 
     // inputs into the static arrays (host or device sources)
     ce = cudaMemcpyAsync(a->phase, phase, (size_t)N3, cudaMemcpyDefault, s);
@@ -146,15 +133,15 @@ extern "C" hmg_status hmg_equilibrium_noalloc(const uint8_t* phase, int N, doubl
     if (ce != cudaSuccess) return cuda_fail(ce, "input copy");
 
     const double k3[3] = {km, ki, kc};
-    GridDesc g = make_desc(gp, true, k3, a->phase, 1);   // gp owns no device table
-    g.tw64 = a->tw;
+    GridDesc g = make_desc(gp, k3, a->phase, a->exps, 1);
+    g.twf = a->tw;
     // e (in g_field) -> tau = (k + k0) e (in g_spec) -> packed spectrum (in g_field)
     launch_e_to_tau<double>(g, 0, a->field, a->spec, s);
     launch_x_forward<double>(g, XF_FLUX, 1u, a->spec, a->field, a->partial, s);
-    launch_reduce(a->partial, 1, x_ctas(g), 3, a->red + 16, s);
+    launch_reduce(a->partial, 1, fx_x_ctas(g), 3, a->red + 16, s);
     launch_y_pass<double>(g, true, 1u, a->field, s);
     launch_z_pass<double>(g, Z_EQ, 1u, a->field, a->partial + kMaxPartials, s);
-    launch_reduce(a->partial + kMaxPartials, 1, z_ctas(g), 1, a->red + 32, s);
+    launch_reduce(a->partial + kMaxPartials, 1, fx_z_ctas(g), 1, a->red + 32, s);
     double h[48];
     ce = cudaGetLastError();
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(h, a->red + 16, 32 * sizeof(double), cudaMemcpyDeviceToHost, s);

@@ -19,6 +19,7 @@ void set_error(const char* fmt, ...);
 extern thread_local std::string g_last_error;
 
 bool valid_length(int L);
+void fixed_twiddles(int L, int4* out);
 bool valid_N(int N);
 bool is_device_ptr(const void* p);
 cudaError_t copy_in(void* dst_dev, const void* src, size_t bytes, cudaStream_t st);
@@ -44,7 +45,8 @@ struct GridPlan {
     int N = 0;
     FftPlan pN{}, pM{};
     float2* tw32 = nullptr;
-    double2* tw64 = nullptr;
+    int4* twf = nullptr;          // FP64 passes: fixed-point twiddles and projector reciprocals
+    long long* rcp = nullptr;
     ~GridPlan();
 };
 
@@ -55,7 +57,8 @@ struct SolveState {
     int nslots = 0;
     uint8_t* phase = nullptr;
     double* tau64 = nullptr;
-    void* spec64 = nullptr;
+    void* spec64 = nullptr;       // block fixed point (hmg_fixed.cuh) between the FP64 passes
+    int* exps = nullptr;          // its exponents: 6 N^2 per slot
     float* f32buf = nullptr;
     float* r32 = nullptr;
     void* spec32 = nullptr;
@@ -68,7 +71,8 @@ struct SolveState {
     void free_all(::hmg_ctx* c);
 };
 
-GridDesc make_desc(const GridPlan& gp, bool fp64, const double k[3], const uint8_t* phase_d, int nslots,
+// exps: 6 N^2 nslots integers of scratch for the FP64 passes (SolveState::exps).
+GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d, int* exps, int nslots,
                    int scheme = HMG_SCHEME_EYRE_MILTON, double beta = 2.0);
 
 // Pick the faster z-pass variant of the FP32 register-resident path for g.N by timing
