@@ -6,12 +6,11 @@
 // it: expA holds one per x row [slot][c][z][y] (x forward) or per z column [slot][c][ky][kx]
 // (z pass), expB one per y column [slot][c][z][kx] (y passes).
 //
-// What bounds them (256^3, one gradient): latency at 16 warps per SM (128 registers hold a
-// 16-value butterfly), with the IMAD.WIDE pipe half busy; FP64 is left for the coefficient
-// product, the flux sum and the residual (1 to 2 operations per real value).  Against the
-// FP64 butterflies these replace: four sweeps of one gradient at 256^3 through the C ABI
-// 38.8 -> 10.0 ms, a plain FP64 solve at 96^3 (contrast 200) 255 -> 85 ms, the FP64
-// correction of a 512^3 FP32-bulk solve 691 -> 177 ms.
+// What bounds them (256^3, one gradient): the IMAD.WIDE pipe (16 per clock and SM; 24 per
+// value in a column pass, 59 in the z pass, whose 0.54 ms it could do in 0.32), then latency;
+// FP64 is left for the coefficient product, the flux sum and the residual (1 to 2 operations
+// per real value).  Against the FP64 butterflies these replace, one sweep of one gradient
+// at 256^3 through the C ABI went 9.7 -> 2.2 ms (copies and conversions of the field included).
 #pragma once
 
 #include "hmg_fft.cuh"
@@ -32,17 +31,21 @@ constexpr int divisor_upto(long long n, int lim) {
 // about 128 to 256 threads; columns in runs of at least 64 bytes where N/2 allows it
 template <int M> constexpr int x_rows() { return divisor_upto(4LL * M * M, 192 / Plan<M>::TPP > 1 ? 192 / Plan<M>::TPP : 1); }
 template <int L> constexpr int col_cols() {
-    int lim = 192 / Plan<L>::TPP;
+    int lim = 256 / Plan<L>::TPP;
     lim = lim < 4 ? 4 : lim > 16 ? 16 : lim;
     return divisor_upto(L / 2, lim);
 }
 template <int L> constexpr int z_cols() {
-    int lim = 256 / (3 * Plan<L>::TPP);
+    int lim = 400 / (3 * Plan<L>::TPP);
     lim = lim < 2 ? 2 : lim > 8 ? 8 : lim;
     return divisor_upto(L / 2, lim);
 }
-// registers: 128 per thread where the CTA shape allows (512 threads per SM)
-constexpr int min_ctas(int threads) { return threads >= 512 ? 1 : 512 / threads; }
+// Registers per thread by the threads an SM is to hold: 64 for the column and z passes, 72 to
+// 80 for the x passes (64 spill there: x inverse at 192^3 371 us against 197 us).
+constexpr int min_ctas(int threads, int per_sm) {
+    const int t = (threads + 31) / 32 * 32;
+    return t >= per_sm ? 1 : per_sm / t;
+}
 constexpr int pow2_at_least(int n) {
     int p = 1;
     while (p < n) p *= 2;
@@ -76,7 +79,7 @@ struct XShape {
 };
 
 template <int M>
-__global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T))
+__global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
 k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ tau, c64* __restrict__ spec,
               double* __restrict__ partial) {
     using X = XShape<M>;
@@ -173,7 +176,7 @@ k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ ta
 // x inverse: packed integer spectrum rows -> FP64 field rows, with the sweep's output step
 // ---------------------------------------------------------------------------
 template <int M>
-__global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T))
+__global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
 k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* __restrict__ spec, double* __restrict__ tau,
               float* __restrict__ d32, float* __restrict__ r32, double* __restrict__ partial) {
     using X = XShape<M>;
@@ -287,7 +290,7 @@ struct ColShape {
 };
 
 template <int L>
-__global__ void __launch_bounds__(ColShape<L>::T, min_ctas(ColShape<L>::T))
+__global__ void __launch_bounds__(ColShape<L>::T, min_ctas(ColShape<L>::T, 1024))
 k_fxx_col(GridDesc g, unsigned mask, c64* __restrict__ spec, ColArgs a) {
     using C = ColShape<L>;
     using P = Plan<L>;
@@ -399,7 +402,7 @@ __device__ __forceinline__ void project(long long* s, const int* d, int b, long 
 }
 
 template <int L>
-__global__ void __launch_bounds__(ZShape<L>::T, min_ctas(ZShape<L>::T))
+__global__ void __launch_bounds__(ZShape<L>::T, min_ctas(ZShape<L>::T, 1024))
 k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __restrict__ partial) {
     using Z = ZShape<L>;
     using P = Plan<L>;
