@@ -6,62 +6,97 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "hmg_internal.h"
 
 namespace hmg {
 
-constexpr int kVoxChunk = 512;       // spheres staged in shared memory per pass
-constexpr int kVoxPerThread = 4;     // consecutive x voxels per thread
+constexpr int kVoxChunk = 512;       // spheres (cylinders) staged in shared memory per pass
+constexpr int kVoxPerThread = 4;     // consecutive x voxels per thread (cylinders)
 
-__device__ __forceinline__ long long axis_d2(long long v, long long c, long long S) {
+__device__ __forceinline__ long long axis_d(long long v, long long c, long long S) {
     long long d = v - c;
     if (d < 0) d += S;
     const long long e = S - d;
-    d = d < e ? d : e;
-    return d * d;
+    return d < e ? d : e;
 }
 
-// One CTA covers a run of kThreads * kVoxPerThread voxels along x-major order.
+// Spheres.  A CTA covers `rows` whole x rows of one z plane; a thread a run of kRun voxels of
+// one row.  Each chunk of spheres is first cut down to those that reach the CTA's band of
+// rows: the z distance is one value, and a row y of the band lies within half a band of its
+// middle, so a sphere whose y distance to the middle exceeds that by more than the radius
+// left at this z cannot reach it.  A voxel then sees the few spheres of its band (about 5 of
+// 100 at 40 %) instead of all of them, and its row's squared distance is formed once per run.
+// Bound by the 64-bit compares of the voxels near spheres; 256^3 with 100 spheres through the
+// C ABI 4.26 -> 0.088 ms (every voxel against every sphere before).
+constexpr int kRun = 16;
+
 __global__ void __launch_bounds__(kThreads)
-k_voxelize(const long long* __restrict__ q, int n, int N, long long S, uint8_t* __restrict__ out) {
-    __shared__ long long sq[kVoxChunk * 5];
-    const long long N3 = (long long)N * N * N;
-    const long long first = ((long long)blockIdx.x * kThreads + threadIdx.x) * kVoxPerThread;
-    const long long G2 = 2 * 4096;
-    long long d2yz[kVoxPerThread];
-    long long vx[kVoxPerThread], vy[kVoxPerThread], vz[kVoxPerThread];
-    int ph[kVoxPerThread];
-#pragma unroll
-    for (int t = 0; t < kVoxPerThread; ++t) {
-        const long long i = first + t;
-        const long long ii = i < N3 ? i : 0;
-        const long long x = ii % N, y = (ii / N) % N, z = ii / ((long long)N * N);
-        vx[t] = x * G2 + 4096;
-        vy[t] = y * G2 + 4096;
-        vz[t] = z * G2 + 4096;
-        ph[t] = 0;
-        d2yz[t] = 0;
-    }
+k_voxelize(const long long* __restrict__ q, int n, int N, long long S, int rows, bool vec, uint8_t* __restrict__ out) {
+    __shared__ long long sx[kVoxChunk], sy[kVoxChunk], sz2[kVoxChunk], so[kVoxChunk], si[kVoxChunk];
+    __shared__ int cnt;
+    const long long G = 4096;
+    const int bands = (N + rows - 1) / rows;
+    const int z = blockIdx.x / bands, y0 = blockIdx.x % bands * rows;
+    const int runs = (N + kRun - 1) / kRun;                  // runs per row
+    const int y = y0 + threadIdx.x / runs, x0 = threadIdx.x % runs * kRun;
+    const bool mine = threadIdx.x < rows * runs && y < N;
+    const long long vz = (2 * z + 1) * G, vy = (2 * y + 1) * G;
+    const int ylast = min(y0 + rows, N) - 1;
+    const long long ymid = (y0 + ylast + 1) * G, yhalf = (ylast - y0) * G;   // rows lie in ymid +- yhalf
+    unsigned core = 0, outer = 0;                            // one bit per voxel of the run
     for (int base = 0; base < n; base += kVoxChunk) {
-        const int cnt = (n - base) < kVoxChunk ? (n - base) : kVoxChunk;
+        __syncthreads();                                     // the list of the chunk before has been read
+        if (threadIdx.x == 0) cnt = 0;
         __syncthreads();
-        for (int k = threadIdx.x; k < cnt * 5; k += blockDim.x) sq[k] = q[(long long)base * 5 + k];
+        for (int k = threadIdx.x; k < min(n - base, kVoxChunk); k += blockDim.x) {
+            const long long* c = q + (long long)(base + k) * 5;
+            const long long dz = axis_d(vz, c[2], S), dz2 = dz * dz;
+            const long long dy = max(axis_d(ymid, c[1], S) - yhalf, 0LL);   // least y distance of the band's rows
+            if (dz2 + dy * dy <= c[3]) {
+                const int s = atomicAdd(&cnt, 1);
+                sx[s] = c[0];
+                sy[s] = c[1];
+                sz2[s] = dz2;
+                so[s] = c[3];
+                si[s] = c[4];
+            }
+        }
         __syncthreads();
+        if (!mine) continue;
         for (int s = 0; s < cnt; ++s) {
-            const long long cx = sq[5 * s], cy = sq[5 * s + 1], cz = sq[5 * s + 2];
-            const long long ro2 = sq[5 * s + 3], ri2 = sq[5 * s + 4];
+            const long long dy = axis_d(vy, sy[s], S);
+            const long long d2 = sz2[s] + dy * dy;
+            const long long ro = so[s] - d2, ri = si[s] - d2;   // what is left for dx^2
+            if (ro < 0) continue;
 #pragma unroll
-            for (int t = 0; t < kVoxPerThread; ++t) {
-                const long long d2 = axis_d2(vx[t], cx, S) + axis_d2(vy[t], cy, S) + axis_d2(vz[t], cz, S);
-                if (d2 <= ri2) ph[t] = 1;
-                else if (d2 <= ro2 && ph[t] == 0) ph[t] = 2;
+            for (int t = 0; t < kRun; ++t) {
+                int dx = (2 * (x0 + t) + 1) * (int)G - (int)sx[s];   // S <= 2^22: 32-bit distances
+                if (dx < 0) dx += (int)S;
+                dx = min(dx, (int)S - dx);
+                const long long dx2 = (long long)dx * dx;
+                outer |= (dx2 <= ro ? 1u : 0u) << t;
+                core |= (dx2 <= ri ? 1u : 0u) << t;
             }
         }
     }
+    if (!mine) return;
+    uint8_t* o = out + ((long long)z * N + y) * N + x0;
+    if (vec) {   // N a multiple of kRun, output 16-byte aligned
+        unsigned w[kRun / 4];
 #pragma unroll
-    for (int t = 0; t < kVoxPerThread; ++t) {
-        const long long i = first + t;
-        if (i < N3) out[i] = (uint8_t)ph[t];
+        for (int i = 0; i < kRun / 4; ++i) {
+            w[i] = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const unsigned c = core >> (4 * i + t) & 1u, e = outer >> (4 * i + t) & 1u;
+                w[i] |= (c ? 1u : 2u * e) << (8 * t);
+            }
+        }
+        *reinterpret_cast<uint4*>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+        for (int t = 0; t < kRun && x0 + t < N; ++t) o[t] = (uint8_t)(core >> t & 1u ? 1u : 2u * (outer >> t & 1u));
     }
 }
 
@@ -135,10 +170,9 @@ void launch_voxelize_cyl(const long long* q, int n, int N, long long S, uint8_t*
 }
 
 void launch_voxelize(const long long* q, int n, int N, long long S, uint8_t* out, cudaStream_t st) {
-    const long long N3 = (long long)N * N * N;
-    const long long per = (long long)kThreads * kVoxPerThread;
-    const int blocks = (int)((N3 + per - 1) / per);
-    k_voxelize<<<blocks, kThreads, 0, st>>>(q, n, N, S, out);
+    const int runs = (N + kRun - 1) / kRun, rows = std::max(1, std::min(N, kThreads / runs));
+    const bool vec = N % kRun == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+    k_voxelize<<<N * ((N + rows - 1) / rows), kThreads, 0, st>>>(q, n, N, S, rows, vec, out);
 }
 
 }  // namespace hmg
