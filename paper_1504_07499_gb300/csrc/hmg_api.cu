@@ -369,17 +369,24 @@ int autotune_z(::hmg_ctx* c, GridDesc g, SolveState* s, cudaStream_t st) {
 
 }  // namespace hmg
 
+bool hmg_ctx::reserve(size_t bytes) {
+    size_t cur = pool->used.load();
+    do {
+        if (pool->limit && cur + bytes > pool->limit) return false;
+    } while (!pool->used.compare_exchange_weak(cur, cur + bytes));
+    return true;
+}
+
+void hmg_ctx::unreserve(size_t bytes) { pool->used -= bytes; }
+
 void* hmg_ctx::alloc(size_t bytes) {
     if (bytes == 0) return nullptr;
     // reserve the bytes in the (possibly shared) budget first
-    size_t cur = pool->used.load();
-    do {
-        if (pool->limit && cur + bytes > pool->limit) return nullptr;
-    } while (!pool->used.compare_exchange_weak(cur, cur + bytes));
+    if (!reserve(bytes)) return nullptr;
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
-        pool->used -= bytes;
+        unreserve(bytes);
         return nullptr;
     }
     sizes[p] = bytes;
@@ -394,6 +401,21 @@ void hmg_ctx::release(void* p) {
         sizes.erase(it);
     }
     cudaFree(p);
+}
+
+void* hmg_ctx::scratch_get(size_t bytes) {
+    if (bytes <= kScratchBytes && scratch) return scratch;
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes <= kScratchBytes ? kScratchBytes : bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (bytes <= kScratchBytes) scratch = p;
+    return p;
+}
+
+void hmg_ctx::scratch_put(void* p) {
+    if (p && p != scratch) cudaFree(p);
 }
 
 namespace hmg {

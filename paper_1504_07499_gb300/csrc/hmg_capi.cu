@@ -138,6 +138,7 @@ hmg_status hmg_destroy(hmg_ctx* ctx) {
         }
         cudaStreamSynchronize(ctx->stream);
         ctx->solve.free_all(ctx);
+        if (ctx->scratch) cudaFree(ctx->scratch);
         ctx->plans.clear();
         cudaStreamSynchronize(ctx->stream64);
         cudaStreamDestroy(ctx->stream64);
@@ -255,17 +256,21 @@ hmg_status voxelize_impl(hmg_ctx* ctx, const hmg_sphere* spheres, size_t n, cons
         }
     }
     // the spheres must not overlap (periodic minimum image; touching is allowed)
+    std::vector<double> w(3 * n);   // centres wrapped into the unit cube
+    for (size_t i = 0; i < n; ++i) {
+        const double a[3] = {h[i].cx, h[i].cy, h[i].cz};
+        for (int c = 0; c < 3; ++c) w[3 * i + c] = a[c] - std::floor(a[c]);
+    }
     for (size_t i = 0; i < n; ++i)
         for (size_t j = i + 1; j < n; ++j) {
+            const double rr = h[i].r + h[j].r, lim = rr * rr * (1.0 - 1e-12);
             double d2 = 0.0;
-            const double a[3] = {h[i].cx, h[i].cy, h[i].cz}, b[3] = {h[j].cx, h[j].cy, h[j].cz};
-            for (int c = 0; c < 3; ++c) {
-                double d = std::fabs((a[c] - std::floor(a[c])) - (b[c] - std::floor(b[c])));
+            for (int c = 0; c < 3 && d2 < lim; ++c) {   // the sum only grows: most pairs end at x
+                double d = std::fabs(w[3 * i + c] - w[3 * j + c]);
                 d = std::min(d, 1.0 - d);
                 d2 += d * d;
             }
-            const double rr = h[i].r + h[j].r;
-            if (d2 < rr * rr * (1.0 - 1e-12)) {
+            if (d2 < lim) {
                 set_error("spheres %zu and %zu overlap", i, j);
                 return HMG_INVALID_ARG;
             }
@@ -311,9 +316,10 @@ hmg_status voxelize_impl(hmg_ctx* ctx, const hmg_sphere* spheres, size_t n, cons
     const size_t N3 = (size_t)N * N * N;
     const bool dev_out = is_device_ptr(phase_out);
     const size_t qbytes = (q.size() + qc.size()) * sizeof(long long);
-    if (cudaMalloc(&qd, qbytes) != cudaSuccess || (!dev_out && cudaMalloc(&tmp, N3) != cudaSuccess)) {
+    qd = (long long*)ctx->scratch_get(qbytes);
+    if (!qd || (!dev_out && cudaMalloc(&tmp, N3) != cudaSuccess)) {
         cudaGetLastError();
-        if (qd) cudaFree(qd);
+        ctx->scratch_put(qd);
         set_error("cannot allocate voxelization buffers");
         return HMG_OUT_OF_MEMORY;
     }
@@ -328,7 +334,7 @@ hmg_status voxelize_impl(hmg_ctx* ctx, const hmg_sphere* spheres, size_t n, cons
     if (ev >= 0) ctx->tracer.end(ev, HMG_K_OTHER, (double)N3, ctx->stream);
     if (!dev_out) cudaMemcpyAsync(phase_out, tmp, N3, cudaMemcpyDeviceToHost, ctx->stream);
     st = check_launch(ctx, "voxelize");
-    cudaFree(qd);
+    ctx->scratch_put(qd);
     if (tmp) cudaFree(tmp);
     return st;
 }

@@ -181,12 +181,20 @@ struct hmg_ctx {
     std::map<int, std::shared_ptr<hmg::GridPlan>> plans;
     hmg::SolveState solve;
     std::shared_ptr<hmg::GridPlan> plan(int N);
+    bool reserve(size_t bytes);     // of the budget
+    void unreserve(size_t bytes);
     void* alloc(size_t bytes);
     void release(void* p);
     hmg::Server* server = nullptr;
     std::mutex server_mu;              // guards the creation of `server`
     hmg::Tracer tracer;
     std::map<int, int> ztune;   // autotuned z-pass variant per grid size (FP32 path)
+    // Device scratch of the placement and voxelization calls (sphere lists), kept for the
+    // life of the context; a larger need allocates for the call.
+    static constexpr size_t kScratchBytes = 64 * 1024;
+    void* scratch = nullptr;
+    void* scratch_get(size_t bytes);   // nullptr: out of device memory
+    void scratch_put(void* p);
 };
 
 namespace hmg {
