@@ -35,7 +35,7 @@ void set_error(const char* fmt, ...) {
 }
 
 // ---------------------------------------------------------------------------
-// FFT schedules and twiddles
+// grid sizes and twiddles
 // ---------------------------------------------------------------------------
 
 bool valid_length(int L) {
@@ -46,21 +46,6 @@ bool valid_length(int L) {
 }
 
 bool valid_N(int N) { return N >= 8 && N <= 512 && N % 2 == 0 && valid_length(N); }
-
-void make_plan(int L, FftPlan* p) {
-    int a = 0, b = 0, t = L;
-    while (t % 2 == 0) { t /= 2; ++a; }
-    while (t % 3 == 0) { t /= 3; ++b; }
-    p->L = L;
-    p->nst = 0;
-    for (int i = 0; i < b; ++i) p->rad[p->nst++] = 3;
-    int n8 = a / 3, rem = a % 3;
-    if (rem == 1 && n8 > 0) { --n8; rem = 4; }  // 16 = 4 * 4 instead of 8 * 2
-    for (int i = 0; i < n8; ++i) p->rad[p->nst++] = 8;
-    if (rem == 4) { p->rad[p->nst++] = 4; p->rad[p->nst++] = 4; }
-    else if (rem == 2) p->rad[p->nst++] = 4;
-    else if (rem == 1) p->rad[p->nst++] = 2;
-}
 
 // w_L^k = exp(-2 pi i k / L), k < L, rounded to 62 fractional bits: {re high, re low, im high,
 // im low} with value high 2^-30 + low 2^-62, low signed.  Angles are reduced to the first
@@ -82,12 +67,6 @@ void fixed_twiddles(int L, int4* out) {
     }
 }
 
-static int pow2_divisor(long long v) {
-    int p = 1;
-    while (v % (2LL * p) == 0 && p < (1 << 20)) p *= 2;
-    return p;
-}
-
 GridPlan::~GridPlan() {
     if (tw32) cudaFree(tw32);
     if (twf) cudaFree(twf);
@@ -103,10 +82,6 @@ std::shared_ptr<hmg::GridPlan> hmg_ctx::plan(int N) {
     auto gp = std::make_shared<GridPlan>();
     gp->N = N;
     const int M = N / 2;
-    make_plan(N, &gp->pN);
-    make_plan(M, &gp->pM);
-    gp->pN.tw_off = 0;
-    gp->pM.tw_off = N;
     std::vector<float2> h32(N + M);
     std::vector<int4> hf(N + M);
     fixed_twiddles(N, hf.data());
@@ -156,8 +131,6 @@ GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d
     g.NN = (long long)N * N;
     g.N3 = g.NN * N;
     g.NNM = g.NN * M;
-    g.pN = gp.pN;
-    g.pM = gp.pM;
     g.tw32 = gp.tw32;
     g.twf = gp.twf;
     g.rcp = gp.rcp;
@@ -201,22 +174,10 @@ GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d
     for (int s = 0; s < kMaxSlots; ++s)
         for (int c = 0; c < 3; ++c) g.E[s][c] = (s == c) ? 1.0 : 0.0;
     g.nslots = nslots;
-    set_tiles(g);
     g.expA = exps;
     g.expB = exps ? exps + 3 * (size_t)nslots * g.NN : nullptr;
     g.phase = phase_d;
     return g;
-}
-
-void set_tiles(GridDesc& g) {
-    const int tile = 2048;                      // complex values per x-pass CTA buffer
-    int rows = 1;
-    while (rows * 2 * g.M <= tile) rows *= 2;
-    rows = std::min(rows, pow2_divisor(g.NN));
-    g.rows = rows;
-    const int pm = pow2_divisor(g.M);
-    g.Py = std::min(16, pm);
-    g.Pz = std::min(8, pm);
 }
 
 static float time_launches(cudaStream_t st, const std::function<void()>& f, int reps) {
@@ -345,7 +306,7 @@ int autotune_z(::hmg_ctx* c, GridDesc g, SolveState* s, cudaStream_t st) {
     int xpbest = 0;
     g.zvar = zbest;
     g.xyvar = xybest;
-    if (chain_sweeps(g)) {
+    if (chain_sweeps(g) && fast_x_ctas(g)) {
         float xms[2];
         for (int v = 0; v < 2; ++v) {
             g.xpers = v;

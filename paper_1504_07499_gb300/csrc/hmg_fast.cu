@@ -60,7 +60,7 @@ k_fy(GridDesc g, unsigned mask, float2* __restrict__ spec) {
     float2 v[E];
 #pragma unroll
     for (int n1 = 0; n1 < E; ++n1) v[n1] = base[(long long)(TP * n1 + t) * M];
-    const float2* twL = g.tw32 + g.pN.tw_off;
+    const float2* twL = g.tw32;
     stage1_write<L, FWD>(v, t, twL, sh + p, P);
     __syncthreads();
     stage2_read<L, FWD>(v, t, sh + p, P);
@@ -115,7 +115,7 @@ k_fz3(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__
     const int kx = kb * P + p;
     float2* base = spec + (long long)slot * 3 * NNM + (long long)ky * M + kb * P + p;
     constexpr long long rowz = (long long)N * M;     // stride between z rows
-    const float2* twL = g.tw32 + g.pN.tw_off;
+    const float2* twL = g.tw32;
     float2 v[3][E];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
@@ -224,7 +224,7 @@ k_fz3_p(const __grid_constant__ CUtensorMap zmap, GridDesc g, unsigned mask, flo
     };
     if (threadIdx.x == 0) issue(item);
     __syncthreads();
-    const float2* twL = g.tw32 + g.pN.tw_off;
+    const float2* twL = g.tw32;
     const float scale = (float)(1.0 / (double)g.N3);
     const float ga = (float)g.ga, gb = (float)g.gb;
     uint32_t parity = 0;
@@ -301,7 +301,7 @@ k_fzs(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__
     const int kx = kb * P + p;
     float2* base = spec + (long long)slot * 3 * NNM + c * NNM + (long long)ky * M + kb * P + p;
     constexpr long long rowz = (long long)N * M;     // stride between z rows
-    const float2* twL = g.tw32 + g.pN.tw_off;
+    const float2* twL = g.tw32;
     float2* shc = sh + c * NS + p;
     float2 v[E];
 #pragma unroll
@@ -406,8 +406,8 @@ __device__ __forceinline__ int pair_index(uchar2 q) { return q.x | (q.y << 2); }
 // The caller synchronizes the CTA before the first read.
 template <int M>
 __device__ __forceinline__ void stage_twiddles(float2* tws, const GridDesc& g) {
-    const float2* twM = g.tw32 + g.pM.tw_off;
-    const float2* twN = g.tw32 + g.pN.tw_off;
+    const float2* twM = g.tw32 + g.N;
+    const float2* twN = g.tw32;
     for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) tws[i] = i < M ? __ldg(&twM[i]) : __ldg(&twN[i - M]);
 }
 
@@ -855,7 +855,7 @@ __device__ __forceinline__ void y_columns(const GridDesc& g, float2* base, int t
     float2 v[E];
 #pragma unroll
     for (int n1 = 0; n1 < E; ++n1) v[n1] = base[(long long)(TP * n1 + t) * M];
-    const float2* twL = g.tw32 + g.pN.tw_off;
+    const float2* twL = g.tw32;
     stage1_write<L, FWD>(v, t, twL, sh, P);
     __syncthreads();
     stage2_read<L, FWD>(v, t, sh, P);
@@ -1189,7 +1189,7 @@ bool fast_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec
 
 bool chain_sweeps(const GridDesc& g) {
     // a relaxed scheme needs the old field in every x inverse: its sweeps are not chained
-    return !g.nochain && g.relax == 0.0 && !(g.xyvar == 1 && fused_cluster(g.N)) && fast_x_ctas(g) > 0;
+    return !g.nochain && g.relax == 0.0 && !(g.xyvar == 1 && fused_cluster(g.N));
 }
 
 namespace {
@@ -1235,7 +1235,7 @@ bool fast_take_wait_failure() {
 bool fast_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec, float* tau, const float* r32,
                   cudaStream_t st) {
     float2* sp = reinterpret_cast<float2*>(spec);
-    if (!fast_x_ctas(g)) return false;
+    if (!fast_x_ctas(g)) return gen_x_round(g, addr, wtau, mask, spec, tau, r32, st);
     // the persistent form of the correction sweeps (r added) of 24-value rows would keep
     // r in registers beside the transform and spill; those use the plain kernel
     if (g.xpers && !(addr && fast_split_e(g.M) > 16)) {

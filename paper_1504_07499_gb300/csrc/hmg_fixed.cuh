@@ -76,20 +76,39 @@ HMG_HD long long mul_r2(long long x) { return x - mulq<kQ1mR2>(x); }
 HMG_HD long long mul_h3(long long x) { return x - mulq<kQ1mH3>(x); }
 HMG_HD long long half(long long x) { return (x + 1) >> 1; }
 
-// a (c - i s) for (c, s) = (1 - C1, S) and the like
-template <long long C1, long long S>
-HMG_HD c64 rot_1c_s(c64 a) {   // c = 1 - C1, s = S
-    return c64{a.x - mulq<C1>(a.x) + mulq<S>(a.y), a.y - mulq<C1>(a.y) - mulq<S>(a.x)};
+// a (c - i s) with c = C or 1 - C (CM), s = S or 1 - S (SM)
+template <long long C, bool CM, long long S, bool SM>
+HMG_HD c64 rot(c64 a) {
+    const long long cx = CM ? a.x - mulq<C>(a.x) : mulq<C>(a.x), cy = CM ? a.y - mulq<C>(a.y) : mulq<C>(a.y);
+    const long long sx = SM ? a.x - mulq<S>(a.x) : mulq<S>(a.x), sy = SM ? a.y - mulq<S>(a.y) : mulq<S>(a.y);
+    return c64{cx + sy, cy - sx};
 }
-template <long long C, long long S1>
-HMG_HD c64 rot_c_1s(c64 a) {   // c = C, s = 1 - S1
-    return c64{mulq<C>(a.x) + (a.y - mulq<S1>(a.y)), mulq<C>(a.y) - (a.x - mulq<S1>(a.x))};
+
+// the same operations on FP32 pairs (hmg_gen32_kernels.cuh)
+HMG_HD float2 mkc(float x, float y) { return make_float2(x, y); }
+#ifdef __CUDA_ARCH__
+HMG_HD float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
+HMG_HD float2 operator-(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+#else
+HMG_HD float2 operator+(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+HMG_HD float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+#endif
+HMG_HD float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }
+HMG_HD float2 swap_ri(float2 a) { return make_float2(a.y, a.x); }
+HMG_HD float mul_r2(float x) { return x * 0.70710678118654752f; }
+HMG_HD float mul_h3(float x) { return x * 0.86602540378443865f; }
+HMG_HD float half(float x) { return 0.5f * x; }
+template <long long C, bool CM, long long S, bool SM>
+HMG_HD float2 rot(float2 a) {
+    constexpr double u = 1.0 / 18446744073709551616.0;   // 2^-64
+    constexpr float c = (float)(CM ? 1.0 - (double)C * u : (double)C * u);
+    constexpr float s = (float)(SM ? 1.0 - (double)S * u : (double)S * u);
+    return make_float2(c * a.x + s * a.y, c * a.y - s * a.x);
 }
-template <long long C1, long long S1>
-HMG_HD c64 rot_1c_1s(c64 a) {   // c = 1 - C1, s = 1 - S1
-    return c64{a.x - mulq<C1>(a.x) + (a.y - mulq<S1>(a.y)), a.y - mulq<C1>(a.y) - (a.x - mulq<S1>(a.x))};
-}
-HMG_HD c64 rot8(c64 a) { return c64{mul_r2(a.x + a.y), mul_r2(a.y - a.x)}; }   // a exp(-i pi/4)
+template <class T>
+HMG_HD T neg(T a) { return mkc(-a.x, -a.y); }
+template <class T>
+HMG_HD T rot8(T a) { return mkc(mul_r2(a.x + a.y), mul_r2(a.y - a.x)); }   // a exp(-i pi/4)
 
 // a w / 4 for a table twiddle w = (r.h 2^-30 + r.l 2^-62) + i (...) : {r.h, r.l, i.h, i.l}
 HMG_HD c64 cmul4(c64 a, int4 w) {
@@ -191,68 +210,34 @@ HMG_HD double from_fixed(long long v, int e) {
 // ---------------------------------------------------------------------------
 template <int R> struct Dft;
 template <> struct Dft<2> {
-    HMG_HD static void run(c64* v) {
-        const c64 a = v[0];
+    template <class T> HMG_HD static void run(T* v) {
+        const T a = v[0];
         v[0] = a + v[1];
         v[1] = a - v[1];
     }
 };
 template <> struct Dft<3> {
-    HMG_HD static void run(c64* v) {
-        const c64 t = v[1] + v[2], u = v[1] - v[2];
-        const c64 m = c64{v[0].x - half(t.x), v[0].y - half(t.y)};
-        const c64 h = c64{mul_h3(u.y), -mul_h3(u.x)};   // -i sqrt(3)/2 u
+    template <class T> HMG_HD static void run(T* v) {
+        const T t = v[1] + v[2], u = v[1] - v[2];
+        const T m = mkc(v[0].x - half(t.x), v[0].y - half(t.y));
+        const T h = mkc(mul_h3(u.y), -mul_h3(u.x));   // -i sqrt(3)/2 u
         v[0] = v[0] + t;
         v[1] = m + h;
         v[2] = m - h;
     }
 };
 template <> struct Dft<4> {
-    HMG_HD static void run(c64* v) {
-        const c64 a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = mul_mi(v[1] - v[3]);
+    template <class T> HMG_HD static void run(T* v) {
+        const T a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = mul_mi(v[1] - v[3]);
         v[0] = a + c;
         v[1] = b + d;
         v[2] = a - c;
         v[3] = b - d;
     }
 };
-// coprime factors: index maps without twiddles (Good 1958)
-template <> struct Dft<6> {
-    HMG_HD static void run(c64* v) {
-        c64 a[3] = {v[0], v[2], v[4]}, b[3] = {v[3], v[5], v[1]};   // n = 3 a + 2 b mod 6
-        Dft<3>::run(a);
-        Dft<3>::run(b);
-        // k = 3 q + 4 c mod 6 for (k mod 2, k mod 3) = (q, c)
-        v[0] = a[0] + b[0];
-        v[3] = a[0] - b[0];
-        v[4] = a[1] + b[1];
-        v[1] = a[1] - b[1];
-        v[2] = a[2] + b[2];
-        v[5] = a[2] - b[2];
-    }
-};
-template <> struct Dft<12> {
-    HMG_HD static void run(c64* v) {
-        // n = 3 n4 + 4 n3 mod 12, k = 9 k4 + 4 k3 mod 12
-        c64 s[3][4];
-#pragma unroll
-        for (int n3 = 0; n3 < 3; ++n3) {
-#pragma unroll
-            for (int n4 = 0; n4 < 4; ++n4) s[n3][n4] = v[(3 * n4 + 4 * n3) % 12];
-            Dft<4>::run(s[n3]);
-        }
-#pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) {
-            c64 t[3] = {s[0][k4], s[1][k4], s[2][k4]};
-            Dft<3>::run(t);
-#pragma unroll
-            for (int k3 = 0; k3 < 3; ++k3) v[(9 * k4 + 4 * k3) % 12] = t[k3];
-        }
-    }
-};
 template <> struct Dft<8> {
-    HMG_HD static void run(c64* v) {
-        c64 a[4], b[4];
+    template <class T> HMG_HD static void run(T* v) {
+        T a[4], b[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             a[r] = v[r] + v[r + 4];
@@ -271,25 +256,22 @@ template <> struct Dft<8> {
     }
 };
 template <> struct Dft<9> {
-    HMG_HD static void run(c64* v) {
-        c64 s[3][3];
+    template <class T> HMG_HD static void run(T* v) {
+        T s[3][3];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) s[b][a] = v[3 * a + b];
             Dft<3>::run(s[b]);
         }
-        s[1][1] = rot_1c_1s<kQ1mC40, kQ1mS40>(s[1][1]);
-        s[1][2] = rot_c_1s<kQC80, kQ1mS80>(s[1][2]);
-        s[2][1] = rot_c_1s<kQC80, kQ1mS80>(s[2][1]);
-        {   // exp(-i 160 deg) = -exp(+i 20 deg): c = -cos 20, s = sin 20
-            const c64 a = s[2][2];
-            const c64 r = c64{a.x - mulq<kQ1mC20>(a.x), a.y - mulq<kQ1mC20>(a.y)};
-            s[2][2] = c64{mulq<kQS20>(a.y) - r.x, -r.y - mulq<kQS20>(a.x)};
-        }
+        s[1][1] = rot<kQ1mC40, true, kQ1mS40, true>(s[1][1]);
+        s[1][2] = rot<kQC80, false, kQ1mS80, true>(s[1][2]);
+        s[2][1] = rot<kQC80, false, kQ1mS80, true>(s[2][1]);
+        // exp(-i 160 deg) = -i exp(-i 70 deg), cos 70 = sin 20, sin 70 = cos 20
+        s[2][2] = mul_mi(rot<kQS20, false, kQ1mC20, true>(s[2][2]));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            c64 t[3] = {s[0][k], s[1][k], s[2][k]};
+            T t[3] = {s[0][k], s[1][k], s[2][k]};
             Dft<3>::run(t);
             v[k] = t[0];
             v[k + 3] = t[1];
@@ -298,35 +280,66 @@ template <> struct Dft<9> {
     }
 };
 template <> struct Dft<16> {
-    HMG_HD static void run(c64* v) {
-        c64 s[4][4];
+    template <class T> HMG_HD static void run(T* v) {
+        T s[4][4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
 #pragma unroll
             for (int a = 0; a < 4; ++a) s[b][a] = v[4 * a + b];
             Dft<4>::run(s[b]);
         }
-        s[1][1] = rot_1c_s<kQ1mC8, kQS8>(s[1][1]);
+        s[1][1] = rot<kQ1mC8, true, kQS8, false>(s[1][1]);
         s[1][2] = rot8(s[1][2]);
-        s[1][3] = rot_c_1s<kQS8, kQ1mC8>(s[1][3]);
+        s[1][3] = rot<kQS8, false, kQ1mC8, true>(s[1][3]);
         s[2][1] = rot8(s[2][1]);
         s[2][2] = mul_mi(s[2][2]);
         s[2][3] = mul_mi(rot8(s[2][3]));
-        s[3][1] = rot_c_1s<kQS8, kQ1mC8>(s[3][1]);
+        s[3][1] = rot<kQS8, false, kQ1mC8, true>(s[3][1]);
         s[3][2] = mul_mi(rot8(s[3][2]));
-        {   // exp(-i 9 pi/8) = -exp(-i pi/8)
-            const c64 r = rot_1c_s<kQ1mC8, kQS8>(s[3][3]);
-            s[3][3] = c64{-r.x, -r.y};
-        }
+        s[3][3] = neg(rot<kQ1mC8, true, kQS8, false>(s[3][3]));   // exp(-i 9 pi/8)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            c64 t[4] = {s[0][k], s[1][k], s[2][k], s[3][k]};
+            T t[4] = {s[0][k], s[1][k], s[2][k], s[3][k]};
             Dft<4>::run(t);
 #pragma unroll
             for (int q = 0; q < 4; ++q) v[k + 4 * q] = t[q];
         }
     }
 };
+// R = A B with coprime factors: index maps without twiddles (Good 1958).  Input n = B a + A b
+// mod R, output k = U a' + V b' mod R with U = 1 mod A, 0 mod B and V = 0 mod A, 1 mod B.
+template <int A, int B>
+struct CoprimeDft {
+    static constexpr int R = A * B;
+    HMG_HD static constexpr int unit(int one, int zero) {
+        int u = zero;
+        while (u % one != 1) u += zero;
+        return u;
+    }
+    template <class T> HMG_HD static void run(T* v) {
+        constexpr int U = unit(A, B), V = unit(B, A);
+        T s[B][A];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+#pragma unroll
+            for (int a = 0; a < A; ++a) s[b][a] = v[(B * a + A * b) % R];
+            Dft<A>::run(s[b]);
+        }
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+            T t[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) t[b] = s[b][a];
+            Dft<B>::run(t);
+#pragma unroll
+            for (int b = 0; b < B; ++b) v[(U * a + V * b) % R] = t[b];
+        }
+    }
+};
+template <> struct Dft<6> : CoprimeDft<2, 3> {};
+template <> struct Dft<12> : CoprimeDft<4, 3> {};
+template <> struct Dft<18> : CoprimeDft<2, 9> {};
+template <> struct Dft<24> : CoprimeDft<8, 3> {};
 
 // Component bits a radix may start from: R 2^(b + 1/2) < 2^63 without twiddles (`first`),
 // R 2^(b + 1/2) / 4 < 2^63 and b <= 62 behind the /4 of the twiddle product (`later`).

@@ -90,7 +90,7 @@ k_xy_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
                 if (MODE == XF_FLUX) acc += v[n1].x + v[n1].y;
             }
         }
-        fast::stage1_write<M, true>(v, tx, g.tw32 + g.pM.tw_off, xb + r * G::RS, 1);
+        fast::stage1_write<M, true>(v, tx, g.tw32 + g.N, xb + r * G::RS, 1);
     }
     __syncthreads();
     if (tid < G::XT) fast::stage2_read<M, true>(v, tx, xb + r * G::RS, 1);
@@ -110,7 +110,7 @@ k_xy_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
     // real-to-complex split and scatter of coefficient kx to the owner of its column block
     cluster.barrier_wait(std::move(started));
     if (tid < G::XT) {
-        const float2* twN = g.tw32 + g.pN.tw_off;
+        const float2* twN = g.tw32;
         const float2* rs = xb + r * G::RS;
 #pragma unroll
         for (int j = 0; j < EX; ++j) {
@@ -138,7 +138,7 @@ k_xy_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
         for (int n1 = 0; n1 < EY; ++n1) v[n1] = yb[(TPY * n1 + ty) * CW + p];
     }
     __syncthreads();
-    if (tid < G::YT) fast::stage1_write<N, true>(v, ty, g.tw32 + g.pN.tw_off, yb + p, CW);
+    if (tid < G::YT) fast::stage1_write<N, true>(v, ty, g.tw32, yb + p, CW);
     __syncthreads();
     if (tid < G::YT) {
         fast::stage2_read<N, true>(v, ty, yb + p, CW);
@@ -180,7 +180,7 @@ k_yx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
         const float2* src = spec + ((long long)slot * 3 + c) * NN * M + (long long)z * N * M + rank * CW + p;
 #pragma unroll
         for (int n1 = 0; n1 < EY; ++n1) v[n1] = src[(long long)(TPY * n1 + ty) * M];
-        fast::stage1_write<N, false>(v, ty, g.tw32 + g.pN.tw_off, yb + p, CW);
+        fast::stage1_write<N, false>(v, ty, g.tw32, yb + p, CW);
     }
     __syncthreads();
     cluster.barrier_wait(std::move(started));
@@ -203,7 +203,7 @@ k_yx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
     const int y = rank * RW + r;
     float2* rs = xb + r * G::RS;
     if (tid < G::XT) {
-        const float2* twN = g.tw32 + g.pN.tw_off;
+        const float2* twN = g.tw32;
 #pragma unroll
         for (int n1 = 0; n1 < EX; ++n1) {
             const int k = TPX * n1 + tx;
@@ -223,7 +223,7 @@ k_yx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
         }
     }
     __syncthreads();
-    if (tid < G::XT) fast::stage1_write<M, false>(v, tx, g.tw32 + g.pM.tw_off, rs, 1);
+    if (tid < G::XT) fast::stage1_write<M, false>(v, tx, g.tw32 + g.N, rs, 1);
     __syncthreads();
     if (tid < G::XT) fast::stage2_read<M, false>(v, tx, rs, 1);
     __syncthreads();

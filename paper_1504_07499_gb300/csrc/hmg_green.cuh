@@ -87,7 +87,9 @@ __device__ __forceinline__ void green_mode(int kx, int ky, int kz, int N, R scal
 // projector factor gb / |m'|^2 from the fast reciprocal (__fdividef, error within 2 ulp)
 // and the updates as packed two-lane FP32 operations on (real, imaginary) pairs:
 // s_c <- scale ga s_c - (scale gb d_c / |m'|^2) (m' . s).  The four self-conjugate modes of
-// the packed kx = 0 column (and the DC with its gc E) go through green_mode.
+// the packed kx = 0 column (and the DC with its gc E) go through green_mode.  EXACT: the
+// factor from an IEEE division instead.
+template <bool EXACT = false>
 __device__ __forceinline__ void green_mode_fast(int kx, int ky, int kz, int N, float scale, float ga, float gb,
                                                 bool add_b, const float* cE, float2& s0, float2& s1, float2& s2) {
     const bool special = (kx == 0) && (ky == 0 || ky == N / 2) && (kz == 0 || kz == N / 2);
@@ -97,7 +99,7 @@ __device__ __forceinline__ void green_mode_fast(int kx, int ky, int kz, int N, f
     }
     int d[3];
     const int n2 = mode_dir(kx, signed_mode(ky, N), signed_mode(kz, N), N, d);   // > 0 off the special modes
-    const float gs = scale * __fdividef(gb, (float)n2);
+    const float gs = scale * (EXACT ? __fdiv_rn(gb, (float)n2) : __fdividef(gb, (float)n2));
     const float d0 = (float)d[0], d1 = (float)d[1], d2 = (float)d[2];
     const float2 dot = __ffma2_rn(make_float2(d2, d2), s2,
                                   __ffma2_rn(make_float2(d1, d1), s1, __fmul2_rn(make_float2(d0, d0), s0)));

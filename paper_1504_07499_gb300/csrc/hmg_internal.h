@@ -7,8 +7,7 @@
 
 namespace hmg {
 
-constexpr int kThreads = 256;      // threads per CTA in every FFT pass
-constexpr int kMaxStages = 12;     // radix stages per 1D transform
+constexpr int kThreads = 256;      // threads per CTA of the reductions, pointwise and voxel kernels
 constexpr int kMaxSlots = 3;       // right-hand sides (unit gradients) per RVE
 
 // Every grid size N of the library: even, 2^a 3^b, 8 .. 512.
@@ -16,22 +15,13 @@ constexpr int kMaxSlots = 3;       // right-hand sides (unit gradients) per RVE
     X(8) X(12) X(16) X(18) X(24) X(32) X(36) X(48) X(54) X(64) X(72) X(96) X(108) X(128) X(144) X(162) \
     X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
 
-// Mixed-radix Stockham schedule of one 1D length (radices 2, 3, 4, 8).
-struct FftPlan {
-    int L;                 // transform length
-    int nst;               // number of stages
-    int rad[kMaxStages];   // radix of each stage, first stage first
-    int tw_off;            // offset of the length-L twiddle table exp(-2 pi i k / L)
-};
-
 // Everything a pass kernel needs about one RVE: sizes, FFT schedules, the
 // per-phase coefficient table, and the device fields (FP32 or FP64 copies).
 struct GridDesc {
     int N, M;              // grid size and N/2 (complex length of an x row)
     long long NN, N3;      // N*N and N^3
     long long NNM;         // complex entries per component spectrum: N*N*M
-    FftPlan pN, pM;        // schedules for lengths N (y, z) and M (x)
-    const float2* tw32;    // twiddle tables (all lengths, concatenated)
+    const float2* tw32;    // twiddles w_N^k (k < N) then w_M^k (k < M)
     // FP64 passes in block fixed point (hmg_fixed.cuh): twiddles w_N^k (k < N) then w_M^k
     // (k < M), projector reciprocals, exponents of the spectrum's pencils (3 N^2 per slot each)
     const int4* twf;
@@ -56,8 +46,6 @@ struct GridDesc {
     double relax;
     double E[kMaxSlots][3];  // macroscopic gradient of each right-hand side
     int nslots;            // right-hand sides held in the fields
-    int rows;              // x-pass rows per CTA
-    int Py, Pz;            // columns per CTA in the y and z passes
     int zvar;              // z-pass kernel variant of the register-resident path (autotuned)
     int xyvar;             // 1: fused x + y cluster kernels, 0: separate x and y passes (autotuned)
     int nochain;           // 1: FP32 sweeps of a block are not chained through k_fx_round
@@ -107,12 +95,7 @@ void launch_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* sp
                       const float* r32, float* d32, float* r32_out, double* partial,
                       cudaStream_t st);
 
-// Tile sizes of the generic FP32 shared-memory passes (x rows per CTA, y and z columns per CTA).
-void set_tiles(GridDesc& g);
-int x_ctas(const GridDesc& g);   // CTAs per right-hand side of the generic x passes
-int z_ctas(const GridDesc& g);   // CTAs per right-hand side of the generic z pass
 // CTAs per right-hand side of the x / z passes that launch_* runs for precision R
-// (FP32: the register-resident kernels where one exists, else the generic ones)
 template <typename R> int x_ctas_for(const GridDesc& g);
 template <typename R> int z_ctas_for(const GridDesc& g);
 
@@ -128,8 +111,8 @@ bool fast_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec
 // spectrum; adds r (addr; per-slot flag in flags mode) and stores the updated field (wtau).
 bool fast_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec, float* tau, const float* r32,
                   cudaStream_t st);
-// FP32 sweeps of a block are chained (x inverse + next x forward in one kernel):
-// register-resident x kernels exist for g.N, separate x and y passes, chaining not off.
+// FP32 sweeps of a block are chained (x inverse + next x forward in one kernel): separate x
+// and y passes, no relaxation, chaining not off.
 bool chain_sweeps(const GridDesc& g);
 // y inverse + x round trip + y forward of each plane in one persistent kernel (sizes 64,
 // 128, 192, 256; not for relaxed schemes); false when it does not apply.
@@ -141,6 +124,18 @@ bool fast_yxy(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec
 bool fast_take_wait_failure();
 int fast_x_ctas(const GridDesc& g);
 int fast_z_ctas(const GridDesc& g);
+
+// FP32 passes of the sizes hmg_fast.cu does not serve (hmg_gen32.cu); false there for the others.
+int gen_x_ctas(const GridDesc& g);
+int gen_z_ctas(const GridDesc& g);
+bool gen_x_forward(const GridDesc& g, int mode, unsigned mask, const float* tau, void* spec, double* partial,
+                   cudaStream_t st);
+bool gen_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, float* tau, const float* r32,
+                   double* partial, cudaStream_t st);
+bool gen_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec, float* tau, const float* r32,
+                 cudaStream_t st);
+bool gen_col(const GridDesc& g, bool zdir, bool forward, unsigned mask, void* spec, cudaStream_t st);
+bool gen_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st);
 
 // FP64 passes (hmg_fixed_*.cu); XI_PLAIN, XI_INPLACE, XI_INPLACE_RES and XI_DIFF.
 int fx_x_ctas(const GridDesc& g);

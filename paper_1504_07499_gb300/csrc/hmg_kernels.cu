@@ -11,9 +11,9 @@
 // L0 = -k0 I), steps 2-7 read tau^{n+1} = (I - 2P)(Y tau^n) + 2 k0 E, and
 // e^n - e_comp^n = (tau^n - tau^{n+1}) / (2 k0), so no field but tau is stored.
 // (The basic scheme runs through the same passes on e itself, with its own Y and the
-// Green step -P; GridDesc carries the scheme's coefficients.)  These generic kernels
-// serve the FP32 sizes without register-resident kernels (hmg_fast.cu); FP64 passes run in
-// block fixed point (hmg_fixed.cuh).
+// Green step -P; GridDesc carries the scheme's coefficients.)  The pass kernels are in
+// hmg_fast.cu and hmg_gen32_kernels.cuh (FP32) and hmg_fixed_kernels.cuh (FP64); this file
+// holds their dispatch by precision and size, the reductions and the pointwise helpers.
 //
 // Spectrum layout: after the x pass each row of N reals becomes N/2 complex values
 // (x-major rows, same byte size as the real field); entry kx = 0 packs the two real
@@ -25,8 +25,6 @@
 
 #include <type_traits>
 
-#include "hmg_fft.cuh"
-#include "hmg_green.cuh"
 #include "hmg_internal.h"
 
 namespace hmg {
@@ -34,11 +32,6 @@ namespace hmg {
 // ---------------------------------------------------------------------------
 // small device helpers
 // ---------------------------------------------------------------------------
-
-template <typename R>
-__device__ __forceinline__ R sel3(int ph, double a, double b, double c) {
-    return R(ph == 0 ? a : (ph == 1 ? b : c));
-}
 
 // Fixed-order CTA sum of one double per thread; result valid in thread 0.
 __device__ double block_sum(double v, double* sh) {
@@ -51,251 +44,6 @@ __device__ double block_sum(double v, double* sh) {
     double r = sh[0];
     __syncthreads();
     return r;
-}
-
-// ---------------------------------------------------------------------------
-// x forward: rows of N reals -> N/2 packed complex values
-// ---------------------------------------------------------------------------
-
-template <typename R, int MODE>
-__global__ void __launch_bounds__(kThreads)
-k_x_forward(GridDesc g, unsigned mask, const R* __restrict__ tau, typename Cplx<R>::T* __restrict__ spec,
-            double* __restrict__ partial) {
-    using T2 = typename Cplx<R>::T;
-    const int slot = blockIdx.y;
-    if (!slot_active(g, mask, slot)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    const int M = g.M, N = g.N, rows = g.rows;
-    T2* b1 = b0 + rows * M;
-    __shared__ double red[kThreads];
-
-    const long long row0 = (long long)blockIdx.x * rows;   // row = c*NN + z*N + y
-    const T2* src = reinterpret_cast<const T2*>(tau + (long long)slot * 3 * g.N3 + row0 * N);
-    double acc = 0.0;
-    for (int q = threadIdx.x; q < rows * M; q += blockDim.x) {
-        const int rr = q / M, n = q - rr * M;
-        T2 v = src[(long long)rr * M + n];
-        if (MODE != XF_PLAIN) {
-            const long long prow = (row0 + rr) % g.NN;   // (z, y) row of the phase grid
-            const uchar2 ph = *reinterpret_cast<const uchar2*>(g.phase + prow * N + 2 * n);
-            R ca, cb;
-            if (MODE == XF_POLARIZE) {
-                ca = sel3<R>(ph.x, g.Y[0], g.Y[1], g.Y[2]);
-                cb = sel3<R>(ph.y, g.Y[0], g.Y[1], g.Y[2]);
-            } else {
-                ca = sel3<R>(ph.x, g.W[0], g.W[1], g.W[2]);
-                cb = sel3<R>(ph.y, g.W[0], g.W[1], g.W[2]);
-            }
-            v.x *= ca;
-            v.y *= cb;
-            if (MODE == XF_FLUX) acc += (double)v.x + (double)v.y;
-        }
-        b0[q] = v;
-    }
-    if (MODE == XF_FLUX) {
-        double s = block_sum(acc, red);
-        if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
-    }
-    __syncthreads();
-    T2* res = fft_smem<true>(b0, b1, g.pM, TwTable<T2>::get(g), rows, M, 1);
-    // real-to-complex split: X_k = E_k + w_N^k O_k with E, O the DFTs of the even and
-    // odd samples, E_k = (Z_k + conj Z_{M-k})/2, O_k = (Z_k - conj Z_{M-k})/(2i)
-    const T2* twN = TwTable<T2>::get(g) + g.pN.tw_off;
-    T2* dst = spec + (long long)slot * 3 * g.NNM + row0 * M;
-    for (int q = threadIdx.x; q < rows * M; q += blockDim.x) {
-        const int rr = q / M, k = q - rr * M;
-        const T2 z = res[rr * M + k];
-        T2 out;
-        if (k == 0) {
-            out = mk(z.x + z.y, z.x - z.y);
-        } else {
-            const T2 zm = res[rr * M + (M - k)];
-            const T2 e = mk(R(0.5) * (z.x + zm.x), R(0.5) * (z.y - zm.y));
-            const T2 o = mk(R(0.5) * (z.y + zm.y), R(-0.5) * (z.x - zm.x));
-            out = cadd(e, cmul(o, __ldg(&twN[k])));
-        }
-        dst[(long long)rr * M + k] = out;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// x inverse: N/2 packed complex values -> N reals, with the sweep's output step
-// ---------------------------------------------------------------------------
-
-template <typename R, int MODE>
-__global__ void __launch_bounds__(kThreads)
-k_x_inverse(GridDesc g, unsigned mask, const typename Cplx<R>::T* __restrict__ spec, R* __restrict__ tau,
-            const float* __restrict__ r32, double* __restrict__ partial) {
-    using T2 = typename Cplx<R>::T;
-    const int slot = blockIdx.y;
-    if (!slot_active(g, mask, slot)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    const int M = g.M, N = g.N, rows = g.rows;
-    T2* b1 = b0 + rows * M;
-    __shared__ double red[kThreads];
-
-    const long long row0 = (long long)blockIdx.x * rows;
-    const T2* src = spec + (long long)slot * 3 * g.NNM + row0 * M;
-    for (int q = threadIdx.x; q < rows * M; q += blockDim.x) b1[q] = src[q];
-    __syncthreads();
-    // complex-to-real merge: Z'_k = (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k}),
-    // whose length-M inverse DFT gives N x[2n] + i N x[2n+1] (unnormalized)
-    const T2* twN = TwTable<T2>::get(g) + g.pN.tw_off;
-    for (int q = threadIdx.x; q < rows * M; q += blockDim.x) {
-        const int rr = q / M, k = q - rr * M;
-        T2 xk, xm;
-        if (k == 0) {
-            const T2 p = b1[rr * M];
-            xk = mk(p.x, R(0));
-            xm = mk(p.y, R(0));
-        } else {
-            xk = b1[rr * M + k];
-            xm = b1[rr * M + (M - k)];
-        }
-        const T2 s = mk(xk.x + xm.x, xk.y - xm.y);          // X_k + conj X_{M-k}
-        const T2 d = mk(xk.x - xm.x, xk.y + xm.y);          // X_k - conj X_{M-k}
-        const T2 dw = cmulc(d, __ldg(&twN[k]));             // d * w^{-k}
-        b0[q] = mk(s.x - dw.y, s.y + dw.x);                 // s + i dw
-    }
-    __syncthreads();
-    T2* res = fft_smem<false>(b0, b1, g.pM, TwTable<T2>::get(g), rows, M, 1);
-
-    const long long fbase = (long long)slot * 3 * g.N3 + row0 * N;   // element offset of the tile
-    T2* out = reinterpret_cast<T2*>(tau + fbase);
-    // output step: add r (correction sweeps), read the old field for the residual
-    constexpr bool kRes = MODE == XI_INPLACE_RES || MODE == XI_ADD_R_RES;
-    constexpr bool kAddR = MODE == XI_ADD_R_RES || MODE == XI_ADD_R;
-    const bool resid = kRes && (g.dflags ? g.resid != 0 : true);
-    const bool addr = kAddR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
-    double acc = 0.0;
-    const bool relax = g.relax != 0.0;            // uniform: kernel argument
-    const R wn = R(1.0 - g.relax), wo = R(g.relax);
-    for (int q = threadIdx.x; q < rows * M; q += blockDim.x) {
-        T2 v = res[q];
-        if (relax) {   // relaxed schemes: (1 - relax) T(field) + relax field
-            const T2 o = out[q];
-            v = mk(wn * v.x + wo * o.x, wn * v.y + wo * o.y);
-        }
-        if (addr) {
-            const float2 rv = reinterpret_cast<const float2*>(r32 + fbase)[q];
-            v.x += R(rv.x);
-            v.y += R(rv.y);
-        }
-        if (resid) {
-            const T2 o = out[q];
-            const double da = (double)v.x - (double)o.x, db = (double)v.y - (double)o.y;
-            acc += da * da + db * db;
-        }
-        out[q] = v;
-    }
-    if (kRes) {   // uniform across the CTA
-        double s = block_sum(acc, red);
-        if (threadIdx.x == 0 && resid) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// y pass: Py consecutive kx columns of one (component, z) plane, length N along y
-// ---------------------------------------------------------------------------
-
-template <typename R, bool FWD>
-__global__ void __launch_bounds__(kThreads)
-k_y_pass(GridDesc g, unsigned mask, typename Cplx<R>::T* __restrict__ spec) {
-    using T2 = typename Cplx<R>::T;
-    const int slot = blockIdx.y;
-    if (!slot_active(g, mask, slot)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = g.N, M = g.M, P = g.Py;
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    T2* b1 = b0 + N * P;
-    const int nkb = M / P;
-    const int kb = blockIdx.x % nkb;
-    const long long cz = blockIdx.x / nkb;                     // c*N + z
-    T2* base = spec + (long long)slot * 3 * g.NNM + cz * N * M + kb * P;
-    for (int q = threadIdx.x; q < N * P; q += blockDim.x) {
-        const int y = q / P, p = q - y * P;
-        b0[q] = base[(long long)y * M + p];
-    }
-    __syncthreads();
-    T2* res = fft_smem<FWD>(b0, b1, g.pN, TwTable<T2>::get(g), P, 1, P);
-    for (int q = threadIdx.x; q < N * P; q += blockDim.x) {
-        const int y = q / P, p = q - y * P;
-        base[(long long)y * M + p] = res[q];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// z pass: Pz consecutive kx columns at one ky, all three components, length N
-// along z.  Z_ITER: forward, tau_hat <- (ga - gb P) tau_hat / N^3 (+ gc E at DC;
-// Eyre-Milton: (I - 2P) and 2 k0 E), inverse.  Z_EQ: forward, then sum
-// |xi . phi_hat|^2 / N^6 in FP64.
-// ---------------------------------------------------------------------------
-
-template <typename R, int MODE>
-__global__ void __launch_bounds__(kThreads)
-k_z_pass(GridDesc g, unsigned mask, typename Cplx<R>::T* __restrict__ spec, double* __restrict__ partial) {
-    using T2 = typename Cplx<R>::T;
-    const int slot = blockIdx.y;
-    if (!slot_active(g, mask, slot)) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = g.N, M = g.M, P = g.Pz, P3 = 3 * P;
-    T2* b0 = reinterpret_cast<T2*>(smem_raw);
-    T2* b1 = b0 + N * P3;
-    __shared__ double red[kThreads];
-    const int nkb = M / P;
-    const int kb = blockIdx.x % nkb;
-    const int ky = blockIdx.x / nkb;
-    T2* base = spec + (long long)slot * 3 * g.NNM + (long long)ky * M + kb * P;
-    // SMEM layout [z][c][p]: pencil c*P + p, index stride 3P
-    for (int q = threadIdx.x; q < N * P3; q += blockDim.x) {
-        const int z = q / P3, cp = q - z * P3, c = cp / P, p = cp - c * P;
-        b0[q] = base[(long long)c * g.NNM + (long long)z * N * M + p];
-    }
-    __syncthreads();
-    const T2* tw = TwTable<T2>::get(g);
-    T2* res = b0;
-    if (MODE != Z_INV) res = fft_smem<true>(b0, b1, g.pN, tw, P3, 1, P3);
-    T2* other = (res == b0) ? b1 : b0;
-
-    if (MODE == Z_ITER || MODE == Z_ITER_NOB || MODE == Z_EQ) {
-        const bool addb = g.dflags ? (g.dflags[slot] & SF_ADDB) != 0 : MODE == Z_ITER;
-        const R scale = R(1.0 / (double)g.N3);
-        const R cE[3] = {R(g.gc * g.E[slot][0]), R(g.gc * g.E[slot][1]), R(g.gc * g.E[slot][2])};
-        const R ga = R(g.ga), gb = R(g.gb);
-        double acc = 0.0;
-        const double twopi_n = 6.283185307179586476925 / (double)N;
-        for (int q = threadIdx.x; q < N * P; q += blockDim.x) {
-            const int kz = q / P, p = q - kz * P;
-            const int kx = kb * P + p;
-            T2* e = res + kz * P3 + p;
-            T2 s0 = e[0], s1 = e[P], s2 = e[2 * P];
-            if (MODE == Z_EQ) {
-                acc += eq_mode(kx, ky, kz, N, s0, s1, s2);
-            } else {
-                green_mode<R>(kx, ky, kz, N, scale, ga, gb, addb, cE, s0, s1, s2);
-                e[0] = s0;
-                e[P] = s1;
-                e[2 * P] = s2;
-            }
-        }
-        if (MODE == Z_EQ) {
-            // |xi . phi_hat|^2 with xi = 2 pi m'/N and phi_hat = DFT/N^3
-            const double s = block_sum(acc, red) * twopi_n * twopi_n / ((double)g.N3 * (double)g.N3);
-            if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
-            return;
-        }
-        __syncthreads();
-    }
-    if (MODE == Z_ITER || MODE == Z_ITER_NOB || MODE == Z_INV) {
-        if (MODE == Z_INV) other = b1;
-        res = fft_smem<false>(res, other, g.pN, tw, P3, 1, P3);
-    }
-    for (int q = threadIdx.x; q < N * P3; q += blockDim.x) {
-        const int z = q / P3, cp = q - z * P3, c = cp / P, p = cp - c * P;
-        base[(long long)c * g.NNM + (long long)z * N * M + p] = res[q];
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -317,10 +65,13 @@ template <typename R>
 __global__ void k_init_tau(GridDesc g, unsigned mask, R* __restrict__ tau) {
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
+    R v[3][3];   // (k + k0) E_c of each phase, rounded once
+    for (int p = 0; p < 3; ++p)
+        for (int c = 0; c < 3; ++c) v[p][c] = R(g.KP[p] * g.E[slot][c]);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N3; i += (long long)gridDim.x * blockDim.x) {
         const int ph = g.phase[i];
-        const double kp = ph == 0 ? g.KP[0] : (ph == 1 ? g.KP[1] : g.KP[2]);
-        for (int c = 0; c < 3; ++c) tau[((long long)slot * 3 + c) * g.N3 + i] = R(kp * g.E[slot][c]);
+        for (int c = 0; c < 3; ++c)
+            tau[((long long)slot * 3 + c) * g.N3 + i] = ph == 0 ? v[0][c] : (ph == 1 ? v[1][c] : v[2][c]);
     }
 }
 
@@ -333,12 +84,24 @@ __global__ void k_e_to_tau(GridDesc g, int slot, const double* __restrict__ e, R
     }
 }
 
+// e = tau / (k + k0).  The three divisors are known, so each quotient is a product with the
+// rounded reciprocal corrected by one residual step (Brisebarre, Muller & Raina, "Accelerating
+// correctly rounded floating-point division when the divisor is known in advance", 2004):
+// three FP64 operations instead of a divide's ten or so, which bound this kernel.
 template <typename R>
 __global__ void k_tau_to_e(GridDesc g, int slot, const R* __restrict__ tau, double* __restrict__ e) {
+    const double rc[3] = {1.0 / g.KP[0], 1.0 / g.KP[1], 1.0 / g.KP[2]};
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N3; i += (long long)gridDim.x * blockDim.x) {
         const int ph = g.phase[i];
         const double kp = ph == 0 ? g.KP[0] : (ph == 1 ? g.KP[1] : g.KP[2]);
-        for (int c = 0; c < 3; ++c) e[c * g.N3 + i] = (double)tau[((long long)slot * 3 + c) * g.N3 + i] / kp;
+        const double r = ph == 0 ? rc[0] : (ph == 1 ? rc[1] : rc[2]);
+        for (int c = 0; c < 3; ++c) {
+            const double t = (double)tau[((long long)slot * 3 + c) * g.N3 + i];
+            const double q = t * r;
+            const double rem = fma(-q, kp, t);
+            // (an infinite or overflowing quotient has no residual)
+            e[c * g.N3 + i] = isfinite(rem) ? fma(rem, r, q) : t / kp;
+        }
     }
 }
 
@@ -379,69 +142,31 @@ static int pointwise_blocks(long long n) {
     return (int)(b < 152 * 16 ? b : 152 * 16);
 }
 
-int x_ctas(const GridDesc& g) { return (int)(3 * g.NN / g.rows); }
-int z_ctas(const GridDesc& g) { return g.N * (g.M / g.Pz); }
-
 template <> int x_ctas_for<float>(const GridDesc& g) {
     if (g.xyvar == 1 && fused_cluster(g.N)) return fused_xy_ctas(g);
     const int f = fast_x_ctas(g);
-    return f ? f : x_ctas(g);
+    return f ? f : gen_x_ctas(g);
 }
 template <> int x_ctas_for<double>(const GridDesc& g) { return fx_x_ctas(g); }
 template <> int z_ctas_for<float>(const GridDesc& g) {
     const int f = fast_z_ctas(g);
-    return f ? f : z_ctas(g);
+    return f ? f : gen_z_ctas(g);
 }
 template <> int z_ctas_for<double>(const GridDesc& g) { return fx_z_ctas(g); }
 
-template <typename K>
-static void set_smem(K kern, size_t bytes) {
-    // static (2 KB) plus dynamic shared memory above 48 KB needs the opt-in
-    if (bytes > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
+// FP64: block fixed point.  FP32: the kernels of hmg_fast.cu for N = 64, 96, 128, 192, 256 and
+// 512, those of hmg_gen32.cu for every other size.
 template <typename R>
 void launch_x_forward(const GridDesc& g, int mode, unsigned mask, const R* tau, void* spec,
                       double* partial, cudaStream_t st) {
-    if constexpr (std::is_same<R, double>::value) {
-        fx_x_forward(g, mode, mask, tau, spec, partial, st);
-    } else {
-        using T2 = typename Cplx<R>::T;
-        if (fast_x_forward(g, mode, mask, tau, spec, partial, st)) return;
-        const size_t sm = 2ull * g.rows * g.M * sizeof(T2);
-        dim3 grid(x_ctas(g), g.nslots);
-        T2* sp = reinterpret_cast<T2*>(spec);
-        if (mode == XF_PLAIN) {
-            set_smem(k_x_forward<R, XF_PLAIN>, sm);
-            k_x_forward<R, XF_PLAIN><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
-        } else if (mode == XF_POLARIZE) {
-            set_smem(k_x_forward<R, XF_POLARIZE>, sm);
-            k_x_forward<R, XF_POLARIZE><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
-        } else {
-            set_smem(k_x_forward<R, XF_FLUX>, sm);
-            k_x_forward<R, XF_FLUX><<<grid, kThreads, sm, st>>>(g, mask, tau, sp, partial);
-        }
-    }
+    if constexpr (std::is_same<R, double>::value) fx_x_forward(g, mode, mask, tau, spec, partial, st);
+    else if (!fast_x_forward(g, mode, mask, tau, spec, partial, st)) gen_x_forward(g, mode, mask, tau, spec, partial, st);
 }
 
 template <typename R>
 void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st) {
-    if constexpr (std::is_same<R, double>::value) {
-        fx_y(g, forward, mask, spec, st);
-    } else {
-        using T2 = typename Cplx<R>::T;
-        if (fast_y(g, forward, mask, spec, st)) return;
-        const size_t sm = 2ull * g.N * g.Py * sizeof(T2);
-        dim3 grid(3 * g.N * (g.M / g.Py), g.nslots);
-        T2* sp = reinterpret_cast<T2*>(spec);
-        if (forward) {
-            set_smem(k_y_pass<R, true>, sm);
-            k_y_pass<R, true><<<grid, kThreads, sm, st>>>(g, mask, sp);
-        } else {
-            set_smem(k_y_pass<R, false>, sm);
-            k_y_pass<R, false><<<grid, kThreads, sm, st>>>(g, mask, sp);
-        }
-    }
+    if constexpr (std::is_same<R, double>::value) fx_y(g, forward, mask, spec, st);
+    else if (!fast_y(g, forward, mask, spec, st)) gen_col(g, false, forward, mask, spec, st);
 }
 
 template <typename R>
@@ -449,49 +174,16 @@ void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, doubl
     if constexpr (std::is_same<R, double>::value) {
         if (mode == Z_FWD || mode == Z_INV) fx_z_plain(g, mode == Z_FWD, mask, spec, st);
         else fx_z(g, mode, mask, spec, partial, st);
-    } else {
-        using T2 = typename Cplx<R>::T;
-        if (fast_z(g, mode, mask, spec, partial, st)) return;
-        const size_t sm = 2ull * 3 * g.N * g.Pz * sizeof(T2);
-        dim3 grid(z_ctas(g), g.nslots);
-        T2* sp = reinterpret_cast<T2*>(spec);
-#define HMG_Z(MODE_)                     \
-    set_smem(k_z_pass<R, MODE_>, sm);    \
-    k_z_pass<R, MODE_><<<grid, kThreads, sm, st>>>(g, mask, sp, partial)
-        switch (mode) {
-            case Z_FWD: HMG_Z(Z_FWD); break;
-            case Z_INV: HMG_Z(Z_INV); break;
-            case Z_ITER: HMG_Z(Z_ITER); break;
-            case Z_ITER_NOB: HMG_Z(Z_ITER_NOB); break;
-            default: HMG_Z(Z_EQ); break;
-        }
-#undef HMG_Z
+    } else if (!fast_z(g, mode, mask, spec, partial, st)) {
+        gen_z(g, mode, mask, spec, partial, st);
     }
 }
 
 template <typename R>
 void launch_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, R* tau,
                       const float* r32, float* d32, float* r32_out, double* partial, cudaStream_t st) {
-    if constexpr (std::is_same<R, double>::value) {
-        fx_x_inverse(g, mode, mask, spec, tau, d32, r32_out, partial, st);
-    } else {
-        using T2 = typename Cplx<R>::T;
-        if (fast_x_inverse(g, mode, mask, spec, tau, r32, partial, st)) return;
-        const size_t sm = 2ull * g.rows * g.M * sizeof(T2);
-        dim3 grid(x_ctas(g), g.nslots);
-        const T2* sp = reinterpret_cast<const T2*>(spec);
-#define HMG_XI(MODE_)                      \
-    set_smem(k_x_inverse<R, MODE_>, sm);   \
-    k_x_inverse<R, MODE_><<<grid, kThreads, sm, st>>>(g, mask, sp, tau, r32, partial)
-        switch (mode) {
-            case XI_PLAIN: HMG_XI(XI_PLAIN); break;
-            case XI_INPLACE: HMG_XI(XI_INPLACE); break;
-            case XI_INPLACE_RES: HMG_XI(XI_INPLACE_RES); break;
-            case XI_ADD_R_RES: HMG_XI(XI_ADD_R_RES); break;
-            default: HMG_XI(XI_ADD_R); break;
-        }
-#undef HMG_XI
-    }
+    if constexpr (std::is_same<R, double>::value) fx_x_inverse(g, mode, mask, spec, tau, d32, r32_out, partial, st);
+    else if (!fast_x_inverse(g, mode, mask, spec, tau, r32, partial, st)) gen_x_inverse(g, mode, mask, spec, tau, r32, partial, st);
 }
 
 template <typename R>

@@ -40,10 +40,9 @@ struct DeviceGuard {
     }
 };
 
-// FFT schedules and twiddle tables of one grid size.
+// Tables of one grid size.
 struct GridPlan {
     int N = 0;
-    FftPlan pN{}, pM{};
     float2* tw32 = nullptr;
     int4* twf = nullptr;          // FP64 passes: fixed-point twiddles and projector reciprocals
     long long* rcp = nullptr;
