@@ -26,6 +26,7 @@
 #include "hmg_fft.cuh"
 #include "hmg_green.cuh"
 #include "hmg_internal.h"
+#include "hmg_launch.cuh"
 #include "hmg_regfft.cuh"
 
 namespace hmg {
@@ -48,6 +49,7 @@ template <int L, int P, bool FWD>
 __global__ void __launch_bounds__(P * Split<L>::TP, col_min_ctas<L, 3>())
 k_fy(GridDesc g, unsigned mask, float2* __restrict__ spec) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // xslots<L>() * P
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(P * Split<L>::TP, 3)
 k_fz3(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__ partial) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
     constexpr int NS = xslots<L>() * P;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // 3 * NS
@@ -211,11 +214,12 @@ k_fz3_p(const __grid_constant__ CUtensorMap zmap, GridDesc g, unsigned mask, flo
     float2* sh = reinterpret_cast<float2*>(dsm + Z::x_off) + p;  // one component at a time
     const int nkb = M / P;
     const int nitems = g.nslots * nper;
+    const uint32_t mb = async::smem_addr(&mbar);
+    if (threadIdx.x == 0) async::mbar_init(mb);
+    grid_begin();
     int item = blockIdx.x;
     while (item < nitems && !slot_active(g, mask, item / nper)) item += gridDim.x;
     if (item >= nitems) return;
-    const uint32_t mb = async::smem_addr(&mbar);
-    if (threadIdx.x == 0) async::mbar_init(mb);
     auto issue = [&](int it) {   // thread 0: the three component columns of item `it`
         const int slot = it / nper, b = it % nper;
         async::mbar_expect(mb, (uint32_t)Z::stage_bytes);
@@ -287,6 +291,7 @@ __global__ void __launch_bounds__(3 * P * Split<L>::TP, col_min_ctas<L, 2>())
 k_fzs(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__ partial) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
     constexpr int NS = xslots<L>() * P;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // 3 * NS
@@ -535,6 +540,9 @@ __global__ void __launch_bounds__(RW * Split<M>::TP, 1024 / (RW * Split<M>::TP))
 k_fx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* __restrict__ spec,
              double* __restrict__ partial) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
+    __shared__ float2 tws[2 * M];
+    stage_twiddles<M>(tws, g);
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // RW * RS
@@ -549,8 +557,6 @@ k_fx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
     const long long row = comp * g.NN + rblk * RW + r;              // c*NN + z*N + y
     const long long pidx = comp * (g.NN / RW) + rblk;               // component-major CTA index
     const float2* src = reinterpret_cast<const float2*>(tau + (long long)slot * 3 * g.N3 + row * N);
-    __shared__ float2 tws[2 * M];
-    stage_twiddles<M>(tws, g);
     if (MODE != XF_PLAIN)
         coef_pairs(lut, (float)(MODE == XF_POLARIZE ? g.Y[0] : g.W[0]), (float)(MODE == XF_POLARIZE ? g.Y[1] : g.W[1]),
                    (float)(MODE == XF_POLARIZE ? g.Y[2] : g.W[2]));
@@ -626,6 +632,9 @@ __global__ void __launch_bounds__(RW * Split<M>::TP, fx_inverse_min_threads<M, M
 k_fx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* __restrict__ tau,
              const float* __restrict__ r32, double* __restrict__ partial) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
+    __shared__ float2 tws[2 * M];
+    stage_twiddles<M>(tws, g);
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // RW * RS
@@ -644,8 +653,6 @@ k_fx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
     float2 old[E], radd[E];
     if (res || relax) s2_load<M>(old, out, t);
     if (addr) s2_load<M>(radd, reinterpret_cast<const float2*>(r32 + fbase), t);
-    __shared__ float2 tws[2 * M];
-    stage_twiddles<M>(tws, g);
     __syncthreads();
     float2 v[E];
     row_inverse<M, TP, E>(v, t, sh + r * RS, spec + (long long)slot * 3 * g.NNM + row * M, tws, tws + M);
@@ -678,10 +685,14 @@ __global__ void __launch_bounds__(RW * Split<M>::TP, 512 / (RW * Split<M>::TP))
 k_fx_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau,
            const float* __restrict__ r32) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
+    __shared__ float2 lut[16];
+    __shared__ float2 tws[2 * M];
+    coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
+    stage_twiddles<M>(tws, g);
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) float2 sh[];   // RW * RS
-    __shared__ float2 lut[16];
     const int N = g.N;
     const int t = threadIdx.x % TP, r = threadIdx.x / TP;
     // component fastest across CTAs (phase rows reused from L2, as in k_fx_forward)
@@ -695,11 +706,8 @@ k_fx_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     if (addr) s2_load<M>(radd, reinterpret_cast<const float2*>(r32 + fbase), t);
     uchar2 q[E];
     s2_load_phase<M>(q, reinterpret_cast<const uchar2*>(g.phase + (row % g.NN) * N), t);
-    coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
     float2* sp = spec + (long long)slot * 3 * g.NNM + row * M;
     float2* rs = sh + r * RS;
-    __shared__ float2 tws[2 * M];
-    stage_twiddles<M>(tws, g);
     __syncthreads();   // tables and coefficient pairs
     const float2* twM = tws;
     const float2* twN = tws + M;
@@ -755,13 +763,14 @@ k_fx_round_p(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __rest
     __shared__ int s_ok;
     const int t = threadIdx.x % TP, r = threadIdx.x / TP;
     const int nitems = g.nslots * nblk;
-    int item = blockIdx.x;
-    while (item < nitems && !slot_active(g, mask, item / nblk)) item += gridDim.x;
-    if (item >= nitems) return;
     const uint32_t mb = async::smem_addr(&mbar);
     if (threadIdx.x == 0) async::mbar_init(mb);
     coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
     stage_twiddles<M>(tws, g);
+    grid_begin();
+    int item = blockIdx.x;
+    while (item < nitems && !slot_active(g, mask, item / nblk)) item += gridDim.x;
+    if (item >= nitems) return;
     // thread 0: stage the spectrum rows and phase rows of block `it`
     auto issue = [&](int it) {
         const int slot = it / nblk, b = it % nblk;
@@ -877,6 +886,7 @@ k_yxy(GridDesc g, unsigned mask, float2* spec, float* __restrict__ tau, const fl
     __shared__ float2 tws[2 * M];
     coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
     stage_twiddles<M>(tws, g);
+    grid_begin();
     __syncthreads();
     const float2* twM = tws;
     const float2* twN = tws + M;
@@ -942,9 +952,9 @@ namespace {
 // Launch with `bytes` of dynamic shared memory.  Static plus dynamic shared memory
 // above 48 KB needs the opt-in, so it is requested whenever the two could exceed it.
 template <typename K, typename... Args>
-void launch_dyn(K kern, dim3 grid, int threads, size_t bytes, cudaStream_t st, Args... args) {
+void launch_dyn(K kern, dim3 grid, int threads, size_t bytes, cudaStream_t st, const GridDesc& g, Args... args) {
     if (bytes > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    kern<<<grid, threads, bytes, st>>>(args...);
+    launch_kernel(small_grid(g, sizeof(float)), kern, grid, threads, bytes, st, g, args...);
 }
 constexpr int pow2_cols(int cap, int M) {
     int p = 1;
@@ -1068,7 +1078,7 @@ bool launch_fz3_p(int mode, cudaStream_t st, const GridDesc& g, unsigned mask, f
         auto kern = mode == Z_ITER ? fast::k_fz3_p<L, P, Z_ITER> : fast::k_fz3_p<L, P, Z_ITER_NOB>;
         const int nper = g.N * (g.M / P);
         const int grid = persistent_grid(kern, T, sm, nper * g.nslots);
-        kern<<<grid, T, sm, st>>>(map, g, mask, sp, nper);
+        launch_kernel(small_grid(g, sizeof(float)), kern, grid, T, sm, st, map, g, mask, sp, nper);
         return true;
     }
 }
@@ -1201,7 +1211,7 @@ void launch_round_p(const GridDesc& g, unsigned mask, float2* sp, float* tau, co
     auto kern = fast::k_fx_round_p<M, RW, ADDR, WTAU>;
     const int nblk = fast_x_ctas(g);
     const int grid = persistent_grid(kern, T, sm, nblk * g.nslots);
-    kern<<<grid, T, sm, st>>>(g, mask, sp, tau, r32, nblk);
+    launch_kernel(small_grid(g, sizeof(float)), kern, grid, T, sm, st, g, mask, sp, tau, r32, nblk);
 }
 }  // namespace
 
@@ -1287,7 +1297,7 @@ void launch_yxy(const GridDesc& g, unsigned mask, float2* sp, float* tau, const 
     constexpr size_t sm = fast::YxyShape<L>::smem;
     const int nper = 3 * g.N;
     const int grid = persistent_grid(kern, 256, sm, nper * g.nslots);
-    kern<<<grid, 256, sm, st>>>(g, mask, sp, tau, r32, nper);
+    launch_kernel(small_grid(g, sizeof(float)), kern, grid, 256, sm, st, g, mask, sp, tau, r32, nper);
 }
 }  // namespace
 

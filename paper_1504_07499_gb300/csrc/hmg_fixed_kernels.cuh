@@ -16,6 +16,7 @@
 #include "hmg_fft.cuh"
 #include "hmg_fixed.cuh"
 #include "hmg_green.cuh"
+#include "hmg_launch.cuh"
 
 namespace hmg {
 namespace fx {
@@ -86,6 +87,7 @@ k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ ta
     using P = Plan<M>;
     using S = typename X::S;
     constexpr int N = X::N, RW = X::RW, TPP = X::TPP, T = X::T, J = M / P::R0;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -183,6 +185,7 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* __restrict__ spec,
     using P = Plan<M>;
     using S = typename X::S;
     constexpr int N = X::N, RW = X::RW, TPP = X::TPP, T = X::T, J = M / P::R0;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -296,6 +299,7 @@ k_fxx_col(GridDesc g, unsigned mask, c64* __restrict__ spec, ColArgs a) {
     using P = Plan<L>;
     using S = typename C::S;
     constexpr int M = C::M, NP = C::NP, TPP = C::TPP, T = C::T, J = L / P::R0;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -408,6 +412,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
     using P = Plan<L>;
     using S = typename Z::S;
     constexpr int N = L, M = Z::M, NP = Z::NP, P3 = Z::P3, TPP = Z::TPP, T = Z::T, J = L / P::R0;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -550,9 +555,9 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
 // launchers of one length
 // ---------------------------------------------------------------------------
 template <class K, class... Args>
-void launch(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+void launch(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, const GridDesc& g, Args... args) {
     if (smem > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<grid, threads, smem, st>>>(args...);
+    launch_kernel(small_grid(g, sizeof(double)), kern, grid, threads, smem, st, g, args...);
 }
 
 }  // namespace fx

@@ -10,9 +10,9 @@ namespace hmg {
 
 namespace {
 template <class K, class... Args>
-void launch(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+void launch(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, const GridDesc& g, Args... args) {
     if (smem > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<grid, threads, smem, st>>>(args...);
+    launch_kernel(small_grid(g, sizeof(float)), kern, grid, threads, smem, st, g, args...);
 }
 }  // namespace
 

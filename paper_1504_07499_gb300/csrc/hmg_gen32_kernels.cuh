@@ -15,6 +15,7 @@
 #include "hmg_fft.cuh"
 #include "hmg_fixed.cuh"
 #include "hmg_green.cuh"
+#include "hmg_launch.cuh"
 
 namespace hmg {
 namespace g32 {
@@ -259,6 +260,7 @@ k_gx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
     using X = XShape<M>;
     using P = Plan<M>;
     constexpr int N = X::N, RW = X::RW, T = X::T;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -296,6 +298,7 @@ k_gx_inverse(GridDesc g, unsigned mask, int mode, const float2* __restrict__ spe
     using X = XShape<M>;
     using P = Plan<M>;
     constexpr int N = X::N, RW = X::RW, T = X::T;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -346,6 +349,7 @@ k_gx_round(GridDesc g, unsigned mask, int add, int wtau, float2* __restrict__ sp
     using P = Plan<M>;
     using S = typename X::S;
     constexpr int N = X::N, RW = X::RW;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -399,6 +403,7 @@ k_gcol(GridDesc g, unsigned mask, int zdir, int inverse, float2* __restrict__ sp
     using C = ColShape<L>;
     using P = Plan<L>;
     constexpr int M = C::M, NP = C::NP;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -432,6 +437,7 @@ k_gz(GridDesc g, unsigned mask, int mode, float2* __restrict__ spec, double* __r
     using P = Plan<L>;
     using S = ColSlots<Z::P3>;
     constexpr int N = L, M = Z::M, NP = Z::NP, P3 = Z::P3, T = Z::T;
+    grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "hmg_internal.h"
+#include "hmg_launch.cuh"
 
 namespace hmg {
 
@@ -52,6 +53,7 @@ __device__ double block_sum(double v, double* sh) {
 
 __global__ void k_reduce(const double* __restrict__ partial, int count, int groups, double* __restrict__ out) {
     __shared__ double red[kThreads];
+    grid_begin();
     const int slot = blockIdx.x / groups, grp = blockIdx.x % groups;
     const int per = count / groups;
     const double* p = partial + (long long)slot * count + (long long)grp * per;
@@ -209,7 +211,7 @@ bool launch_yx_inverse(const GridDesc& g, int mode, unsigned mask, const void* s
 }
 
 void launch_reduce(const double* partial, int nslots, int count, int groups, double* out, cudaStream_t st) {
-    k_reduce<<<nslots * groups, kThreads, 0, st>>>(partial, count, groups, out);
+    launch_kernel(true, k_reduce, dim3(nslots * groups), kThreads, 0, st, partial, count, groups, out);
 }
 
 template <typename R>
