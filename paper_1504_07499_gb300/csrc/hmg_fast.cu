@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "hmg_async.cuh"
 #include "hmg_fft.cuh"
@@ -836,6 +837,454 @@ k_fx_round_p(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __rest
 }
 
 // ---------------------------------------------------------------------------
+// x passes of row pairs (N = 64, 128, 192, 256): two real rows a, b (neighbouring y) as one
+// complex row z = a + i b of length N.  Against one row of N reals as N / 2 complex values, the
+// split and merge need no twiddle factors (Z_k = A_k + i B_k, and A_k, B_k come back from Z_k
+// and conj Z_{N-k} by additions) and half the lane exchanges, and with N = TP^2 a thread's
+// twiddles w_N^(t j) are the same in both directions, so a persistent kernel keeps them in
+// registers.  The x round trip was bound by L1 (87 %): about 418 wavefronts per four rows
+// of 256 became about 288.  256^3, three gradients, per launch: 313 -> 292 us averaged over a solve's
+// forms, 0.84 of the copy bandwidth on their bytes (plain form 293 -> 235 us); sweeps at 64^3
+// 28.2 -> 26.0 us, at 192^3 about 510 -> 480 us.
+// ---------------------------------------------------------------------------
+
+// Merge of the packed row spectra a, b (a[n1] = A at k = TP n1 + t < N / 2) into the stage-1
+// layout of the pair, v[n1] = Z[TP n1 + t]; Z[N - k] = conj A_k + i conj B_k goes to the partner
+// lane's upper half (thread 0 keeps its own).
+template <int L, int TP, int E>
+__device__ __forceinline__ void pair_merge(float2* v, const float2* a, const float2* b, int t) {
+    const int pl = partner_lane<TP>(t);
+    float2 w[E / 2];
+#pragma unroll
+    for (int n1 = 0; n1 < E / 2; ++n1) {
+        v[n1] = make_float2(a[n1].x - b[n1].y, a[n1].y + b[n1].x);
+        w[n1] = make_float2(a[n1].x + b[n1].y, b[n1].x - a[n1].y);
+    }
+#pragma unroll
+    for (int j = E / 2; j < E; ++j) {
+        v[j] = shfl2(w[E - 1 - j], pl);
+        if (t == 0) v[j] = j == E / 2 ? make_float2(a[0].y, b[0].y) : w[(E - j) % (E / 2)];
+    }
+    if (t == 0) v[0] = make_float2(a[0].x, b[0].x);   // entry 0 packs X(0) and X(N/2)
+}
+
+// Split of the pair's transform v[kb] = Z[t + TP kb] into the packed row spectra, k < N / 2.
+template <int L, int TP, int E>
+__device__ __forceinline__ void pair_split(const float2* v, int t, float2* __restrict__ da, float2* __restrict__ db) {
+    const int pl = partner_lane<TP>(t);
+#pragma unroll
+    for (int kb = 0; kb < E / 2; ++kb) {
+        const int k = t + TP * kb;
+        const float2 z = v[kb];
+        float2 zm = shfl2(v[E - 1 - kb], pl);
+        if (kb > 0 && t == 0) zm = v[E - kb];
+        float2 A = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
+        float2 B = make_float2(0.5f * (z.y + zm.y), -0.5f * (z.x - zm.x));
+        if (k == 0) {
+            A = make_float2(z.x, v[E / 2].x);
+            B = make_float2(z.y, v[E / 2].y);
+        }
+        da[k] = A;
+        db[k] = B;
+    }
+}
+
+// The pair's values in the stage-2 layout: v[i TP + m] = (a, b) at p = t KPT + i + E m.
+template <int L>
+__device__ __forceinline__ void pair_load(float2* v, const float* __restrict__ ra, const float* __restrict__ rb, int t) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
+#pragma unroll
+    for (int m = 0; m < TP; ++m) {
+        if constexpr (KPT % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < KPT; i += 2) {
+                const float2 x = *reinterpret_cast<const float2*>(ra + t * KPT + i + E * m);
+                const float2 y = *reinterpret_cast<const float2*>(rb + t * KPT + i + E * m);
+                v[i * TP + m] = make_float2(x.x, y.x);
+                v[(i + 1) * TP + m] = make_float2(x.y, y.y);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                v[i * TP + m] = make_float2(ra[t * KPT + i + E * m], rb[t * KPT + i + E * m]);
+        }
+    }
+}
+template <int L>
+__device__ __forceinline__ void pair_store(float* __restrict__ ra, float* __restrict__ rb, const float2* v, int t) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
+#pragma unroll
+    for (int m = 0; m < TP; ++m) {
+        if constexpr (KPT % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < KPT; i += 2) {
+                const float2 x = v[i * TP + m], y = v[(i + 1) * TP + m];
+                *reinterpret_cast<float2*>(ra + t * KPT + i + E * m) = make_float2(x.x, y.x);
+                *reinterpret_cast<float2*>(rb + t * KPT + i + E * m) = make_float2(x.y, y.y);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KPT; ++i) {
+                ra[t * KPT + i + E * m] = v[i * TP + m].x;
+                rb[t * KPT + i + E * m] = v[i * TP + m].y;
+            }
+        }
+    }
+}
+template <int L>
+__device__ __forceinline__ void pair_load_phase(uchar2* q, const uint8_t* __restrict__ pa, const uint8_t* __restrict__ pb,
+                                                int t) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
+#pragma unroll
+    for (int m = 0; m < TP; ++m) {
+        if constexpr (KPT % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < KPT; i += 2) {
+                const uchar2 x = *reinterpret_cast<const uchar2*>(pa + t * KPT + i + E * m);
+                const uchar2 y = *reinterpret_cast<const uchar2*>(pb + t * KPT + i + E * m);
+                q[i * TP + m] = make_uchar2(x.x, y.x);
+                q[(i + 1) * TP + m] = make_uchar2(x.y, y.y);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KPT; ++i)
+                q[i * TP + m] = make_uchar2(pa[t * KPT + i + E * m], pb[t * KPT + i + E * m]);
+        }
+    }
+}
+
+// Twiddles of the pair transforms: the table w_N^k staged in shared memory, or (N = TP^2) this
+// thread's w_N^(t j), j < TP, in registers.
+template <int L>
+struct PairTwSmem {
+    const float2* tab;
+};
+template <int L>
+struct PairTwReg {
+    float2 w[Split<L>::TP];
+    __device__ __forceinline__ void load(const float2* __restrict__ tab, int t) {
+#pragma unroll
+        for (int j = 1; j < Split<L>::TP; ++j) w[j] = __ldg(&tab[(t * j) % L]);
+    }
+};
+
+// Inverse transform of a pair from its packed row spectra (shared or global memory), leaving
+// the stage-2 layout; forward transform from that layout, split and stored to da, db.
+template <int L, class TW>
+__device__ __forceinline__ void pair_inverse_merged(float2* v, int t, float2* rs, const TW& tw) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP;
+    RegDFT<E, false>::run(v);
+#pragma unroll
+    for (int k1 = 1; k1 < E; ++k1) {
+        if constexpr (std::is_same<TW, PairTwReg<L>>::value) v[k1] = cmulc(v[k1], tw.w[k1]);
+        else v[k1] = cmulc(v[k1], tw.tab[(t * k1) % L]);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < E; ++k1) rs[xslot<L>(k1, t)] = v[k1];
+    row_sync<TP>();
+    stage2_read<L, false>(v, t, rs, 1);
+}
+template <int L, class TW>
+__device__ __forceinline__ void pair_inverse(float2* v, int t, float2* rs, const float2* sa, const float2* sb, const TW& tw) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP;
+    float2 a[E / 2], b[E / 2];
+#pragma unroll
+    for (int n1 = 0; n1 < E / 2; ++n1) {
+        a[n1] = sa[TP * n1 + t];
+        b[n1] = sb[TP * n1 + t];
+    }
+    pair_merge<L, TP, E>(v, a, b, t);
+    pair_inverse_merged<L>(v, t, rs, tw);
+}
+template <int L, class TW>
+__device__ __forceinline__ void pair_forward(float2* v, int t, float2* rs, const TW& tw, float2* __restrict__ da,
+                                             float2* __restrict__ db) {
+    constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        const int k1 = t * KPT + i;
+        RegDFT<TP, true>::run(v + i * TP);
+#pragma unroll
+        for (int n2 = 0; n2 < TP; ++n2) {
+            float2 x = v[i * TP + n2];
+            if (n2 > 0) {
+                if constexpr (std::is_same<TW, PairTwReg<L>>::value) x = cmul(x, tw.w[n2]);
+                else x = cmul(x, tw.tab[(n2 * k1) % L]);
+            }
+            rs[xslot<L>(k1, n2)] = x;
+        }
+    }
+    row_sync<TP>();
+    rstage1_read<L, true>(v, t, rs, 1);   // v[kb] = Z[t + TP kb]
+    pair_split<L, TP, E>(v, t, da, db);
+}
+
+template <int L>
+__device__ __forceinline__ void stage_pair_twiddles(float2* tws, const GridDesc& g) {
+    for (int i = threadIdx.x; i < L; i += blockDim.x) tws[i] = __ldg(&g.tw32[i]);
+}
+
+template <int L>
+struct PairShape {
+    static constexpr int M = L / 2, E = Split<L>::E, TP = Split<L>::TP;
+    static constexpr int NP = 128 / TP, RW = 2 * NP;         // pairs and rows per CTA of 128 threads
+    static constexpr int RS = row_stride<L>();               // exchange buffer of a pair
+};
+
+template <int L, int MODE>
+__global__ void __launch_bounds__(128, 8)
+k_px_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* __restrict__ spec,
+             double* __restrict__ partial) {
+    using S = PairShape<L>;
+    constexpr int E = S::E, TP = S::TP, M = S::M;
+    __shared__ float2 tws[L];
+    stage_pair_twiddles<L>(tws, g);
+    grid_begin();
+    const int slot = blockIdx.y;
+    if (!slot_active(g, mask, slot)) return;
+    extern __shared__ __align__(16) float2 sh[];   // NP * RS
+    __shared__ double red[128];
+    __shared__ float2 lut[16];
+    const int t = threadIdx.x % TP, r = threadIdx.x / TP;
+    // component fastest across CTAs, so the three components of a (z, y) block read the
+    // same phase rows close together in time (L2 hits)
+    const int comp = blockIdx.x % 3;
+    const long long rblk = blockIdx.x / 3;
+    const long long row = comp * g.NN + rblk * S::RW + 2 * r;       // c*NN + z*N + y, the pair's first row
+    const long long pidx = comp * (g.NN / S::RW) + rblk;            // component-major CTA index
+    const float* src = tau + (long long)slot * 3 * g.N3 + row * L;
+    if (MODE != XF_PLAIN)
+        coef_pairs(lut, (float)(MODE == XF_POLARIZE ? g.Y[0] : g.W[0]), (float)(MODE == XF_POLARIZE ? g.Y[1] : g.W[1]),
+                   (float)(MODE == XF_POLARIZE ? g.Y[2] : g.W[2]));
+    __syncthreads();
+    float2 v[E];
+    pair_load<L>(v, src, src + L, t);
+    float acc = 0.f;
+    if (MODE != XF_PLAIN) {
+        uchar2 q[E];
+        const uint8_t* ph = g.phase + (row % g.NN) * L;
+        pair_load_phase<L>(q, ph, ph + L, t);
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            // rounded products (never contracted into the transform's adds), as in the round trip
+            v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
+            if (MODE == XF_FLUX) acc += v[j].x + v[j].y;
+        }
+    }
+    if (MODE == XF_FLUX) {
+        const double s = block_sum_d((double)acc, red);
+        if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + pidx] = s;
+    }
+    float2* dst = spec + (long long)slot * 3 * g.NNM + row * M;
+    pair_forward<L>(v, t, sh + r * S::RS, PairTwSmem<L>{tws}, dst, dst + M);
+}
+
+// threads per SM the register bound aims at, as fx_inverse_min_threads
+template <int L, int MODE>
+constexpr int px_inverse_ctas() {
+    return (MODE == XI_ADD_R_RES || MODE == XI_INPLACE_RES || Split<L>::E > 16) ? 4 : 6;
+}
+
+template <int L, int MODE>
+__global__ void __launch_bounds__(128, px_inverse_ctas<L, MODE>())
+k_px_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* __restrict__ tau,
+             const float* __restrict__ r32, double* __restrict__ partial) {
+    using S = PairShape<L>;
+    constexpr int E = S::E, TP = S::TP, M = S::M;
+    __shared__ float2 tws[L];
+    stage_pair_twiddles<L>(tws, g);
+    grid_begin();
+    const int slot = blockIdx.y;
+    if (!slot_active(g, mask, slot)) return;
+    extern __shared__ __align__(16) float2 sh[];   // NP * RS
+    __shared__ double red[128];
+    const int t = threadIdx.x % TP, r = threadIdx.x / TP;
+    const long long row = (long long)blockIdx.x * S::RW + 2 * r;
+    const long long fbase = (long long)slot * 3 * g.N3 + row * L;
+    float* out = tau + fbase;
+    // prefetch the old field (and r) for the output step: in flight during the FFT
+    constexpr bool kRes = MODE == XI_INPLACE_RES || MODE == XI_ADD_R_RES;
+    constexpr bool kAddR = MODE == XI_ADD_R_RES || MODE == XI_ADD_R;
+    const bool res = kRes && (g.dflags ? g.resid != 0 : true);
+    const bool addr = kAddR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
+    const bool relax = g.relax != 0.0;   // relaxed schemes keep a fraction of the old field
+    float2 old[E], radd[E];
+    if (res || relax) pair_load<L>(old, out, out + L, t);
+    if (addr) pair_load<L>(radd, r32 + fbase, r32 + fbase + L, t);
+    __syncthreads();
+    float2 v[E];
+    const float2* src = spec + (long long)slot * 3 * g.NNM + row * M;
+    pair_inverse<L>(v, t, sh + r * S::RS, src, src + M, PairTwSmem<L>{tws});
+    float acc = 0.f;
+    const float wn = (float)(1.0 - g.relax), wo = (float)g.relax;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        if (relax) v[j] = make_float2(wn * v[j].x + wo * old[j].x, wn * v[j].y + wo * old[j].y);
+        if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
+        if (res) {
+            const float da = v[j].x - old[j].x, db = v[j].y - old[j].y;
+            acc += da * da + db * db;
+        }
+    }
+    pair_store<L>(out, out + L, v, t);
+    if (kRes) {   // uniform across the CTA (kernel argument and per-slot flag)
+        const double s = block_sum_d((double)acc, red);
+        if (threadIdx.x == 0 && res) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
+    }
+}
+
+// x inverse of one sweep fused with the polarization and x forward of the next (k_fx_round),
+// on row pairs; same float operations as k_px_inverse followed by k_px_forward.
+template <int L, bool ADDR, bool WTAU>
+__global__ void __launch_bounds__(128, 4)
+k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau, const float* __restrict__ r32) {
+    using S = PairShape<L>;
+    constexpr int E = S::E, TP = S::TP, M = S::M;
+    __shared__ float2 lut[16];
+    __shared__ float2 tws[L];
+    coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
+    stage_pair_twiddles<L>(tws, g);
+    grid_begin();
+    const int slot = blockIdx.y;
+    if (!slot_active(g, mask, slot)) return;
+    extern __shared__ __align__(16) float2 sh[];   // NP * RS
+    const int t = threadIdx.x % TP, r = threadIdx.x / TP;
+    // component fastest across CTAs (phase rows reused from L2, as in k_px_forward)
+    const long long row = (blockIdx.x % 3) * g.NN + (long long)(blockIdx.x / 3) * S::RW + 2 * r;
+    const long long fbase = (long long)slot * 3 * g.N3 + row * L;
+    const bool addr = ADDR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
+    // loads for the update and the polarization: in flight during the inverse FFT
+    float2 radd[E];
+    if (addr) pair_load<L>(radd, r32 + fbase, r32 + fbase + L, t);
+    uchar2 q[E];
+    const uint8_t* ph = g.phase + (row % g.NN) * L;
+    pair_load_phase<L>(q, ph, ph + L, t);
+    float2* sp = spec + (long long)slot * 3 * g.NNM + row * M;
+    float2* rs = sh + r * S::RS;
+    __syncthreads();   // tables and coefficient pairs
+    float2 v[E];
+    pair_inverse<L>(v, t, rs, sp, sp + M, PairTwSmem<L>{tws});
+#pragma unroll
+    for (int j = 0; j < E; ++j)
+        if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
+    if (WTAU) pair_store<L>(tau + fbase, tau + fbase + L, v, t);
+#pragma unroll
+    for (int j = 0; j < E; ++j) v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
+    row_sync<TP>();   // the pair's threads have read their stage-2 values from rs
+    pair_forward<L>(v, t, rs, PairTwSmem<L>{tws}, sp, sp + M);
+}
+
+// Dynamic shared memory of k_px_round_p: staged spectrum rows, phase rows, exchange buffers
+// (padding as RoundSmem).
+template <int L>
+struct PairSmem {
+    using S = PairShape<L>;
+    static constexpr int SROW = S::M + 8, PROW = L + 32;
+    static constexpr size_t phase_off = (size_t)S::RW * SROW * sizeof(float2);
+    static constexpr size_t x_off = (phase_off + (size_t)S::RW * PROW + 15) / 16 * 16;
+    static constexpr size_t total = x_off + (size_t)S::NP * S::RS * sizeof(float2);
+};
+
+// k_px_round as a persistent kernel with the next rows staged by bulk copies (k_fx_round_p).
+template <int L, bool ADDR, bool WTAU>
+__global__ void __launch_bounds__(128, 4)
+k_px_round_p(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau,
+             const float* __restrict__ r32, int nblk) {
+    using S = PairShape<L>;
+    using D = PairSmem<L>;
+    constexpr int E = S::E, TP = S::TP, M = S::M, RW = S::RW;
+    constexpr bool kReg = E == TP;   // this thread's twiddles fit in registers
+    extern __shared__ __align__(128) unsigned char dsm[];
+    float2* sspec = reinterpret_cast<float2*>(dsm);
+    unsigned char* sphase = dsm + D::phase_off;
+    __shared__ float2 lut[16];
+    __shared__ float2 tws[kReg ? 1 : L];
+    __shared__ __align__(8) unsigned long long mbar;
+    __shared__ int s_ok;
+    const int t = threadIdx.x % TP, r = threadIdx.x / TP;
+    const int nitems = g.nslots * nblk;
+    const uint32_t mb = async::smem_addr(&mbar);
+    if (threadIdx.x == 0) async::mbar_init(mb);
+    coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
+    typename std::conditional<kReg, PairTwReg<L>, PairTwSmem<L>>::type tw;
+    if constexpr (kReg) {
+        tw.load(g.tw32, t);
+    } else {
+        stage_pair_twiddles<L>(tws, g);
+        tw.tab = tws;
+    }
+    grid_begin();
+    int item = blockIdx.x;
+    while (item < nitems && !slot_active(g, mask, item / nblk)) item += gridDim.x;
+    if (item >= nitems) return;
+    // thread 0: stage the spectrum rows and phase rows of block `it`
+    auto issue = [&](int it) {
+        const int slot = it / nblk, b = it % nblk;
+        const long long row0 = (b % 3) * g.NN + (long long)(b / 3) * RW;
+        const float2* src = spec + (long long)slot * 3 * g.NNM + row0 * M;
+        async::mbar_expect(mb, (uint32_t)(RW * M * sizeof(float2) + RW * L));
+        for (int rr = 0; rr < RW; ++rr)
+            async::bulk_g2s(async::smem_addr(sspec + rr * D::SROW), src + (long long)rr * M, M * sizeof(float2), mb);
+        const uint8_t* prow = g.phase + (long long)(b / 3) * RW * L;
+        for (int rr = 0; rr < RW; ++rr)
+            async::bulk_g2s(async::smem_addr(sphase + rr * D::PROW), prow + (long long)rr * L, L, mb);
+    };
+    if (threadIdx.x == 0) issue(item);
+    __syncthreads();   // barrier initialized, tables staged
+    float2* rs = reinterpret_cast<float2*>(dsm + D::x_off) + r * S::RS;
+    uint32_t parity = 0;
+    while (item < nitems) {
+        const int slot = item / nblk, b = item % nblk;
+        const long long row = (b % 3) * g.NN + (long long)(b / 3) * RW + 2 * r;   // c*NN + z*N + y
+        const long long fbase = (long long)slot * 3 * g.N3 + row * L;
+        const bool addr = ADDR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
+        float2 radd[E];
+        if (addr) pair_load<L>(radd, r32 + fbase, r32 + fbase + L, t);
+        // this block's copies: one thread decides for the CTA whether the wait succeeded
+        if (threadIdx.x == 0) s_ok = async::mbar_wait(mb, parity) ? 1 : 0;
+        __syncthreads();
+        if (!s_ok) {
+            if (threadIdx.x == 0) atomicOr(&g_wait_fail, 1u);
+            return;
+        }
+        async::mbar_wait(mb, parity);   // complete already: the copied bytes are visible here
+        parity ^= 1u;
+        float2 v[E];
+        {
+            float2 xa[E / 2], xb[E / 2];
+            const float2* sa = sspec + 2 * r * D::SROW;
+#pragma unroll
+            for (int n1 = 0; n1 < E / 2; ++n1) {
+                xa[n1] = sa[TP * n1 + t];
+                xb[n1] = sa[D::SROW + TP * n1 + t];
+            }
+            pair_merge<L, TP, E>(v, xa, xb, t);
+        }
+        uchar2 q[E];
+        pair_load_phase<L>(q, sphase + 2 * r * D::PROW, sphase + (2 * r + 1) * D::PROW, t);
+        __syncthreads();   // every thread holds its rows: the buffers take the next block
+        int nxt = item + gridDim.x;
+        while (nxt < nitems && !slot_active(g, mask, nxt / nblk)) nxt += gridDim.x;
+        if (threadIdx.x == 0 && nxt < nitems) issue(nxt);
+        // x inverse (step 5), update (step 7), optional store, polarization (step 2)
+        pair_inverse_merged<L>(v, t, rs, tw);
+#pragma unroll
+        for (int j = 0; j < E; ++j)
+            if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
+        if (WTAU) pair_store<L>(tau + fbase, tau + fbase + L, v, t);
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
+        row_sync<TP>();   // the pair's threads have read their stage-2 values from rs
+        // forward transform (step 3) and split, written over the rows it came from
+        float2* dst = spec + (long long)slot * 3 * g.NNM + row * M;
+        pair_forward<L>(v, t, rs, tw, dst, dst + M);
+        row_sync<TP>();   // rs is reused by the next block (s_ok and the staging buffers are
+                          // next written after CTA barriers every thread has passed)
+        item = nxt;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // y inverse + x round trip + y forward of a (component, z) plane in one persistent kernel.
 // A CTA takes whole planes: it transforms the plane's columns along y in place, then its
 // rows (x inverse, update, polarization of the next sweep, x forward), then its columns
@@ -851,9 +1300,9 @@ template <int L>
 struct YxyShape {
     static constexpr int M = L / 2;
     static constexpr int P = 256 / Split<L>::TP;        // columns per y step
-    static constexpr int RW = 256 / Split<M>::TP;       // rows per x step
+    static constexpr int RW = 2 * 256 / Split<L>::TP;   // rows per x step (pairs)
     static constexpr int SY = P * xslots<L>();
-    static constexpr int SX = RW * row_stride<M>();
+    static constexpr int SX = RW / 2 * row_stride<L>();
     static constexpr size_t smem = sizeof(float2) * (SY > SX ? SY : SX);
 };
 
@@ -880,16 +1329,14 @@ k_yxy(GridDesc g, unsigned mask, float2* spec, float* __restrict__ tau, const fl
     using S = YxyShape<L>;
     constexpr int M = S::M, P = S::P, RW = S::RW;
     constexpr int N = L;
-    constexpr int EX = Split<M>::E, TPX = Split<M>::TP, RS = row_stride<M>();
+    constexpr int EX = Split<L>::E, TPX = Split<L>::TP, RS = row_stride<L>();
     extern __shared__ __align__(16) float2 sh[];
     __shared__ float2 lut[16];
-    __shared__ float2 tws[2 * M];
+    __shared__ float2 tws[L];
     coef_pairs(lut, (float)g.Y[0], (float)g.Y[1], (float)g.Y[2]);
-    stage_twiddles<M>(tws, g);
+    stage_pair_twiddles<L>(tws, g);
     grid_begin();
     __syncthreads();
-    const float2* twM = tws;
-    const float2* twN = tws + M;
     const int nitems = g.nslots * nper;
     for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
         const int slot = item / nper, pz = item % nper;   // pz = component * N + z
@@ -909,24 +1356,25 @@ k_yxy(GridDesc g, unsigned mask, float2* spec, float* __restrict__ tau, const fl
             const bool addr = ADDR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
             float2* rs = sh + r * RS;
             for (int rb = 0; rb < N / RW; ++rb) {
-                const int y = rb * RW + r;
-                const long long row = (long long)pz * N + y;                   // c*NN + z*N + y
+                const int y = rb * RW + 2 * r;
+                const long long row = (long long)pz * N + y;                   // c*NN + z*N + y, the pair's first row
                 const long long fbase = (long long)slot * 3 * g.N3 + row * N;
                 float2 radd[EX];
-                if (addr) s2_load<M>(radd, reinterpret_cast<const float2*>(r32 + fbase), t);
+                if (addr) pair_load<L>(radd, r32 + fbase, r32 + fbase + L, t);
                 uchar2 q[EX];
-                s2_load_phase<M>(q, reinterpret_cast<const uchar2*>(g.phase + (row % g.NN) * N), t);
+                const uint8_t* ph = g.phase + (row % g.NN) * N;
+                pair_load_phase<L>(q, ph, ph + L, t);
                 float2* sp = plane + (long long)y * M;
                 float2 v[EX];
-                row_inverse<M, TPX, EX>(v, t, rs, sp, twM, twN);
+                pair_inverse<L>(v, t, rs, sp, sp + M, PairTwSmem<L>{tws});
 #pragma unroll
                 for (int j = 0; j < EX; ++j)
                     if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
-                if (WTAU) s2_store<M>(reinterpret_cast<float2*>(tau + fbase), v, t);
+                if (WTAU) pair_store<L>(tau + fbase, tau + fbase + L, v, t);
 #pragma unroll
                 for (int j = 0; j < EX; ++j) v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
                 row_sync<TPX>();
-                row_forward_split<M, TPX, EX>(v, t, rs, twM, twN, sp);
+                pair_forward<L>(v, t, rs, PairTwSmem<L>{tws}, sp, sp + M);
                 row_sync<TPX>();
             }
         }
@@ -1008,6 +1456,9 @@ template <int L> constexpr int fz_cols() { return pow2_cols(128 / fast::Split<L>
 // x passes run 128-thread CTAs: their barriers stall fewer warps and the load phases of
 // the CTAs on an SM drift apart (x round trip 400 -> 376 us at 256^3 against 256 threads)
 template <int M> constexpr int fx_rows() { return 128 / fast::Split<M>::TP; }
+// Grid sizes whose x passes run on row pairs; 96 and 512 keep single rows, whose transforms
+// hold half the values per thread (12 and 16 against 24 and 32).
+constexpr bool pair_rows(int N) { return N == 64 || N == 128 || N == 192 || N == 256; }
 }  // namespace
 
 #define HMG_FAST_LEN(L, X) \
@@ -1129,13 +1580,13 @@ bool fast_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* part
 
 int fast_x_ctas(const GridDesc& g) {
     int RW = 0;
-    switch (g.M) {
-        case 32: RW = fx_rows<32>(); break;
-        case 48: RW = fx_rows<48>(); break;
-        case 64: RW = fx_rows<64>(); break;
-        case 96: RW = fx_rows<96>(); break;
-        case 128: RW = fx_rows<128>(); break;
-        case 256: RW = fx_rows<256>(); break;
+    switch (g.N) {
+        case 64: RW = fast::PairShape<64>::RW; break;
+        case 96: RW = fx_rows<48>(); break;
+        case 128: RW = fast::PairShape<128>::RW; break;
+        case 192: RW = fast::PairShape<192>::RW; break;
+        case 256: RW = fast::PairShape<256>::RW; break;
+        case 512: RW = fx_rows<256>(); break;
         default: return 0;
     }
     if ((3 * g.NN) % RW || g.NN % RW) return 0;
@@ -1146,23 +1597,31 @@ bool fast_x_forward(const GridDesc& g, int mode, unsigned mask, const float* tau
                     cudaStream_t st) {
     float2* sp = reinterpret_cast<float2*>(spec);
     if (!fast_x_ctas(g)) return false;
-#define FXF(M)                                                                                                 \
+#define FXF(N_)                                                                                                \
     {                                                                                                          \
-        constexpr int RW = fx_rows<M>();                                                                       \
-        constexpr int T = RW * fast::Split<M>::TP;                                                             \
         dim3 grid(fast_x_ctas(g), g.nslots);                                                                   \
-        const size_t sm = sizeof(float2) * RW * fast::row_stride<M>();                                         \
-        if (mode == XF_PLAIN) launch_dyn(fast::k_fx_forward<M, RW, XF_PLAIN>, grid, T, sm, st, g, mask, tau, sp, partial); \
-        else if (mode == XF_POLARIZE) launch_dyn(fast::k_fx_forward<M, RW, XF_POLARIZE>, grid, T, sm, st, g, mask, tau, sp, partial); \
-        else launch_dyn(fast::k_fx_forward<M, RW, XF_FLUX>, grid, T, sm, st, g, mask, tau, sp, partial);        \
+        if constexpr (pair_rows(N_)) {                                                                         \
+            const size_t sm = sizeof(float2) * fast::PairShape<N_>::NP * fast::PairShape<N_>::RS;              \
+            auto k = mode == XF_PLAIN      ? fast::k_px_forward<N_, XF_PLAIN>                                  \
+                     : mode == XF_POLARIZE ? fast::k_px_forward<N_, XF_POLARIZE>                               \
+                                           : fast::k_px_forward<N_, XF_FLUX>;                                  \
+            launch_dyn(k, grid, 128, sm, st, g, mask, tau, sp, partial);                                       \
+        } else {                                                                                               \
+            constexpr int M = N_ / 2, RW = fx_rows<M>();                                                       \
+            const size_t sm = sizeof(float2) * RW * fast::row_stride<M>();                                     \
+            auto k = mode == XF_PLAIN      ? fast::k_fx_forward<M, RW, XF_PLAIN>                               \
+                     : mode == XF_POLARIZE ? fast::k_fx_forward<M, RW, XF_POLARIZE>                            \
+                                           : fast::k_fx_forward<M, RW, XF_FLUX>;                               \
+            launch_dyn(k, grid, RW * fast::Split<M>::TP, sm, st, g, mask, tau, sp, partial);                   \
+        }                                                                                                      \
     }
-    switch (g.M) {
-        HMG_FAST_LEN(32, FXF)
-        HMG_FAST_LEN(48, FXF)
+    switch (g.N) {
         HMG_FAST_LEN(64, FXF)
         HMG_FAST_LEN(96, FXF)
         HMG_FAST_LEN(128, FXF)
+        HMG_FAST_LEN(192, FXF)
         HMG_FAST_LEN(256, FXF)
+        HMG_FAST_LEN(512, FXF)
         default: return false;
     }
 #undef FXF
@@ -1174,26 +1633,34 @@ bool fast_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec
     if (!fast_x_ctas(g)) return false;
     if (mode != XI_PLAIN && mode != XI_INPLACE && mode != XI_INPLACE_RES && mode != XI_ADD_R_RES && mode != XI_ADD_R)
         return false;
-#define FXI(M)                                                                                                         \
-    {                                                                                                                  \
-        constexpr int RW = fx_rows<M>();                                                                               \
-        constexpr int T = RW * fast::Split<M>::TP;                                                                     \
-        dim3 grid(fast_x_ctas(g), g.nslots);                                                                           \
-        const size_t sm = sizeof(float2) * RW * fast::row_stride<M>();                                                 \
-        if (mode == XI_INPLACE_RES) launch_dyn(fast::k_fx_inverse<M, RW, XI_INPLACE_RES>, grid, T, sm, st, g, mask, sp, tau, r32, partial); \
-        else if (mode == XI_ADD_R_RES) launch_dyn(fast::k_fx_inverse<M, RW, XI_ADD_R_RES>, grid, T, sm, st, g, mask, sp, tau, r32, partial); \
-        else if (mode == XI_ADD_R) launch_dyn(fast::k_fx_inverse<M, RW, XI_ADD_R>, grid, T, sm, st, g, mask, sp, tau, r32, partial); \
-        else launch_dyn(fast::k_fx_inverse<M, RW, XI_INPLACE>, grid, T, sm, st, g, mask, sp, tau, r32, partial);        \
+#define FXI_PICK(K, ...)                                                \
+    (mode == XI_INPLACE_RES ? fast::K<__VA_ARGS__, XI_INPLACE_RES>       \
+     : mode == XI_ADD_R_RES ? fast::K<__VA_ARGS__, XI_ADD_R_RES>         \
+     : mode == XI_ADD_R     ? fast::K<__VA_ARGS__, XI_ADD_R>             \
+                            : fast::K<__VA_ARGS__, XI_INPLACE>)
+#define FXI(N_)                                                                                             \
+    {                                                                                                       \
+        dim3 grid(fast_x_ctas(g), g.nslots);                                                                \
+        if constexpr (pair_rows(N_)) {                                                                      \
+            const size_t sm = sizeof(float2) * fast::PairShape<N_>::NP * fast::PairShape<N_>::RS;           \
+            launch_dyn(FXI_PICK(k_px_inverse, N_), grid, 128, sm, st, g, mask, sp, tau, r32, partial);      \
+        } else {                                                                                            \
+            constexpr int M = N_ / 2, RW = fx_rows<M>();                                                    \
+            const size_t sm = sizeof(float2) * RW * fast::row_stride<M>();                                  \
+            launch_dyn(FXI_PICK(k_fx_inverse, M, RW), grid, RW * fast::Split<M>::TP, sm, st, g, mask, sp,   \
+                       tau, r32, partial);                                                                  \
+        }                                                                                                   \
     }
-    switch (g.M) {
-        HMG_FAST_LEN(32, FXI)
-        HMG_FAST_LEN(48, FXI)
+    switch (g.N) {
         HMG_FAST_LEN(64, FXI)
         HMG_FAST_LEN(96, FXI)
         HMG_FAST_LEN(128, FXI)
+        HMG_FAST_LEN(192, FXI)
         HMG_FAST_LEN(256, FXI)
+        HMG_FAST_LEN(512, FXI)
         default: return false;
     }
+#undef FXI_PICK
 #undef FXI
 }
 
@@ -1203,28 +1670,33 @@ bool chain_sweeps(const GridDesc& g) {
 }
 
 namespace {
-template <int M, bool ADDR, bool WTAU>
-void launch_round_p(const GridDesc& g, unsigned mask, float2* sp, float* tau, const float* r32, cudaStream_t st) {
-    constexpr int RW = fx_rows<M>();
-    constexpr int T = RW * fast::Split<M>::TP;
-    constexpr size_t sm = fast::RoundSmem<M, RW>::total;
-    auto kern = fast::k_fx_round_p<M, RW, ADDR, WTAU>;
+// The x round trip of size N: as a persistent kernel (staged rows) or one launch per CTA.
+template <int N, bool ADDR, bool WTAU>
+void launch_round(bool persistent, const GridDesc& g, unsigned mask, float2* sp, float* tau, const float* r32,
+                  cudaStream_t st) {
     const int nblk = fast_x_ctas(g);
-    const int grid = persistent_grid(kern, T, sm, nblk * g.nslots);
-    launch_kernel(small_grid(g, sizeof(float)), kern, grid, T, sm, st, g, mask, sp, tau, r32, nblk);
-}
-}  // namespace
-
-namespace {
-int fast_split_e(int M) {
-    switch (M) {
-        case 32: return fast::Split<32>::E;
-        case 48: return fast::Split<48>::E;
-        case 64: return fast::Split<64>::E;
-        case 96: return fast::Split<96>::E;
-        case 128: return fast::Split<128>::E;
-        case 256: return fast::Split<256>::E;
-        default: return 0;
+    const dim3 grid(nblk, g.nslots);
+    if constexpr (pair_rows(N)) {
+        using S = fast::PairShape<N>;
+        if (persistent) {
+            auto kern = fast::k_px_round_p<N, ADDR, WTAU>;
+            constexpr size_t sm = fast::PairSmem<N>::total;
+            const int ctas = persistent_grid(kern, 128, sm, nblk * g.nslots);
+            launch_kernel(small_grid(g, sizeof(float)), kern, ctas, 128, sm, st, g, mask, sp, tau, r32, nblk);
+        } else {
+            launch_dyn(fast::k_px_round<N, ADDR, WTAU>, grid, 128, sizeof(float2) * S::NP * S::RS, st, g, mask, sp, tau, r32);
+        }
+    } else {
+        constexpr int M = N / 2, RW = fx_rows<M>(), T = RW * fast::Split<M>::TP;
+        if (persistent) {
+            auto kern = fast::k_fx_round_p<M, RW, ADDR, WTAU>;
+            constexpr size_t sm = fast::RoundSmem<M, RW>::total;
+            const int ctas = persistent_grid(kern, T, sm, nblk * g.nslots);
+            launch_kernel(small_grid(g, sizeof(float)), kern, ctas, T, sm, st, g, mask, sp, tau, r32, nblk);
+        } else {
+            launch_dyn(fast::k_fx_round<M, RW, ADDR, WTAU>, grid, T, sizeof(float2) * RW * fast::row_stride<M>(), st, g,
+                       mask, sp, tau, r32);
+        }
     }
 }
 }  // namespace
@@ -1246,45 +1718,23 @@ bool fast_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* 
                   cudaStream_t st) {
     float2* sp = reinterpret_cast<float2*>(spec);
     if (!fast_x_ctas(g)) return gen_x_round(g, addr, wtau, mask, spec, tau, r32, st);
-    // the persistent form of the correction sweeps (r added) of 24-value rows would keep
+    // the persistent form of the correction sweeps (r added) of 24-value rows (N = 192) would keep
     // r in registers beside the transform and spill; those use the plain kernel
-    if (g.xpers && !(addr && fast_split_e(g.M) > 16)) {
-#define FXRP(M)                                                                            \
-    {                                                                                      \
-        if (addr && wtau) launch_round_p<M, true, true>(g, mask, sp, tau, r32, st);        \
-        else if (addr) launch_round_p<M, true, false>(g, mask, sp, tau, r32, st);          \
-        else if (wtau) launch_round_p<M, false, true>(g, mask, sp, tau, r32, st);          \
-        else launch_round_p<M, false, false>(g, mask, sp, tau, r32, st);                   \
+    const bool pers = g.xpers && !(addr && g.N == 192);
+#define FXR(N_)                                                                              \
+    {                                                                                        \
+        if (addr && wtau) launch_round<N_, true, true>(pers, g, mask, sp, tau, r32, st);      \
+        else if (addr) launch_round<N_, true, false>(pers, g, mask, sp, tau, r32, st);        \
+        else if (wtau) launch_round<N_, false, true>(pers, g, mask, sp, tau, r32, st);        \
+        else launch_round<N_, false, false>(pers, g, mask, sp, tau, r32, st);                 \
     }
-        switch (g.M) {
-            HMG_FAST_LEN(32, FXRP)
-            HMG_FAST_LEN(48, FXRP)
-            HMG_FAST_LEN(64, FXRP)
-            HMG_FAST_LEN(96, FXRP)
-            HMG_FAST_LEN(128, FXRP)
-            HMG_FAST_LEN(256, FXRP)
-            default: return false;
-        }
-#undef FXRP
-    }
-#define FXR(M)                                                                                                      \
-    {                                                                                                               \
-        constexpr int RW = fx_rows<M>();                                                                            \
-        constexpr int T = RW * fast::Split<M>::TP;                                                                  \
-        dim3 grid(fast_x_ctas(g), g.nslots);                                                                        \
-        const size_t sm = sizeof(float2) * RW * fast::row_stride<M>();                                              \
-        if (addr && wtau) launch_dyn(fast::k_fx_round<M, RW, true, true>, grid, T, sm, st, g, mask, sp, tau, r32);   \
-        else if (addr) launch_dyn(fast::k_fx_round<M, RW, true, false>, grid, T, sm, st, g, mask, sp, tau, r32);     \
-        else if (wtau) launch_dyn(fast::k_fx_round<M, RW, false, true>, grid, T, sm, st, g, mask, sp, tau, r32);     \
-        else launch_dyn(fast::k_fx_round<M, RW, false, false>, grid, T, sm, st, g, mask, sp, tau, r32);              \
-    }
-    switch (g.M) {
-        HMG_FAST_LEN(32, FXR)
-        HMG_FAST_LEN(48, FXR)
+    switch (g.N) {
         HMG_FAST_LEN(64, FXR)
         HMG_FAST_LEN(96, FXR)
         HMG_FAST_LEN(128, FXR)
+        HMG_FAST_LEN(192, FXR)
         HMG_FAST_LEN(256, FXR)
+        HMG_FAST_LEN(512, FXR)
         default: return false;
     }
 #undef FXR
