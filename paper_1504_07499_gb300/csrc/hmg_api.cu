@@ -174,6 +174,7 @@ GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d
     for (int s = 0; s < kMaxSlots; ++s)
         for (int c = 0; c < 3; ++c) g.E[s][c] = (s == c) ? 1.0 : 0.0;
     g.nslots = nslots;
+    g.comps = 3;
     g.expA = exps;
     g.expB = exps ? exps + 3 * (size_t)nslots * g.NN : nullptr;
     g.phase = phase_d;
@@ -413,7 +414,7 @@ bool SolveState::ensure(Context* c, int N_, bool fp64_, int nslots_) {
     partial = (double*)c->alloc(np * sizeof(double));
     partial2 = (double*)c->alloc(np * sizeof(double));
     partial3 = (double*)c->alloc(np * sizeof(double));
-    red = (double*)c->alloc(64 * sizeof(double));
+    red = (double*)c->alloc(kRedDoubles * sizeof(double));
     bool ok = phase && tau64 && spec64 && exps && partial && partial2 && partial3 && red &&
               (fp64 || (f32buf && r32 && spec32));
     if (!ok) {
@@ -429,7 +430,18 @@ void SolveState::free_all(Context* c) {
         c->release(*p);
         *p = nullptr;
     }
+    if (pin) cudaFreeHost(pin);
+    pin = nullptr;
     N = 0;
+}
+
+bool SolveState::pinned() {
+    if (!pin && cudaMallocHost(&pin, (kRedDoubles + 8) * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        pin = nullptr;
+        set_error("cannot allocate pinned host memory");
+    }
+    return pin != nullptr;
 }
 
 // ---------------------------------------------------------------------------
@@ -529,7 +541,7 @@ static constexpr int kind_of(int k) {
 
 template <typename R>
 void Solver::sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, const float* r32in,
-                   float* d32, float* r32out, int red_off) {
+                   float* d32, float* r32out, double* sums, const StopRule& stop) {
     const double f = (double)popc(mask) * 3.0 * (double)g.N3;   // field elements moved per array
     const double F = sizeof(R);
     const bool fused = std::is_same<R, float>::value && g.xyvar == 1 && fused_cluster(g.N) != 0;
@@ -556,7 +568,7 @@ void Solver::sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, c
                    launch_x_inverse<R>(g, ximode, mask, spec, field, r32in, d32, r32out, pb, st));
     }
     if (ximode == XI_INPLACE_RES || ximode == XI_ADD_R_RES || ximode == XI_DIFF)
-        HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 1, s->red + red_off, st));
+        HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 1, sums, st, stop));
 }
 
 bool Solver::chained() const { return chain_sweeps(g); }
@@ -565,7 +577,7 @@ void Solver::block_sweep(unsigned mask, int b, int blk, int zmode, bool addr, co
     const bool last = b == blk - 1;
     const int ximode = addr ? (last ? XI_ADD_R_RES : XI_ADD_R) : (last ? XI_INPLACE_RES : XI_INPLACE);
     if (!chained()) {
-        sweep<float>(mask, s->f32buf, s->spec32, zmode, ximode, r32in, nullptr, nullptr, red_off);
+        sweep<float>(mask, s->f32buf, s->spec32, zmode, ximode, r32in, nullptr, nullptr, s->red + red_off);
         return;
     }
     const double f = (double)popc(mask) * 3.0 * (double)g.N3;   // field elements moved per array
@@ -634,6 +646,23 @@ double Solver::eps_from_sum(double sum, int slot) const {
     return std::sqrt(sum / (double)g.N3) * g.epsf / nE;
 }
 
+// Smallest sum whose eps_comp is not below tol: every rounded operation of eps_from_sum is
+// monotone, so one threshold on the sum gives the same decisions without a root and two
+// divisions in the reduction kernel.  Bisection over the bit patterns of positive doubles.
+double Solver::least_sum(double tol, int slot) const {
+    uint64_t lo = 0, hi = 0x7ff0000000000000ull;   // eps(lo) < tol <= eps(hi)
+    while (hi - lo > 1) {
+        const uint64_t mid = lo + (hi - lo) / 2;
+        double x;
+        memcpy(&x, &mid, sizeof x);
+        if (eps_from_sum(x, slot) < tol) lo = mid;
+        else hi = mid;
+    }
+    double x;
+    memcpy(&x, &hi, sizeof x);
+    return x;
+}
+
 // eq check of the slots in `mask`; fills eps_eq and the mean flux <k e>
 template <typename R>
 bool Solver::check_eq(unsigned mask, const R* field, void* spec, double eps_eq[3], double flux[3][3]) {
@@ -652,15 +681,28 @@ bool Solver::check_eq(unsigned mask, const R* field, void* spec, double eps_eq[3
     return true;
 }
 
-// Plain FP64 method: the Algorithm of §3 in its printed order.
+// Plain FP64 method: the Algorithm of §3 in its printed order, per gradient.  Up to kAhead64
+// sweeps are launched before the host looks at their residuals: the reduction of each residual
+// clears its gradient's flag on the device when step 1 is due (or the residual is not a
+// number), and the sweeps behind it skip that gradient.  Every gradient goes through the
+// sequence of sweeps and tests that one look per sweep would give.
 hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9]) {
+    if (!s->pinned()) return HMG_OUT_OF_MEMORY;
     const unsigned all = (1u << g.nslots) - 1u;
     HMG_TRACED(HMG_K_OTHER, 0.0, launch_init_tau<double>(g, all, s->tau64, st));
     double eps_comp[3] = {INFINITY, INFINITY, INFINITY}, eps_eq[3] = {INFINITY, INFINITY, INFINITY};
     double flux[3][3] = {};
     int iters[3] = {0, 0, 0}, status[3] = {HMG_NOT_CONVERGED, HMG_NOT_CONVERGED, HMG_NOT_CONVERGED};
-    unsigned active = all;
-    for (int n = 0; n < max_iter && active; ++n) {
+    unsigned active = max_iter > 0 ? all : 0u;
+    StopRule stop;
+    stop.flags = reinterpret_cast<int*>(s->red + 56);
+    for (int sl = 0; sl < g.nslots; ++sl) stop.least[sl] = least_sum(tol, sl);
+    Solver ahead = *this;
+    ahead.g.dflags = stop.flags;
+    double* h = s->pin;                                           // sums of the block's sweeps
+    int* hf = reinterpret_cast<int*>(s->pin + kRedDoubles);       // flags as set before the block
+    double rate = 0.0;                                            // last contraction per sweep
+    while (active) {
         unsigned eqm = 0;
         for (int sl = 0; sl < g.nslots; ++sl)
             if (((active >> sl) & 1u) && eps_comp[sl] < tol) eqm |= 1u << sl;
@@ -673,16 +715,43 @@ hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9
                 }
             if (!active) break;
         }
-        sweep<double>(active, s->tau64, s->spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr);
-        double h[3];
-        if (!fetch(h, 0, g.nslots)) return HMG_CUDA_ERROR;
+        // sweeps to launch: as many as the slowest gradient still seems to need
+        int blk = 1;
+        for (int sl = 0; sl < g.nslots; ++sl) {
+            hf[sl] = (active >> sl) & 1u ? SF_ACTIVE : 0;
+            if (!hf[sl]) continue;
+            double need = kAhead64;
+            if (std::isfinite(eps_comp[sl]) && rate > 0.0 && rate < 1.0)
+                need = eps_comp[sl] > tol ? std::ceil(std::log(tol / eps_comp[sl]) / std::log(rate)) : 1.0;
+            blk = std::max(blk, (int)std::min((double)kAhead64, need));
+        }
+        for (int sl = 0; sl < g.nslots; ++sl)
+            if ((active >> sl) & 1u) blk = std::min(blk, max_iter - iters[sl]);
+        cudaMemcpyAsync(stop.flags, hf, 3 * sizeof(int), cudaMemcpyHostToDevice, st);
+        for (int b = 0; b < blk; ++b)
+            ahead.sweep<double>(active, s->tau64, s->spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr,
+                                s->red + 64 + 3 * b, stop);
+        cudaError_t ce = cudaMemcpyAsync(h, s->red + 64, 3 * blk * sizeof(double), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+        if (ce != cudaSuccess) {
+            set_error("CUDA error: %s", cudaGetErrorString(ce));
+            return HMG_CUDA_ERROR;
+        }
+        if (tr) tr->collect();
         for (int sl = 0; sl < g.nslots; ++sl) {
             if (!((active >> sl) & 1u)) continue;
-            ++iters[sl];
-            eps_comp[sl] = eps_from_sum(h[sl], sl);
+            for (int b = 0; b < blk; ++b) {
+                if (h[3 * b + sl] < 0.0) break;   // stopped at the sweep before
+                const double before = eps_comp[sl];
+                ++iters[sl];
+                eps_comp[sl] = eps_from_sum(h[3 * b + sl], sl);
+                if (std::isfinite(before) && before > 0.0) rate = eps_comp[sl] / before;
+            }
             if (!std::isfinite(eps_comp[sl])) {
                 status[sl] = HMG_DIVERGED;
                 active &= ~(1u << sl);
+            } else if (iters[sl] >= max_iter) {
+                active &= ~(1u << sl);   // out of sweeps
             }
         }
     }
@@ -737,12 +806,13 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
         return m;
     };
     Solver s64{g, s, st64, tr, s->partial3, s->partial3};
+    if (!s->pinned()) return HMG_OUT_OF_MEMORY;
     cudaEvent_t ready;
     if (cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) != cudaSuccess) {
         set_error("event create failed");
         return HMG_CUDA_ERROR;
     }
-    double h[64];
+    double* h = s->pin;
     int total = 0;
     hmg_status err = HMG_OK;
     while (mask_of(PH_DONE) != all && total < max_iter) {
@@ -754,7 +824,7 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
             cudaStreamWaitEvent(st64, ready, 0);
         }
         if (me) s64.equilibrium<double>(me, s->tau64, s->spec64);
-        if (mo) s64.sweep<double>(mo, s->tau64, s->spec64, Z_ITER, XI_DIFF, nullptr, s->f32buf, s->r32, 48);
+        if (mo) s64.sweep<double>(mo, s->tau64, s->spec64, Z_ITER, XI_DIFF, nullptr, s->f32buf, s->r32, s->red + 48);
         if (me || mo) cudaMemcpyAsync(h + 16, s->red + 16, 40 * sizeof(double), cudaMemcpyDeviceToHost, st64);
         // a block of FP32 sweeps: plain (phase A) and defect-correction (inner)
         const unsigned ma = mask_of(PH_A), mi = mask_of(PH_INNER);
@@ -768,7 +838,7 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
             total += blk - 1;
         }
         cudaError_t ce = cudaStreamSynchronize(st);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st64);
+        if (ce == cudaSuccess && (me || mo)) ce = cudaStreamSynchronize(st64);
         if (ce != cudaSuccess) {
             set_error("CUDA error: %s", cudaGetErrorString(ce));
             err = HMG_CUDA_ERROR;
@@ -883,8 +953,8 @@ hmg_status Solver::finish(const int status[3], const int iters[3], const int it6
     return HMG_OK;
 }
 
-template void Solver::sweep<float>(unsigned, float*, void*, int, int, const float*, float*, float*, int);
-template void Solver::sweep<double>(unsigned, double*, void*, int, int, const float*, float*, float*, int);
+template void Solver::sweep<float>(unsigned, float*, void*, int, int, const float*, float*, float*, double*, const StopRule&);
+template void Solver::sweep<double>(unsigned, double*, void*, int, int, const float*, float*, float*, double*, const StopRule&);
 template bool Solver::check_eq<float>(unsigned, const float*, void*, double*, double (*)[3]);
 template bool Solver::check_eq<double>(unsigned, const double*, void*, double*, double (*)[3]);
 

@@ -50,6 +50,18 @@ hmg_status check_common(hmg_ctx* ctx, int N, const void* p) {
     return HMG_OK;
 }
 
+// Whether kernels may use a caller's buffer in place: device memory of the context's GPU on a
+// 16-byte boundary.  Anything else is copied through the solve state.
+bool in_place(const hmg_ctx* ctx, const void* p) {
+    cudaPointerAttributes a;
+    if (reinterpret_cast<uintptr_t>(p) % 16 != 0) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
+}
+
 // Bring the phase grid onto the device and build the solve descriptor.
 hmg_status prepare(hmg_ctx* ctx, const uint8_t* phase, int N, const double k[3], bool fp64, int nslots,
                    GridDesc* g, int scheme = HMG_SCHEME_EYRE_MILTON, double beta = 2.0) {
@@ -395,9 +407,10 @@ hmg_status solve_impl(hmg_ctx* ctx, const uint8_t* phase, int N, double km, doub
     if (st != HMG_OK) return st;
     if (e_out) {
         const long long N3 = g.N3;
-        double* tmp = reinterpret_cast<double*>(ctx->solve.spec64);   // 9 N^3 doubles of scratch
+        const bool direct = in_place(ctx, e_out);
+        double* tmp = direct ? e_out : reinterpret_cast<double*>(ctx->solve.spec64);   // 9 N^3 doubles of scratch
         for (int j = 0; j < 3; ++j) launch_tau_to_e<double>(g, j, ctx->solve.tau64, tmp + 3 * j * N3, ctx->stream);
-        st = cuda_status(copy_out(e_out, tmp, 9 * N3 * sizeof(double), ctx->stream), "field copy");
+        if (!direct) st = cuda_status(copy_out(e_out, tmp, 9 * N3 * sizeof(double), ctx->stream), "field copy");
         if (st == HMG_OK) st = check_launch(ctx, "field copy");
         if (st != HMG_OK) return st;
     }
@@ -458,22 +471,37 @@ hmg_status hmg_em_iterate(hmg_ctx* ctx, const uint8_t* phase, int N, double km, 
     for (int c = 0; c < 3; ++c) g.E[0][c] = grad_Theta[c];
     SolveState& s = ctx->solve;
     const long long N3 = g.N3;
-    double* tmp = reinterpret_cast<double*>(s.spec64);
-    st = cuda_status(copy_in(tmp, e_inout, 3 * N3 * sizeof(double), ctx->stream), "field copy");
+    const bool direct = in_place(ctx, e_inout);
+    double* tmp = direct ? e_inout : reinterpret_cast<double*>(s.spec64);
+    if (!direct) st = cuda_status(copy_in(tmp, e_inout, 3 * N3 * sizeof(double), ctx->stream), "field copy");
     if (st != HMG_OK) return st;
     Solver sv{g, &s, ctx->stream};
     if (fp64) launch_e_to_tau<double>(g, 0, tmp, s.tau64, ctx->stream);
     else launch_e_to_tau<float>(g, 0, tmp, s.f32buf, ctx->stream);
-    for (int n = 0; n < n_iter; ++n) {
-        if (fp64) sv.sweep<double>(1u, s.tau64, s.spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr);
-        else sv.sweep<float>(1u, s.f32buf, s.spec32, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr);
-        double h;
-        if (!sv.fetch(&h, 0, 1)) return HMG_CUDA_ERROR;
-        if (eps_out) eps_out[n] = sv.eps_from_sum(h, 0);
+    // the sweeps follow each other on the stream; their residual sums are read in one copy per
+    // scratch buffer of them (16 sweeps at 192^3 in FP32: 4.26 -> 3.94 ms)
+    const int room = (int)(hmg_ctx::kScratchBytes / sizeof(double));
+    double* sums = (double*)ctx->scratch_get(hmg_ctx::kScratchBytes);
+    if (!sums) {
+        set_error("cannot allocate residual sums");
+        return HMG_OUT_OF_MEMORY;
+    }
+    std::vector<double> h(std::min(n_iter, room));
+    for (int n = 0; n < n_iter;) {
+        const int cnt = std::min(n_iter - n, room);
+        for (int b = 0; b < cnt; ++b) {
+            if (fp64) sv.sweep<double>(1u, s.tau64, s.spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b);
+            else sv.sweep<float>(1u, s.f32buf, s.spec32, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b);
+        }
+        st = cuda_status(cudaMemcpyAsync(h.data(), sums, cnt * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "sums");
+        if (st == HMG_OK) st = cuda_status(cudaStreamSynchronize(ctx->stream), "em_iterate");
+        if (st != HMG_OK) return st;
+        for (int b = 0; b < cnt && eps_out; ++b) eps_out[n + b] = sv.eps_from_sum(h[b], 0);
+        n += cnt;
     }
     if (fp64) launch_tau_to_e<double>(g, 0, s.tau64, tmp, ctx->stream);
     else launch_tau_to_e<float>(g, 0, s.f32buf, tmp, ctx->stream);
-    st = cuda_status(copy_out(e_inout, tmp, 3 * N3 * sizeof(double), ctx->stream), "field copy");
+    if (!direct) st = cuda_status(copy_out(e_inout, tmp, 3 * N3 * sizeof(double), ctx->stream), "field copy");
     if (st != HMG_OK) return st;
     return check_launch(ctx, "em_iterate");
 }
@@ -494,17 +522,21 @@ hmg_status hmg_equilibrium(hmg_ctx* ctx, const uint8_t* phase, int N, double km,
     st = prepare(ctx, phase, N, k, fp64, 1, &g);
     if (st != HMG_OK) return st;
     SolveState& s = ctx->solve;
-    double* tmp = reinterpret_cast<double*>(s.spec64);
-    st = cuda_status(copy_in(tmp, e, 3 * g.N3 * sizeof(double), ctx->stream), "field copy");
-    if (st != HMG_OK) return st;
+    const double* src = e;
+    if (!in_place(ctx, e)) {
+        double* tmp = reinterpret_cast<double*>(s.spec64);
+        st = cuda_status(copy_in(tmp, e, 3 * g.N3 * sizeof(double), ctx->stream), "field copy");
+        if (st != HMG_OK) return st;
+        src = tmp;
+    }
     Solver sv{g, &s, ctx->stream};
     double eps[3], flux[3][3];
     bool ok;
     if (fp64) {
-        launch_e_to_tau<double>(g, 0, tmp, s.tau64, ctx->stream);
+        launch_e_to_tau<double>(g, 0, src, s.tau64, ctx->stream);
         ok = sv.check_eq<double>(1u, s.tau64, s.spec64, eps, flux);
     } else {
-        launch_e_to_tau<float>(g, 0, tmp, s.f32buf, ctx->stream);
+        launch_e_to_tau<float>(g, 0, src, s.f32buf, ctx->stream);
         ok = sv.check_eq<float>(1u, s.f32buf, s.spec32, eps, flux);
     }
     if (!ok) return HMG_CUDA_ERROR;
@@ -545,48 +577,62 @@ static hmg_status fft_common(hmg_ctx* ctx, int N, int count, hmg_precision preci
     const long long N3 = g.N3;
     double* d64 = s.tau64;          // 3 N^3 doubles: staging of one group of three grids
     double* dsp = reinterpret_cast<double*>(s.spec64);
+    // Device buffers of this GPU are used where they are; the FP64 forward transform works inside
+    // the output buffer unless that is the input.
+    const size_t bytes = (size_t)count * N3 * sizeof(double);
+    const char *ib = reinterpret_cast<const char*>(in), *ob = reinterpret_cast<const char*>(out);
+    const bool apart = in == out || ib + bytes <= ob || ob + bytes <= ib;
+    const bool direct_in = in_place(ctx, in) && apart, direct_out = in_place(ctx, out) && apart;
     for (int base = 0; base < count; base += 3) {
         const int cnt = std::min(3, count - base);
-        cudaMemsetAsync(d64, 0, 3 * N3 * sizeof(double), ctx->stream);
-        st = cuda_status(copy_in(d64, in + (size_t)base * N3, cnt * N3 * sizeof(double), ctx->stream), "copy in");
-        if (st != HMG_OK) return st;
+        if (g.xyvar == 0) g.comps = cnt;   // (the fused x + y kernels take all three)
+        const double* src = in + (size_t)base * N3;
+        double* dst = out + (size_t)base * N3;
+        if (!direct_in) {
+            st = cuda_status(copy_in(d64, src, cnt * N3 * sizeof(double), ctx->stream), "copy in");
+            if (st != HMG_OK) return st;
+            src = d64;
+        }
         if (forward) {
             if (fp64) {
-                launch_x_forward<double>(g, XF_PLAIN, 1u, d64, dsp, nullptr, ctx->stream);
-                launch_y_pass<double>(g, true, 1u, dsp, ctx->stream);
-                launch_z_pass<double>(g, Z_FWD, 1u, dsp, nullptr, ctx->stream);
-                st = cuda_status(copy_out(out + (size_t)base * N3, dsp, cnt * N3 * sizeof(double), ctx->stream), "copy out");
+                double* sp = direct_out && in != out ? dst : dsp;
+                launch_x_forward<double>(g, XF_PLAIN, 1u, src, sp, nullptr, ctx->stream);
+                launch_y_pass<double>(g, true, 1u, sp, ctx->stream);
+                launch_z_pass<double>(g, Z_FWD, 1u, sp, nullptr, ctx->stream);
+                if (sp == dsp) st = cuda_status(copy_out(dst, dsp, cnt * N3 * sizeof(double), ctx->stream), "copy out");
             } else {
                 float* f = s.f32buf;
                 float* sp = reinterpret_cast<float*>(s.spec32);
-                launch_convert<float>(d64, f, 3 * N3, ctx->stream);
+                double* res = direct_out ? dst : dsp;
+                launch_convert<float>(src, f, cnt * N3, ctx->stream);
                 launch_xy_forward<float>(g, XF_PLAIN, 1u, f, sp, nullptr, ctx->stream);
                 launch_z_pass<float>(g, Z_FWD, 1u, sp, nullptr, ctx->stream);
-                launch_convert_back<float>(sp, dsp, 3 * N3, ctx->stream);
-                st = cuda_status(copy_out(out + (size_t)base * N3, dsp, cnt * N3 * sizeof(double), ctx->stream), "copy out");
+                launch_convert_back<float>(sp, res, cnt * N3, ctx->stream);
+                if (!direct_out) st = cuda_status(copy_out(dst, res, cnt * N3 * sizeof(double), ctx->stream), "copy out");
             }
         } else {
+            double* res = direct_out ? dst : d64;
             if (fp64) {
-                cudaMemcpyAsync(dsp, d64, 3 * N3 * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream);
-                launch_z_pass<double>(g, Z_INV, 1u, dsp, nullptr, ctx->stream);
+                launch_z_inverse_from(g, 1u, src, dsp, ctx->stream);
                 launch_y_pass<double>(g, false, 1u, dsp, ctx->stream);
-                launch_x_inverse<double>(g, XI_PLAIN, 1u, dsp, d64, nullptr, nullptr, nullptr, nullptr, ctx->stream);
-                st = cuda_status(copy_out(out + (size_t)base * N3, d64, cnt * N3 * sizeof(double), ctx->stream), "copy out");
+                launch_x_inverse<double>(g, XI_PLAIN, 1u, dsp, res, nullptr, nullptr, nullptr, nullptr, ctx->stream);
             } else {
                 float* f = s.f32buf;
                 float* sp = reinterpret_cast<float*>(s.spec32);
-                launch_convert<float>(d64, sp, 3 * N3, ctx->stream);
+                launch_convert<float>(src, sp, cnt * N3, ctx->stream);
                 launch_z_pass<float>(g, Z_INV, 1u, sp, nullptr, ctx->stream);
                 launch_yx_inverse<float>(g, XI_PLAIN, 1u, sp, f, nullptr, nullptr, nullptr, nullptr, ctx->stream);
-                launch_convert_back<float>(f, d64, 3 * N3, ctx->stream);
-                st = cuda_status(copy_out(out + (size_t)base * N3, d64, cnt * N3 * sizeof(double), ctx->stream), "copy out");
+                launch_convert_back<float>(f, res, cnt * N3, ctx->stream);
             }
+            if (!direct_out) st = cuda_status(copy_out(dst, res, cnt * N3 * sizeof(double), ctx->stream), "copy out");
         }
         if (st != HMG_OK) return st;
-        st = check_launch(ctx, forward ? "fft forward" : "fft inverse");
-        if (st != HMG_OK) return st;
+        if (!(direct_in && direct_out)) {   // host buffers: one group at a time
+            st = check_launch(ctx, forward ? "fft forward" : "fft inverse");
+            if (st != HMG_OK) return st;
+        }
     }
-    return HMG_OK;
+    return check_launch(ctx, forward ? "fft forward" : "fft inverse");
 }
 
 hmg_status hmg_fft_forward(hmg_ctx* ctx, int N, int count, hmg_precision precision, const double* x,

@@ -266,7 +266,7 @@ hmg_status Engine::tick_launch_and_update() {
             if (me[e->index]) sv.equilibrium<double>(me[e->index], e->st.tau64, e->st.spec64);
             if (mo[e->index])
                 sv.sweep<double>(mo[e->index], e->st.tau64, e->st.spec64, Z_ITER, XI_DIFF, nullptr, e->st.f32buf,
-                                 e->st.r32, 48);
+                                 e->st.r32, e->st.red + 48);
             cudaMemcpyAsync(hred + 64 * e->index + 16, e->st.red + 16, 40 * sizeof(double), cudaMemcpyDeviceToHost,
                             st64);
         }

@@ -553,8 +553,8 @@ k_fx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
     const int t = threadIdx.x % TP, r = threadIdx.x / TP;
     // component fastest across CTAs, so the three components of a (z, y) block read the
     // same phase rows close together in time (L2 hits)
-    const int comp = blockIdx.x % 3;
-    const long long rblk = blockIdx.x / 3;
+    const int comp = blockIdx.x % g.comps;
+    const long long rblk = blockIdx.x / g.comps;
     const long long row = comp * g.NN + rblk * RW + r;              // c*NN + z*N + y
     const long long pidx = comp * (g.NN / RW) + rblk;               // component-major CTA index
     const float2* src = reinterpret_cast<const float2*>(tau + (long long)slot * 3 * g.N3 + row * N);
@@ -697,8 +697,8 @@ k_fx_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     const int N = g.N;
     const int t = threadIdx.x % TP, r = threadIdx.x / TP;
     // component fastest across CTAs (phase rows reused from L2, as in k_fx_forward)
-    const int comp = blockIdx.x % 3;
-    const long long rblk = blockIdx.x / 3;
+    const int comp = blockIdx.x % g.comps;
+    const long long rblk = blockIdx.x / g.comps;
     const long long row = comp * g.NN + rblk * RW + r;              // c*NN + z*N + y
     const long long fbase = (long long)slot * 3 * g.N3 + row * N;
     const bool addr = ADDR && (g.dflags ? (g.dflags[slot] & SF_ADDR) != 0 : true);
@@ -1048,8 +1048,8 @@ k_px_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
     const int t = threadIdx.x % TP, r = threadIdx.x / TP;
     // component fastest across CTAs, so the three components of a (z, y) block read the
     // same phase rows close together in time (L2 hits)
-    const int comp = blockIdx.x % 3;
-    const long long rblk = blockIdx.x / 3;
+    const int comp = blockIdx.x % g.comps;
+    const long long rblk = blockIdx.x / g.comps;
     const long long row = comp * g.NN + rblk * S::RW + 2 * r;       // c*NN + z*N + y, the pair's first row
     const long long pidx = comp * (g.NN / S::RW) + rblk;            // component-major CTA index
     const float* src = tau + (long long)slot * 3 * g.N3 + row * L;
@@ -1470,7 +1470,7 @@ bool fast_y(const GridDesc& g, bool fwd, unsigned mask, void* spec, cudaStream_t
     {                                                                                             \
         constexpr int P = fy_cols<L>();                                                           \
         if (g.M % P) return false;                                                                \
-        dim3 grid(3 * g.N * (g.M / P), g.nslots);                                                 \
+        dim3 grid(g.comps * g.N * (g.M / P), g.nslots);                                                 \
         const size_t sm = sizeof(float2) * fast::xslots<L>() * P;                                 \
         if (fwd) launch_dyn(fast::k_fy<L, P, true>, grid, P * fast::Split<L>::TP, sm, st, g, mask, sp);  \
         else launch_dyn(fast::k_fy<L, P, false>, grid, P * fast::Split<L>::TP, sm, st, g, mask, sp);     \
@@ -1589,8 +1589,8 @@ int fast_x_ctas(const GridDesc& g) {
         case 512: RW = fx_rows<256>(); break;
         default: return 0;
     }
-    if ((3 * g.NN) % RW || g.NN % RW) return 0;
-    return (int)(3 * g.NN / RW);
+    if (g.NN % RW) return 0;
+    return (int)(g.comps * g.NN / RW);
 }
 
 bool fast_x_forward(const GridDesc& g, int mode, unsigned mask, const float* tau, void* spec, double* partial,

@@ -294,7 +294,7 @@ struct ColShape {
 
 template <int L>
 __global__ void __launch_bounds__(ColShape<L>::T, min_ctas(ColShape<L>::T, 1024))
-k_fxx_col(GridDesc g, unsigned mask, c64* __restrict__ spec, ColArgs a) {
+k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
     using C = ColShape<L>;
     using P = Plan<L>;
     using S = typename C::S;
@@ -317,6 +317,7 @@ k_fxx_col(GridDesc g, unsigned mask, c64* __restrict__ spec, ColArgs a) {
     const long long comp = (long long)slot * 3 + cw / L;         // (slot, c)
     const long long first = a.zdir ? comp * L * L * M + (long long)(cw % L) * M + kx : plane * L * M + kx;
     const long long step = a.zdir ? (long long)L * M : M;
+    const c64* in = src + first;   // the same buffer, or the FP64 spectrum of a plain inverse
     c64* base = spec + first;
     // exponent of element i: per (plane, y) for the y forward, per (component, i, kx) otherwise
     const int* ein = a.ein + (!a.zdir && !a.inverse ? plane * L : comp * L * M + kx);
@@ -331,7 +332,7 @@ k_fxx_col(GridDesc g, unsigned mask, c64* __restrict__ spec, ColArgs a) {
 #pragma unroll
             for (int q = 0; q < P::R0; ++q) {
                 const int i = j + q * J;
-                v[it][q] = base[i * step];
+                v[it][q] = in[i * step];
                 if (a.fp64_in)
                     mk = max(mk, max(key_of(__longlong_as_double(v[it][q].x)), key_of(__longlong_as_double(v[it][q].y))));
                 else

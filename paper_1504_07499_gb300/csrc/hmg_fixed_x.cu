@@ -6,7 +6,7 @@ namespace hmg {
 int fx_x_ctas(const GridDesc& g) {
     switch (g.N) {
 #define X(N_) \
-    case N_: return (int)(3 * g.NN / fx::x_rows<N_ / 2>());
+    case N_: return (int)(g.comps * g.NN / fx::x_rows<N_ / 2>());
         HMG_ALL_SIZES(X)
 #undef X
         default: return 0;

@@ -19,7 +19,7 @@ void launch(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, const 
 int gen_x_ctas(const GridDesc& g) {
     switch (g.N) {
 #define X(N_) \
-    case N_: return (int)(3 * g.NN / g32::x_rows<N_ / 2>());
+    case N_: return (int)(g.comps * g.NN / g32::x_rows<N_ / 2>());
         HMG_G32_SIZES(X)
 #undef X
         default: return 0;
@@ -90,7 +90,7 @@ bool gen_col(const GridDesc& g, bool zdir, bool forward, unsigned mask, void* sp
     switch (g.N) {
 #define X(N_)                                                                                               \
     case N_:                                                                                                \
-        launch(g32::k_gcol<N_>, dim3(3 * N_ * (N_ / 2 / g32::ColShape<N_>::NP), g.nslots),                   \
+        launch(g32::k_gcol<N_>, dim3(g.comps * N_ * (N_ / 2 / g32::ColShape<N_>::NP), g.nslots),             \
                g32::ColShape<N_>::T, g32::ColShape<N_>::smem, st, g, mask, zdir ? 1 : 0, forward ? 0 : 1,    \
                reinterpret_cast<float2*>(spec));                                                            \
         return true;

@@ -46,6 +46,8 @@ struct GridDesc {
     double relax;
     double E[kMaxSlots][3];  // macroscopic gradient of each right-hand side
     int nslots;            // right-hand sides held in the fields
+    int comps;             // components (grids of a plain transform) per slot that the x, y and column passes
+                           // of a launch cover, 3 but for a plain transform of one or two grids
     int zvar;              // z-pass kernel variant of the register-resident path (autotuned)
     int xyvar;             // 1: fused x + y cluster kernels, 0: separate x and y passes (autotuned)
     int nochain;           // 1: FP32 sweeps of a block are not chained through k_fx_round
@@ -88,6 +90,8 @@ void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, c
 template <typename R>
 void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial,
                    cudaStream_t st);
+// FP64 Z_INV of a plain transform from another buffer
+void launch_z_inverse_from(const GridDesc& g, unsigned mask, const void* src, void* spec, cudaStream_t st);
 // x inverse: writes tau (INPLACE*), adds r (ADD_R, ADD_R_RES), or writes d = new - old to
 // d32 and r32 without touching tau (DIFF).  Residual modes add (new-old)^2 per CTA.
 template <typename R>
@@ -146,7 +150,8 @@ void fx_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, 
                   double* partial, cudaStream_t st);
 void fx_y(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st);
 void fx_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st);
-void fx_z_plain(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st);
+// src: the packed FP64 spectrum an inverse reads (not changed); forward: in place, FP64 out
+void fx_z_plain(const GridDesc& g, bool forward, unsigned mask, const void* src, void* spec, cudaStream_t st);
 inline int fx_rcp_count(int N) { return 3 * (N / 2) * (N / 2) + 1; }
 void fx_rcp_table(long long* rcp, int N);   // device table of fx_rcp_count(N) entries, on the default stream
 
@@ -168,10 +173,17 @@ template <typename R>
 bool launch_yx_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, R* tau, const float* r32,
                        float* d32, float* r32_out, double* partial, cudaStream_t st);
 
+// Per-slot decision taken with a sweep's residual (FP64 solves): flags[slot] is cleared when
+// the residual's sum is below least[slot] or not finite.
+struct StopRule {
+    int* flags = nullptr;
+    double least[kMaxSlots] = {};
+};
+
 // Sum `count` partials of each of `nslots` rows in a fixed order: out[s] = sum_i p[s*count+i].
 // `groups` > 1 splits each row into that many equal consecutive groups (out[s*groups+g]).
-void launch_reduce(const double* partial, int nslots, int count, int groups, double* out,
-                   cudaStream_t st);
+void launch_reduce(const double* partial, int nslots, int count, int groups, double* out, cudaStream_t st,
+                   const StopRule& stop = StopRule());
 
 // Pointwise helpers on the fields.
 template <typename R>

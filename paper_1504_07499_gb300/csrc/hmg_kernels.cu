@@ -34,33 +34,46 @@ namespace hmg {
 // small device helpers
 // ---------------------------------------------------------------------------
 
-// Fixed-order CTA sum of one double per thread; result valid in thread 0.
+// Fixed-order CTA sum of one double per thread (T threads); result valid in thread 0.
+template <int T>
 __device__ double block_sum(double v, double* sh) {
     sh[threadIdx.x] = v;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    for (int s = T / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
         __syncthreads();
     }
-    double r = sh[0];
-    __syncthreads();
-    return r;
+    return sh[0];
 }
 
 // ---------------------------------------------------------------------------
 // reductions and pointwise helpers
 // ---------------------------------------------------------------------------
 
-__global__ void k_reduce(const double* __restrict__ partial, int count, int groups, double* __restrict__ out) {
-    __shared__ double red[kThreads];
+// Sum of the CTA partials of one slot (and group) by one CTA.  The chain of dependent FP64 adds
+// per thread is what it waits for, so large counts take 1024 threads (12 288 partials at 256^3:
+// 42 us with 256 threads) and small ones 256 (the tree over 1024 threads alone takes longer).
+// With stop.flags, a sweep residual also decides whether its slot goes on: the slot's flag is
+// cleared once the sum is below stop.least or not finite, and a slot that has stopped writes -1.
+template <int T>
+__global__ void __launch_bounds__(T)
+k_reduce(const double* __restrict__ partial, int count, int groups, double* __restrict__ out, StopRule stop) {
+    __shared__ double red[T];
     grid_begin();
     const int slot = blockIdx.x / groups, grp = blockIdx.x % groups;
+    const bool live = !stop.flags || (stop.flags[slot] & SF_ACTIVE);
+    if (!live) {   // uniform over the CTA
+        if (threadIdx.x == 0) out[blockIdx.x] = -1.0;
+        return;
+    }
     const int per = count / groups;
     const double* p = partial + (long long)slot * count + (long long)grp * per;
     double acc = 0.0;
-    for (int i = threadIdx.x; i < per; i += blockDim.x) acc += p[i];
-    double s = block_sum(acc, red);
-    if (threadIdx.x == 0) out[blockIdx.x] = s;
+    for (int i = threadIdx.x; i < per; i += T) acc += p[i];
+    const double s = block_sum<T>(acc, red);
+    if (threadIdx.x != 0) return;
+    out[blockIdx.x] = s;
+    if (stop.flags && !(s >= stop.least[slot] && isfinite(s))) stop.flags[slot] = 0;
 }
 
 template <typename R>
@@ -174,11 +187,15 @@ void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, c
 template <typename R>
 void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st) {
     if constexpr (std::is_same<R, double>::value) {
-        if (mode == Z_FWD || mode == Z_INV) fx_z_plain(g, mode == Z_FWD, mask, spec, st);
+        if (mode == Z_FWD || mode == Z_INV) fx_z_plain(g, mode == Z_FWD, mask, spec, spec, st);
         else fx_z(g, mode, mask, spec, partial, st);
     } else if (!fast_z(g, mode, mask, spec, partial, st)) {
         gen_z(g, mode, mask, spec, partial, st);
     }
+}
+
+void launch_z_inverse_from(const GridDesc& g, unsigned mask, const void* src, void* spec, cudaStream_t st) {
+    fx_z_plain(g, false, mask, src, spec, st);
 }
 
 template <typename R>
@@ -210,8 +227,11 @@ bool launch_yx_inverse(const GridDesc& g, int mode, unsigned mask, const void* s
     return false;
 }
 
-void launch_reduce(const double* partial, int nslots, int count, int groups, double* out, cudaStream_t st) {
-    launch_kernel(true, k_reduce, dim3(nslots * groups), kThreads, 0, st, partial, count, groups, out);
+void launch_reduce(const double* partial, int nslots, int count, int groups, double* out, cudaStream_t st,
+                   const StopRule& stop) {
+    const dim3 grid(nslots * groups);
+    if (count / groups > 4096) launch_kernel(true, k_reduce<1024>, grid, 1024, 0, st, partial, count, groups, out, stop);
+    else launch_kernel(true, k_reduce<256>, grid, 256, 0, st, partial, count, groups, out, stop);
 }
 
 template <typename R>

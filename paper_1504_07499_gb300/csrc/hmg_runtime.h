@@ -65,7 +65,10 @@ struct SolveState {
     double* partial2 = nullptr;   // equilibrium norm (z pass)
     double* partial3 = nullptr;   // FP64 work: correction sweep residual and flux average
     double* red = nullptr;   // [0,16): FP32 sweep sums, [16,32): flux sums, [32,48): eq sums,
-                             // [48,56): FP64 sweep sums
+                             // [48,56): FP64 sweep sums, [56,64): slot flags of an FP64 block (int),
+                             // [64,96): its sweep sums
+    double* pin = nullptr;   // pinned host copy of red and room for flags, made by the first solve
+    bool pinned();
     bool ensure(::hmg_ctx* c, int N, bool fp64, int nslots);
     void free_all(::hmg_ctx* c);
 };
@@ -98,6 +101,11 @@ struct Tracer {
     void reset();
     ~Tracer();
 };
+
+// Sweeps of a plain FP64 solve launched ahead of the host: each slot's residual decides on the
+// device whether its later sweeps of the block run, and the host follows once per block.
+constexpr int kAhead64 = 8;
+constexpr int kRedDoubles = 96;
 
 // FP32 sweeps of the bulk solver run in blocks of this many; the last sweep of a
 // block computes the residual and the host reads it once per block.
@@ -135,10 +143,10 @@ struct Solver {
     Tracer* tr = nullptr;
     double* psweep = nullptr;   // partial sums of sweeps (nullptr: s->partial)
     double* pflux = nullptr;    // partial sums of the flux average (nullptr: s->partial)
-    // one sweep of steps 2-7; residual modes leave the per-slot sums at red[red_off + slot]
+    // one sweep of steps 2-7; residual modes leave the per-slot sums at sums[slot]
     template <typename R>
     void sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, const float* r32in, float* d32,
-               float* r32out, int red_off = 0);
+               float* r32out, double* sums, const StopRule& stop = StopRule());
     // Sweep b of a block of blk FP32 sweeps on f32buf / spec32 (plain: Z_ITER without r;
     // correction: Z_ITER_NOB with r added).  Where the register-resident x kernels exist
     // the sweeps of a block are chained: the x inverse of sweep b and the x forward of
@@ -152,6 +160,7 @@ struct Solver {
     bool check_eq(unsigned mask, const R* field, void* spec, double eps_eq[3], double flux[3][3]);
     bool fetch(double* h, int off, int count);
     double eps_from_sum(double sum, int slot) const;
+    double least_sum(double tol, int slot) const;
     hmg_status run_fp64(int max_iter, double tol, hmg_info* info, double K[9]);
     hmg_status run_bulk(int max_iter, double tol, hmg_info* info, double K[9], cudaStream_t st64);
     hmg_status finish(const int status[3], const int iters[3], const int it64[3], const double eps_comp[3],
