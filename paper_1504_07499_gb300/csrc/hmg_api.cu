@@ -171,6 +171,7 @@ GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d
         g.relax = 1.0 - 0.5 * beta;
         g.epsf = 1.0 / (beta * k0);
     }
+    for (int p = 0; p < 3; ++p) g.YN[p] = g.Y[p] * (1.0 / (double)g.N3);
     for (int s = 0; s < kMaxSlots; ++s)
         for (int c = 0; c < 3; ++c) g.E[s][c] = (s == c) ? 1.0 : 0.0;
     g.nslots = nslots;
@@ -571,6 +572,41 @@ void Solver::sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, c
         HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 1, sums, st, stop));
 }
 
+template <typename R>
+void Solver::sweeps(unsigned mask, R* field, void* spec, int n, double* sums, int stride, const StopRule& stop) {
+    constexpr bool f64 = std::is_same<R, double>::value;
+    // The FP64 round trip pays where field and spectrum stay in L2 (kernels alone, us, two passes
+    // against one: 32^3 19 and 12, 72^3 86 and 55, one gradient at 128^3 140 and 94); beyond it
+    // reads and writes of one more array per kernel cost what they save (96^3 163 and 162,
+    // 192^3 357 and 360, 256^3 709 and 974).
+    const bool in_l2 = g.nslots * 3 * (double)g.N3 * sizeof(double) <= 56e6;
+    if (g.relax != 0.0 || (f64 ? !in_l2 : !fast_x_round_res_available(g))) {
+        for (int b = 0; b < n; ++b)
+            sweep<R>(mask, field, spec, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b * stride, stop);
+        return;
+    }
+    const double f = (double)popc(mask) * 3.0 * (double)g.N3, F = sizeof(R);   // field elements moved per array
+    double* pb = psweep ? psweep : s->partial;
+    for (int b = 0; b < n; ++b) {
+        if (b == 0)
+            HMG_TRACED(kind_of<R>(HMG_K_X_FORWARD), f * 2 * F + (double)g.N3,
+                       launch_x_forward<R>(g, XF_POLARIZE, mask, field, spec, nullptr, st));
+        HMG_TRACED(kind_of<R>(HMG_K_Y_FORWARD), f * 2 * F, launch_y_pass<R>(g, true, mask, spec, st));
+        HMG_TRACED(kind_of<R>(HMG_K_Z_GREEN), f * 2 * F, launch_z_pass<R>(g, Z_ITER, mask, spec, nullptr, st));
+        HMG_TRACED(kind_of<R>(HMG_K_Y_INVERSE), f * 2 * F, launch_y_pass<R>(g, false, mask, spec, st));
+        if (b == n - 1) {
+            HMG_TRACED(kind_of<R>(HMG_K_X_INVERSE), f * 3 * F,
+                       launch_x_inverse<R>(g, XI_INPLACE_RES, mask, spec, field, nullptr, nullptr, nullptr, pb, st));
+        } else if constexpr (f64) {
+            HMG_TRACED(HMG_K_FP64, f * 4 * F + (double)g.N3, fx_x_round(g, mask, spec, field, pb, st));
+        } else {
+            HMG_TRACED(HMG_K_X_ROUND, f * 4 * F + (double)g.N3, fast_x_round_res(g, mask, spec, field, pb, st));
+        }
+        HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0,
+                   launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 1, sums + b * stride, st, stop));
+    }
+}
+
 bool Solver::chained() const { return chain_sweeps(g); }
 
 void Solver::block_sweep(unsigned mask, int b, int blk, int zmode, bool addr, const float* r32in, int red_off) {
@@ -728,9 +764,7 @@ hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9
         for (int sl = 0; sl < g.nslots; ++sl)
             if ((active >> sl) & 1u) blk = std::min(blk, max_iter - iters[sl]);
         cudaMemcpyAsync(stop.flags, hf, 3 * sizeof(int), cudaMemcpyHostToDevice, st);
-        for (int b = 0; b < blk; ++b)
-            ahead.sweep<double>(active, s->tau64, s->spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr,
-                                s->red + 64 + 3 * b, stop);
+        ahead.sweeps<double>(active, s->tau64, s->spec64, blk, s->red + 64, 3, stop);
         cudaError_t ce = cudaMemcpyAsync(h, s->red + 64, 3 * blk * sizeof(double), cudaMemcpyDeviceToHost, st);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
         if (ce != cudaSuccess) {
@@ -955,6 +989,8 @@ hmg_status Solver::finish(const int status[3], const int iters[3], const int it6
 
 template void Solver::sweep<float>(unsigned, float*, void*, int, int, const float*, float*, float*, double*, const StopRule&);
 template void Solver::sweep<double>(unsigned, double*, void*, int, int, const float*, float*, float*, double*, const StopRule&);
+template void Solver::sweeps<float>(unsigned, float*, void*, int, double*, int, const StopRule&);
+template void Solver::sweeps<double>(unsigned, double*, void*, int, double*, int, const StopRule&);
 template bool Solver::check_eq<float>(unsigned, const float*, void*, double*, double (*)[3]);
 template bool Solver::check_eq<double>(unsigned, const double*, void*, double*, double (*)[3]);
 

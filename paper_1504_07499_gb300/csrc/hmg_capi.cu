@@ -489,10 +489,8 @@ hmg_status hmg_em_iterate(hmg_ctx* ctx, const uint8_t* phase, int N, double km, 
     std::vector<double> h(std::min(n_iter, room));
     for (int n = 0; n < n_iter;) {
         const int cnt = std::min(n_iter - n, room);
-        for (int b = 0; b < cnt; ++b) {
-            if (fp64) sv.sweep<double>(1u, s.tau64, s.spec64, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b);
-            else sv.sweep<float>(1u, s.f32buf, s.spec32, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b);
-        }
+        if (fp64) sv.sweeps<double>(1u, s.tau64, s.spec64, cnt, sums, 1);
+        else sv.sweeps<float>(1u, s.f32buf, s.spec32, cnt, sums, 1);
         st = cuda_status(cudaMemcpyAsync(h.data(), sums, cnt * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "sums");
         if (st == HMG_OK) st = cuda_status(cudaStreamSynchronize(ctx->stream), "em_iterate");
         if (st != HMG_OK) return st;

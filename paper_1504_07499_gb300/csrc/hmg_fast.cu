@@ -1134,10 +1134,12 @@ k_px_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
 }
 
 // x inverse of one sweep fused with the polarization and x forward of the next (k_fx_round),
-// on row pairs; same float operations as k_px_inverse followed by k_px_forward.
-template <int L, bool ADDR, bool WTAU>
+// on row pairs; same float operations as k_px_inverse followed by k_px_forward.  RES: the field
+// is compared with the stored one before it replaces it (sweeps that report every residual).
+template <int L, bool ADDR, bool WTAU, bool RES = false>
 __global__ void __launch_bounds__(128, 4)
-k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau, const float* __restrict__ r32) {
+k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau, const float* __restrict__ r32,
+           double* __restrict__ partial) {
     using S = PairShape<L>;
     constexpr int E = S::E, TP = S::TP, M = S::M;
     __shared__ float2 lut[16];
@@ -1156,6 +1158,7 @@ k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     // loads for the update and the polarization: in flight during the inverse FFT
     float2 radd[E];
     if (addr) pair_load<L>(radd, r32 + fbase, r32 + fbase + L, t);
+    if (RES) pair_load<L>(radd, tau + fbase, tau + fbase + L, t);   // the old field
     uchar2 q[E];
     const uint8_t* ph = g.phase + (row % g.NN) * L;
     pair_load_phase<L>(q, ph, ph + L, t);
@@ -1164,14 +1167,26 @@ k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     __syncthreads();   // tables and coefficient pairs
     float2 v[E];
     pair_inverse<L>(v, t, rs, sp, sp + M, PairTwSmem<L>{tws});
+    float acc = 0.f;
 #pragma unroll
-    for (int j = 0; j < E; ++j)
+    for (int j = 0; j < E; ++j) {
         if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
+        if (RES) {
+            const float da = v[j].x - radd[j].x, db = v[j].y - radd[j].y;
+            acc += da * da + db * db;
+        }
+    }
     if (WTAU) pair_store<L>(tau + fbase, tau + fbase + L, v, t);
 #pragma unroll
     for (int j = 0; j < E; ++j) v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
     row_sync<TP>();   // the pair's threads have read their stage-2 values from rs
     pair_forward<L>(v, t, rs, PairTwSmem<L>{tws}, sp, sp + M);
+    if (RES) {   // partials in the order of k_px_inverse
+        __shared__ double red[128];
+        const double s = block_sum_d((double)acc, red);
+        if (threadIdx.x == 0)
+            partial[(long long)slot * gridDim.x + (blockIdx.x % 3) * (g.NN / S::RW) + blockIdx.x / 3] = s;
+    }
 }
 
 // Dynamic shared memory of k_px_round_p: staged spectrum rows, phase rows, exchange buffers
@@ -1684,7 +1699,8 @@ void launch_round(bool persistent, const GridDesc& g, unsigned mask, float2* sp,
             const int ctas = persistent_grid(kern, 128, sm, nblk * g.nslots);
             launch_kernel(small_grid(g, sizeof(float)), kern, ctas, 128, sm, st, g, mask, sp, tau, r32, nblk);
         } else {
-            launch_dyn(fast::k_px_round<N, ADDR, WTAU>, grid, 128, sizeof(float2) * S::NP * S::RS, st, g, mask, sp, tau, r32);
+            launch_dyn(fast::k_px_round<N, ADDR, WTAU>, grid, 128, sizeof(float2) * S::NP * S::RS, st, g, mask, sp, tau, r32,
+                       nullptr);
         }
     } else {
         constexpr int M = N / 2, RW = fx_rows<M>(), T = RW * fast::Split<M>::TP;
@@ -1738,6 +1754,21 @@ bool fast_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* 
         default: return false;
     }
 #undef FXR
+}
+
+bool fast_x_round_res_available(const GridDesc& g) { return chain_sweeps(g) && pair_rows(g.N); }
+
+void fast_x_round_res(const GridDesc& g, unsigned mask, void* spec, float* tau, double* partial, cudaStream_t st) {
+    float2* sp = reinterpret_cast<float2*>(spec);
+    const dim3 grid(fast_x_ctas(g), g.nslots);
+#define FXRR(N_)                                                                                                   \
+    case N_:                                                                                                       \
+        launch_dyn(fast::k_px_round<N_, false, true, true>, grid, 128,                                             \
+                   sizeof(float2) * fast::PairShape<N_>::NP * fast::PairShape<N_>::RS, st, g, mask, sp, tau,        \
+                   (const float*)nullptr, partial);                                                                \
+        break;
+    switch (g.N) { FXRR(64) FXRR(128) FXRR(192) FXRR(256) }
+#undef FXRR
 }
 
 namespace {

@@ -497,6 +497,21 @@ __device__ __forceinline__ void transform(c64 (&v)[Plan<L>::I0][Plan<L>::R0], c6
         }
     }
 }
+// f(index, butterfly, value) over the places of the last stage's registers
+template <int L, class F>
+__device__ __forceinline__ void last_places(int t, F f) {
+    using P = Plan<L>;
+    constexpr int J = L / P::RL;
+#pragma unroll
+    for (int it = 0; it < P::IL; ++it) {
+        const int j = t + it * P::TPP;
+        if (J % P::TPP == 0 || j < J) {
+            const int base = (j / P::NL) * P::NL * P::RL + j % P::NL;
+#pragma unroll
+            for (int r = 0; r < P::RL; ++r) f(base + r * P::NL, it, r);
+        }
+    }
+}
 template <int L, class F>
 __device__ __forceinline__ void last_emit(const c64 (&o)[Plan<L>::IL][Plan<L>::RL], int t, F f) {
     stage_emit<L, Plan<L>::RL, Plan<L>::NL, Plan<L>::IL>(o, t, f);

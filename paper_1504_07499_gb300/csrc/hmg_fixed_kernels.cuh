@@ -79,6 +79,91 @@ struct XShape {
     static constexpr size_t smem = sizeof(c64) * S::TOTAL;
 };
 
+// Real split of a row transform (exponent e, scaled from values below 2^E) through shared memory
+// and its store to dst; om: one zeroed word per row.
+template <int M>
+__device__ __forceinline__ void split_store(const GridDesc& g, const c64 (&o)[Plan<M>::IL][Plan<M>::RL], int t, int r,
+                                            long long row, c64* dst, c64* sm, unsigned* om, int E, int e) {
+    using P = Plan<M>;
+    using S = typename XShape<M>::S;
+    constexpr int TPP = P::TPP;
+    if (P::NS > 1) __syncthreads();   // the last stage has been read by every thread
+    unsigned m = 0;
+    last_emit<M>(o, t, [&](int k, c64 z) {
+        m |= mag(z);
+        sm[S::at(k, r)] = z;
+    });
+    atomicOr(&om[r], m);
+    __syncthreads();
+    // real split: X_k = (Z_k + conj Z_{M-k} - i w_N^k (Z_k - conj Z_{M-k})) / 2, stored halved
+    const int sh = max(0, bits_of(om[r]) - 61);
+    e += 1 + sh;
+    for (int k = t; k < M; k += TPP) {
+        c64 z = sm[S::at(k, r)];
+        if (sh) z = shr_round(z, sh);
+        c64 out;
+        if (k == 0) {
+            out = mkc(half(z.x + z.y), half(z.x - z.y));
+        } else {
+            c64 zm = sm[S::at(M - k, r)];
+            if (sh) zm = shr_round(zm, sh);
+            const c64 w = cmul4(mkc(z.y + zm.y, zm.x - z.x), __ldg(&g.twf[k]));
+            out = quarter(mkc(z.x + zm.x, z.y - zm.y)) + w;
+        }
+        dst[k] = out;
+    }
+    if (t == 0) g.expA[row] = exp_is_nan(E) ? kExpNan : e;
+}
+
+// Complex-to-real merge of a packed row spectrum into the first stage of the inverse row
+// transform (a quarter of it; exponent e); returns whether the row is not a number.  key: one
+// word per row, kExpZero.
+template <int M>
+__device__ __forceinline__ bool load_merge(const GridDesc& g, c64 (&v)[Plan<M>::I0][Plan<M>::R0], int t, int r,
+                                           long long row, const c64* src, int* key, int& e) {
+    using P = Plan<M>;
+    constexpr int TPP = P::TPP, J = M / P::R0;
+    const int* ein = g.expB + (long long)((int)row / (2 * M)) * M;   // one exponent per kx of the (slot, c, z) plane
+    int mk = kExpZero;
+#pragma unroll
+    for (int it = 0; it < P::I0; ++it) {
+        const int j = t + it * TPP;
+        if (J % TPP == 0 || j < J) {
+#pragma unroll
+            for (int q = 0; q < P::R0; ++q) {
+                v[it][q] = src[j + q * J];
+                mk = max(mk, __ldg(&ein[j + q * J]) + bits_of(mag(v[it][q])));
+            }
+        }
+    }
+    atomicMax(&key[r], mk);
+    __syncthreads();
+    const int E = key[r];
+    e = E - first_bits(P::R0);
+    // complex-to-real merge, a quarter of it: (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k})
+#pragma unroll
+    for (int it = 0; it < P::I0; ++it) {
+        const int j = t + it * TPP;
+        if (J % TPP == 0 || j < J) {
+#pragma unroll
+            for (int q = 0; q < P::R0; ++q) {
+                const int k = j + q * J, km = k ? M - k : 0;
+                c64 a = shift(v[it][q], __ldg(&ein[k]) - e);
+                c64 b = shift(src[km], __ldg(&ein[km]) - e);
+                if (k == 0) {   // packed X(0) + i X(N/2)
+                    b = mkc(a.y, 0);
+                    a = mkc(a.x, 0);
+                }
+                const c64 s = quarter(mkc(a.x + b.x, a.y - b.y));
+                const c64 d = cmul4(mkc(a.x - b.x, a.y + b.y), conj_tw(__ldg(&g.twf[k])));
+                v[it][q] = swap_ri(mkc(s.x - d.y, s.y + d.x));
+            }
+        }
+    }
+    e += 2;
+    return exp_is_nan(E);
+}
+
 template <int M>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
 k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ tau, c64* __restrict__ spec,
@@ -102,16 +187,15 @@ k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ ta
     }
     const long long row = (long long)slot * 3 * N * N + (long long)blockIdx.x * RW + r;   // slot, c, z, y
     const double2* src = reinterpret_cast<const double2*>(tau) + row * M;
-    const uchar2* ph = reinterpret_cast<const uchar2*>(g.phase) + ((long long)blockIdx.x * RW + r) % ((long long)N * N) * M;
+    const uchar2* ph = reinterpret_cast<const uchar2*>(g.phase) + (long long)((int)(blockIdx.x * RW + r) % (N * N)) * M;
     __syncthreads();
     // load, coefficient product (FP64), largest exponent of the row
     c64 v[P::I0][P::R0];
     double acc = 0.0;
     int mk = kExpZero;
-    const double cs = mode == XF_POLARIZE ? 1.0 / (double)g.N3 : 1.0;   // 1/N^3 of the inverse transform
     double cf[3];
 #pragma unroll
-    for (int p = 0; p < 3; ++p) cf[p] = (mode == XF_FLUX ? g.W[p] : g.Y[p]) * cs;
+    for (int p = 0; p < 3; ++p) cf[p] = mode == XF_FLUX ? g.W[p] : g.YN[p];
 #pragma unroll
     for (int it = 0; it < P::I0; ++it) {
         const int j = t + it * TPP;
@@ -143,31 +227,7 @@ k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ ta
         }
     c64 o[P::IL][P::RL];
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
-    if (P::NS > 1) __syncthreads();   // the last stage has been read by every thread
-    unsigned m = 0;
-    last_emit<M>(o, t, [&](int k, c64 z) {
-        m |= mag(z);
-        sm[S::at(k, r)] = z;
-    });
-    atomicOr(&orm[2 * RW + r], m);
-    __syncthreads();
-    // real split: X_k = (Z_k + conj Z_{M-k} - i w_N^k (Z_k - conj Z_{M-k})) / 2, stored halved
-    const int sh = max(0, bits_of(orm[2 * RW + r]) - 61);
-    e += 1 + sh;
-    c64* dst = spec + row * M;
-    for (int k = t; k < M; k += TPP) {
-        const c64 z = shr_round(sm[S::at(k, r)], sh);
-        c64 out;
-        if (k == 0) {
-            out = mkc(half(z.x + z.y), half(z.x - z.y));
-        } else {
-            const c64 zm = shr_round(sm[S::at(M - k, r)], sh);
-            const c64 w = cmul4(mkc(z.y + zm.y, zm.x - z.x), __ldg(&g.twf[k]));
-            out = quarter(mkc(z.x + zm.x, z.y - zm.y)) + w;
-        }
-        dst[k] = out;
-    }
-    if (t == 0) g.expA[row] = exp_is_nan(E) ? kExpNan : e;
+    split_store<M>(g, o, t, r, row, spec + row * M, sm, orm + 2 * RW, E, e);
     if (mode == XF_FLUX) {
         const double s = cta_sum<T>(acc, red);
         if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
@@ -199,54 +259,16 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* __restrict__ spec,
         if (i < RW) key[i] = kExpZero;
     }
     const long long row = (long long)slot * 3 * N * N + (long long)blockIdx.x * RW + r;   // slot, c, z, y
-    const c64* src = spec + row * M;
-    const int* ein = g.expB + row / N * M;   // one exponent per kx of the (slot, c, z) plane
     __syncthreads();
     c64 v[P::I0][P::R0];
-    int mk = kExpZero;
-#pragma unroll
-    for (int it = 0; it < P::I0; ++it) {
-        const int j = t + it * TPP;
-        if (J % TPP == 0 || j < J) {
-#pragma unroll
-            for (int q = 0; q < P::R0; ++q) {
-                v[it][q] = src[j + q * J];
-                mk = max(mk, __ldg(&ein[j + q * J]) + bits_of(mag(v[it][q])));
-            }
-        }
-    }
-    atomicMax(&key[r], mk);
-    __syncthreads();
-    const int E = key[r];
-    int e = E - first_bits(P::R0);
-    // complex-to-real merge, a quarter of it: (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k})
-#pragma unroll
-    for (int it = 0; it < P::I0; ++it) {
-        const int j = t + it * TPP;
-        if (J % TPP == 0 || j < J) {
-#pragma unroll
-            for (int q = 0; q < P::R0; ++q) {
-                const int k = j + q * J, km = k ? M - k : 0;
-                c64 a = shift(v[it][q], __ldg(&ein[k]) - e);
-                c64 b = shift(src[km], __ldg(&ein[km]) - e);
-                if (k == 0) {   // packed X(0) + i X(N/2)
-                    b = mkc(a.y, 0);
-                    a = mkc(a.x, 0);
-                }
-                const c64 s = quarter(mkc(a.x + b.x, a.y - b.y));
-                const c64 d = cmul4(mkc(a.x - b.x, a.y + b.y), conj_tw(__ldg(&g.twf[k])));
-                v[it][q] = swap_ri(mkc(s.x - d.y, s.y + d.x));
-            }
-        }
-    }
-    e += 2;
+    int e;
+    const bool bad = load_merge<M>(g, v, t, r, row, spec + row * M, key, e);
     c64 o[P::IL][P::RL];
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
     // output step in FP64
     double2* out = reinterpret_cast<double2*>(tau) + row * M;
     float2* dout = reinterpret_cast<float2*>(d32) + row * M;
     float2* rout = reinterpret_cast<float2*>(r32) + row * M;
-    const bool bad = exp_is_nan(E);
     const bool relax = g.relax != 0.0, res = mode == XI_INPLACE_RES || mode == XI_DIFF;
     const double wn = 1.0 - g.relax, wo = g.relax;
     double acc = 0.0;
@@ -271,6 +293,84 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* __restrict__ spec,
         const double s = cta_sum<T>(acc, red);
         if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
     }
+}
+
+// x inverse of one sweep, field store and residual, polarization and x forward of the next, in
+// place on the spectrum: the values and operations of k_fxx_inverse (XI_INPLACE_RES) followed by
+// k_fxx_forward (XF_POLARIZE), without reading the field back (used where it is faster, see
+// Solver::sweeps).
+template <int M>
+__global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
+k_fxx_round(GridDesc g, unsigned mask, c64* spec, double* __restrict__ tau, double* __restrict__ partial) {
+    using X = XShape<M>;
+    using P = Plan<M>;
+    using S = typename X::S;
+    constexpr int N = X::N, RW = X::RW, TPP = X::TPP, T = X::T, J = M / P::R0;
+    grid_begin();
+    const int slot = blockIdx.y;
+    if (!slot_active(g, mask, slot)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    c64* sm = reinterpret_cast<c64*>(smem_raw);
+    __shared__ int key[2 * RW];
+    __shared__ unsigned orm[5 * RW];   // inverse stages, forward stages, spectrum
+    __shared__ double red[pow2_at_least(T)];
+    const int r = threadIdx.x / TPP, t = threadIdx.x % TPP;
+    for (int i = threadIdx.x; i < 5 * RW; i += T) {
+        orm[i] = 0;
+        if (i < 2 * RW) key[i] = kExpZero;
+    }
+    const long long row = (long long)slot * 3 * N * N + (long long)blockIdx.x * RW + r;   // slot, c, z, y
+    c64* sp = spec + row * M;
+    const uchar2* ph = reinterpret_cast<const uchar2*>(g.phase) + (long long)((int)(blockIdx.x * RW + r) % (N * N)) * M;
+    __syncthreads();
+    c64 v[P::I0][P::R0], o[P::IL][P::RL];
+    int e;
+    const bool bad = load_merge<M>(g, v, t, r, row, sp, key, e);
+    transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
+    if (P::NS > 1) __syncthreads();   // the last stage has been read by every thread
+    double2* out = reinterpret_cast<double2*>(tau) + row * M;
+    const double cf[3] = {g.YN[0], g.YN[1], g.YN[2]};
+    double acc = 0.0;
+    int mk = kExpZero;
+    // (loads first: one at a time between the stores they would each wait for memory, 3 to 5
+    // times the kernel's time on grids beyond L2)
+    double2 old[P::IL][P::RL];
+    uchar2 pq[P::IL][P::RL];
+    last_places<M>(t, [&](int k, int it, int q) {
+        old[it][q] = out[k];
+        pq[it][q] = ph[k];
+    });
+    last_places<M>(t, [&](int k, int it, int q) {
+        const c64 z = o[it][q];
+        double2 n = make_double2(from_fixed(z.y, e), from_fixed(z.x, e));
+        if (bad) n = make_double2(nan(""), nan(""));
+        const double da = n.x - old[it][q].x, db = n.y - old[it][q].y;
+        acc += da * da + db * db;
+        out[k] = n;
+        const uchar2 b = pq[it][q];
+        n.x *= coef3(b.x, cf);
+        n.y *= coef3(b.y, cf);
+        mk = max(mk, max(key_of(n.x), key_of(n.y)));
+        sm[S::at(k, r)] = mkc(__double_as_longlong(n.x), __double_as_longlong(n.y));
+    });
+    atomicMax(&key[RW + r], mk);
+    __syncthreads();
+    const int E = key[RW + r];
+    e = E - first_bits(P::R0);
+#pragma unroll
+    for (int it = 0; it < P::I0; ++it)
+        if (J % TPP == 0 || t + it * TPP < J) {
+#pragma unroll
+            for (int q = 0; q < P::R0; ++q) {
+                const c64 d = sm[S::at(t + it * TPP + q * J, r)];
+                v[it][q] = mkc(to_fixed(__longlong_as_double(d.x), e), to_fixed(__longlong_as_double(d.y), e));
+            }
+        }
+    __syncthreads();
+    transform<M, S>(v, o, t, r, sm, orm + 2 * RW, RW, e, g.twf + N);
+    split_store<M>(g, o, t, r, row, sp, sm, orm + 4 * RW, E, e);
+    const double s = cta_sum<T>(acc, red);
+    if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
 }
 
 // ---------------------------------------------------------------------------

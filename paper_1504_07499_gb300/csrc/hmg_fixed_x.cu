@@ -43,4 +43,18 @@ void fx_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, 
     }
 }
 
+void fx_x_round(const GridDesc& g, unsigned mask, void* spec, double* tau, double* partial, cudaStream_t st) {
+    fx::c64* sp = reinterpret_cast<fx::c64*>(spec);
+    const dim3 grid(fx_x_ctas(g), g.nslots);
+    switch (g.N) {
+#define X(N_)                                                                                            \
+    case N_:                                                                                             \
+        fx::launch(fx::k_fxx_round<N_ / 2>, grid, fx::XShape<N_ / 2>::T, fx::XShape<N_ / 2>::smem, st, g, mask, \
+                   sp, tau, partial);                                                                    \
+        break;
+        HMG_ALL_SIZES(X)
+#undef X
+    }
+}
+
 }  // namespace hmg

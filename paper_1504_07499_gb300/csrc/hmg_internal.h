@@ -30,6 +30,7 @@ struct GridDesc {
     int* expB;
     // per-phase coefficients, k0 = sqrt(min k * max k):
     double Y[3];           // (k - k0)/(k + k0): polarization factor of the sweep
+    double YN[3];          // Y / N^3 (FP64 sweeps: the scale of the inverse transform)
     double W[3];           // k/(k + k0): flux factor, phi = W tau
     double KP[3];          // k + k0: tau = (k + k0) e
     double k0;
@@ -115,6 +116,10 @@ bool fast_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec
 // spectrum; adds r (addr; per-slot flag in flags mode) and stores the updated field (wtau).
 bool fast_x_round(const GridDesc& g, bool addr, bool wtau, unsigned mask, void* spec, float* tau, const float* r32,
                   cudaStream_t st);
+// The same with the field stored and its residual partials (sweeps that report every residual;
+// sizes 64, 128, 192, 256 with chaining on).
+bool fast_x_round_res_available(const GridDesc& g);
+void fast_x_round_res(const GridDesc& g, unsigned mask, void* spec, float* tau, double* partial, cudaStream_t st);
 // FP32 sweeps of a block are chained (x inverse + next x forward in one kernel): separate x
 // and y passes, no relaxation, chaining not off.
 bool chain_sweeps(const GridDesc& g);
@@ -148,6 +153,8 @@ void fx_x_forward(const GridDesc& g, int mode, unsigned mask, const double* tau,
                   cudaStream_t st);
 void fx_x_inverse(const GridDesc& g, int mode, unsigned mask, const void* spec, double* tau, float* d32, float* r32,
                   double* partial, cudaStream_t st);
+// x inverse (XI_INPLACE_RES) of one sweep and x forward (XF_POLARIZE) of the next
+void fx_x_round(const GridDesc& g, unsigned mask, void* spec, double* tau, double* partial, cudaStream_t st);
 void fx_y(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st);
 void fx_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st);
 // src: the packed FP64 spectrum an inverse reads (not changed); forward: in place, FP64 out

@@ -147,6 +147,10 @@ struct Solver {
     template <typename R>
     void sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, const float* r32in, float* d32,
                float* r32out, double* sums, const StopRule& stop = StopRule());
+    // n sweeps on a field, each leaving its residual sums at sums + b stride; their x inverse
+    // and the next x forward are one kernel where such a kernel exists (same results)
+    template <typename R>
+    void sweeps(unsigned mask, R* field, void* spec, int n, double* sums, int stride, const StopRule& stop = StopRule());
     // Sweep b of a block of blk FP32 sweeps on f32buf / spec32 (plain: Z_ITER without r;
     // correction: Z_ITER_NOB with r added).  Where the register-resident x kernels exist
     // the sweeps of a block are chained: the x inverse of sweep b and the x forward of
