@@ -11,7 +11,11 @@ namespace hmg {
 
 namespace {
 enum { PH_A = 0, PH_OUTER = 1, PH_EQ = 2, PH_INNER = 3, PH_DONE = 4 };
-constexpr int kSideStreams = 16;
+// RVEs advanced at once within a tick.  Three fill the GPU with small grids and keep each one's
+// fields in L2 through its block of four sweeps; more evict each other (ms per batch at 1, 2, 3, 4,
+// 8, 16 streams: 5 x 64^3 + 4 x 96^3 + 3 x 128^3 418, 392, 390, 404, 419, 443; 12 x 64^3 157, 117, 109,
+// 109, 114, 129).
+constexpr int kSideStreams = 3;
 constexpr double kEta = 1e-4;       // correction sweeps reduce the FP64 residual by this factor
 constexpr int kStall = 24;          // sweeps without a new best FP32 residual = FP32 floor
 
