@@ -613,7 +613,7 @@ void Solver::block_sweep(unsigned mask, int b, int blk, int zmode, bool addr, co
     const bool last = b == blk - 1;
     const int ximode = addr ? (last ? XI_ADD_R_RES : XI_ADD_R) : (last ? XI_INPLACE_RES : XI_INPLACE);
     if (!chained()) {
-        sweep<float>(mask, s->f32buf, s->spec32, zmode, ximode, r32in, nullptr, nullptr, s->red + red_off);
+        sweep<float>(mask, s->f32buf, s->spec32, zmode, ximode, r32in, nullptr, nullptr, sums() + red_off);
         return;
     }
     const double f = (double)popc(mask) * 3.0 * (double)g.N3;   // field elements moved per array
@@ -642,7 +642,7 @@ void Solver::block_sweep(unsigned mask, int b, int blk, int zmode, bool addr, co
     const double xb = f * 3 * F + (addr ? f * F : 0.0);   // spectrum and old field in, field out
     HMG_TRACED(HMG_K_X_INVERSE, xb,
                launch_x_inverse<float>(g, ximode, mask, s->spec32, s->f32buf, r32in, nullptr, nullptr, pb, st));
-    HMG_TRACED(HMG_K_OTHER, 0.0, launch_reduce(pb, g.nslots, x_ctas_for<float>(g), 1, s->red + red_off, st));
+    HMG_TRACED(HMG_K_OTHER, 0.0, launch_reduce(pb, g.nslots, x_ctas_for<float>(g), 1, sums() + red_off, st));
 }
 
 template <typename R>
@@ -656,19 +656,21 @@ void Solver::equilibrium(unsigned mask, const R* field, void* spec) {
     } else {
         HMG_TRACED(kind_of<R>(HMG_K_EQ_X), f * 2 * F + (double)g.N3, launch_x_forward<R>(g, XF_FLUX, mask, field, spec, pb, st));
     }
-    HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 3, s->red + 16, st));
+    HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 3, sums() + 16, st));
     if (!fused) HMG_TRACED(kind_of<R>(HMG_K_Y_FORWARD), f * 2 * F, launch_y_pass<R>(g, true, mask, spec, st));
     HMG_TRACED(kind_of<R>(HMG_K_EQ_Z), f * F, launch_z_pass<R>(g, Z_EQ, mask, spec, s->partial2, st));
-    HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(s->partial2, g.nslots, z_ctas_for<R>(g), 1, s->red + 32, st));
+    HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0, launch_reduce(s->partial2, g.nslots, z_ctas_for<R>(g), 1, sums() + 32, st));
 }
 
 bool Solver::fetch(double* h, int off, int count) {
-    cudaError_t e = cudaMemcpyAsync(h, s->red + off, count * sizeof(double), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaSuccess;
+    if (!host) e = cudaMemcpyAsync(h, s->red + off, count * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         set_error("CUDA error: %s", cudaGetErrorString(e));
         return false;
     }
+    if (host) memcpy(h, host + off, count * sizeof(double));
     if (tr) tr->collect();
     return true;
 }
@@ -724,6 +726,7 @@ bool Solver::check_eq(unsigned mask, const R* field, void* spec, double eps_eq[3
 // sequence of sweeps and tests that one look per sweep would give.
 hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9]) {
     if (!s->pinned()) return HMG_OUT_OF_MEMORY;
+    host = s->pin;
     const unsigned all = (1u << g.nslots) - 1u;
     HMG_TRACED(HMG_K_OTHER, 0.0, launch_init_tau<double>(g, all, s->tau64, st));
     double eps_comp[3] = {INFINITY, INFINITY, INFINITY}, eps_eq[3] = {INFINITY, INFINITY, INFINITY};
@@ -735,7 +738,7 @@ hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9
     for (int sl = 0; sl < g.nslots; ++sl) stop.least[sl] = least_sum(tol, sl);
     Solver ahead = *this;
     ahead.g.dflags = stop.flags;
-    double* h = s->pin;                                           // sums of the block's sweeps
+    const double* h = s->pin + 64;                                // sums of the block's sweeps
     int* hf = reinterpret_cast<int*>(s->pin + kRedDoubles);       // flags as set before the block
     double rate = 0.0;                                            // last contraction per sweep
     while (active) {
@@ -764,9 +767,8 @@ hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9
         for (int sl = 0; sl < g.nslots; ++sl)
             if ((active >> sl) & 1u) blk = std::min(blk, max_iter - iters[sl]);
         cudaMemcpyAsync(stop.flags, hf, 3 * sizeof(int), cudaMemcpyHostToDevice, st);
-        ahead.sweeps<double>(active, s->tau64, s->spec64, blk, s->red + 64, 3, stop);
-        cudaError_t ce = cudaMemcpyAsync(h, s->red + 64, 3 * blk * sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+        ahead.sweeps<double>(active, s->tau64, s->spec64, blk, s->pin + 64, 3, stop);
+        const cudaError_t ce = cudaStreamSynchronize(st);
         if (ce != cudaSuccess) {
             set_error("CUDA error: %s", cudaGetErrorString(ce));
             return HMG_CUDA_ERROR;
@@ -839,14 +841,15 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
             if (state[sl] == ph) m |= 1u << sl;
         return m;
     };
-    Solver s64{g, s, st64, tr, s->partial3, s->partial3};
     if (!s->pinned()) return HMG_OUT_OF_MEMORY;
+    host = s->pin;
+    Solver s64{g, s, st64, tr, s->partial3, s->partial3, s->pin};
     cudaEvent_t ready;
     if (cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) != cudaSuccess) {
         set_error("event create failed");
         return HMG_CUDA_ERROR;
     }
-    double* h = s->pin;
+    const double* h = s->pin;
     int total = 0;
     hmg_status err = HMG_OK;
     while (mask_of(PH_DONE) != all && total < max_iter) {
@@ -858,8 +861,7 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
             cudaStreamWaitEvent(st64, ready, 0);
         }
         if (me) s64.equilibrium<double>(me, s->tau64, s->spec64);
-        if (mo) s64.sweep<double>(mo, s->tau64, s->spec64, Z_ITER, XI_DIFF, nullptr, s->f32buf, s->r32, s->red + 48);
-        if (me || mo) cudaMemcpyAsync(h + 16, s->red + 16, 40 * sizeof(double), cudaMemcpyDeviceToHost, st64);
+        if (mo) s64.sweep<double>(mo, s->tau64, s->spec64, Z_ITER, XI_DIFF, nullptr, s->f32buf, s->r32, s->pin + 48);
         // a block of FP32 sweeps: plain (phase A) and defect-correction (inner)
         const unsigned ma = mask_of(PH_A), mi = mask_of(PH_INNER);
         const int blk = std::max(1, std::min(kResidualEvery, max_iter - total + 1));
@@ -868,7 +870,6 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
                 if (ma) block_sweep(ma, b, blk, Z_ITER, false, nullptr, 0);
                 if (mi) block_sweep(mi, b, blk, Z_ITER_NOB, true, s->r32, 8);
             }
-            cudaMemcpyAsync(h, s->red, 16 * sizeof(double), cudaMemcpyDeviceToHost, st);
             total += blk - 1;
         }
         cudaError_t ce = cudaStreamSynchronize(st);

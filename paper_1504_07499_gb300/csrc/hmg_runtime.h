@@ -67,7 +67,9 @@ struct SolveState {
     double* red = nullptr;   // [0,16): FP32 sweep sums, [16,32): flux sums, [32,48): eq sums,
                              // [48,56): FP64 sweep sums, [56,64): slot flags of an FP64 block (int),
                              // [64,96): its sweep sums
-    double* pin = nullptr;   // pinned host copy of red and room for flags, made by the first solve
+    double* pin = nullptr;   // pinned host memory in the layout of red, written by the reductions of
+                             // a solve (no copy between a block and the host's look at it), and room
+                             // for flags; made by the first solve
     bool pinned();
     bool ensure(::hmg_ctx* c, int N, bool fp64, int nslots);
     void free_all(::hmg_ctx* c);
@@ -143,6 +145,8 @@ struct Solver {
     Tracer* tr = nullptr;
     double* psweep = nullptr;   // partial sums of sweeps (nullptr: s->partial)
     double* pflux = nullptr;    // partial sums of the flux average (nullptr: s->partial)
+    double* host = nullptr;     // pinned host memory the reductions write instead of s->red
+    double* sums() const { return host ? host : s->red; }
     // one sweep of steps 2-7; residual modes leave the per-slot sums at sums[slot]
     template <typename R>
     void sweep(unsigned mask, R* field, void* spec, int zmode, int ximode, const float* r32in, float* d32,
