@@ -81,11 +81,15 @@ __device__ __forceinline__ bool clear_of(float4 a, float4 b, const double* p, co
     return min_image_sq(p[0], p[1], p[2], q[0], q[1], q[2]) > lim;
 }
 
-// Sequential RSA in one CTA.  Each round examines kThreads consecutive candidates in
-// parallel against the accepted centres, then accepts them in draw order: the first
-// candidate still clear is accepted and the later ones are re-examined against it only.
-// out: 3 n doubles; state[0] = spheres placed, state[1] = candidates examined.
-__global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double lim, long long limit,
+// Sequential RSA in one CTA.  Each round examines kThreads candidates in parallel against the
+// accepted centres, then accepts them in draw order: the first candidate still clear is
+// accepted and the later ones are re-examined against it only.  The candidates are items
+// begin .. limit - 1, or, with a list, the candidates list[0 .. limit - 1], which the filter has
+// found clear of the first `known` centres.
+// out: 3 n doubles, the first state[0] of them placed before; state[0] = spheres placed,
+// state[1] = 1 + the last candidate examined.
+__global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double lim, long long begin, long long limit,
+                                                  const int* __restrict__ list, long long list_base,
                                                   double* __restrict__ out, long long* __restrict__ state) {
     __shared__ double acc[3 * kMaxSpheres];
     __shared__ float4 accf[kMaxSpheres];
@@ -93,12 +97,17 @@ __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double l
     __shared__ int s_first, s_count;
     const int t = threadIdx.x;
     const float limf = (float)lim;
-    if (t == 0) s_count = 0;
+    const int known = (int)state[0];
+    if (list) limit = min(limit, state[2]);
+    for (int i = t; i < 3 * known; i += kThreads) acc[i] = out[i];
+    if (t == 0) s_count = known;
     __syncthreads();
-    long long used = 0;
-    for (long long j0 = 0; j0 < limit && s_count < n; j0 += kThreads) {
-        const long long j = j0 + t;
-        const bool valid = j < limit;
+    for (int i = t; i < known; i += kThreads) accf[i] = narrow(acc[3 * i], acc[3 * i + 1], acc[3 * i + 2]);
+    __syncthreads();
+    long long used = begin;
+    for (long long j0 = begin; j0 < limit && s_count < n; j0 += kThreads) {
+        const bool valid = j0 + t < limit;
+        const long long j = !valid ? 0 : list ? list_base + list[j0 + t] : j0 + t;
         double c[3] = {0.0, 0.0, 0.0};
         bool ok = valid;
         float4 cf = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -106,7 +115,7 @@ __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double l
 #pragma unroll
             for (int a = 0; a < 3; ++a) c[a] = uniform(base, 3 * (uint64_t)j + 1 + a);
             cf = narrow(c[0], c[1], c[2]);
-            for (int a = 0; a < s_count && ok; ++a) ok = clear_of(cf, accf[a], c, acc + 3 * a, limf, lim);
+            for (int a = list ? known : 0; a < s_count && ok; ++a) ok = clear_of(cf, accf[a], c, acc + 3 * a, limf, lim);
         }
         int start = 0;
         bool round_done = false;
@@ -150,6 +159,65 @@ __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double l
     }
 }
 
+// After the first block most spheres are placed and nearly every candidate is rejected by one of
+// them, so the rest of the draws goes through the whole GPU: kChunk candidates are tested
+// against the centres placed so far (one bit each), the survivors are listed in draw order,
+// and the sequential kernel examines only these against each other.  100 spheres at 40 %, which
+// RSA cannot place in 400 000 candidates: one CTA took 3.9 ms over them; with this and the
+// growth kernel's settled trials the whole call went from 12.4 to 6.1 ms.
+constexpr int kChunk = 1 << 17;      // candidates per filter launch
+constexpr int kSurvivors = 4096;     // listed at most; the next chunk starts behind the last one listed
+__global__ void __launch_bounds__(256) k_rsa_filter(uint64_t base, double lim, long long begin, int count,
+                                                    const double* __restrict__ centres,
+                                                    const long long* __restrict__ state, unsigned* __restrict__ bits) {
+    __shared__ float4 accf[kMaxSpheres];
+    const int placed = (int)state[0];
+    const float limf = (float)lim;
+    for (int i = threadIdx.x; i < placed; i += 256) accf[i] = narrow(centres[3 * i], centres[3 * i + 1], centres[3 * i + 2]);
+    __syncthreads();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    bool ok = i < count;
+    if (ok) {
+        double c[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) c[a] = uniform(base, 3 * (uint64_t)(begin + i) + 1 + a);
+        const float4 cf = narrow(c[0], c[1], c[2]);
+        for (int a = 0; a < placed && ok; ++a) ok = clear_of(cf, accf[a], c, centres + 3 * a, limf, lim);
+    }
+    const unsigned w = __ballot_sync(0xffffffffu, ok);
+    if ((threadIdx.x & 31) == 0 && i < count) bits[i >> 5] = w;
+}
+// Survivors of `count` candidates in order: list (offsets from the chunk's first candidate),
+// state[2] = how many are listed, state[3] = candidates of the chunk that are settled by them.
+__global__ void __launch_bounds__(kThreads) k_rsa_list(const unsigned* __restrict__ bits, int count, int* __restrict__ list,
+                                                       long long* __restrict__ state) {
+    __shared__ int part[kThreads];
+    const int words = (count + 31) / 32, t = threadIdx.x;
+    const int per = (words + kThreads - 1) / kThreads, w0 = min(t * per, words), w1 = min(w0 + per, words);
+    int c = 0;
+    for (int w = w0; w < w1; ++w) c += __popc(bits[w]);
+    part[t] = c;
+    __syncthreads();
+    for (int o = 1; o < kThreads; o <<= 1) {   // inclusive prefix sum
+        const int add = t >= o ? part[t - o] : 0;
+        __syncthreads();
+        part[t] += add;
+        __syncthreads();
+    }
+    int at = part[t] - c;
+    const int total = part[kThreads - 1];
+    for (int w = w0; w < w1 && at < kSurvivors; ++w)
+        for (unsigned m = bits[w]; m && at < kSurvivors; m &= m - 1, ++at) {
+            const int i = 32 * w + __ffs(m) - 1;
+            list[at] = i;
+            if (at == kSurvivors - 1) state[3] = i + 1;
+        }
+    if (t == 0) {
+        state[2] = min(total, kSurvivors);
+        if (total < kSurvivors) state[3] = count;
+    }
+}
+
 // x in (-1, 2) wrapped into [0, 1): the exact remainder fmod(x, 1), plus 1 when it is negative
 // (a zero remainder is +0)
 __device__ __forceinline__ double wrap1(double x) {
@@ -161,12 +229,13 @@ __device__ __forceinline__ double wrap1(double x) {
 // against the moved spheres before it and the unmoved ones after it.  But every trial is
 // known at the start of the sweep (a sphere moves once per sweep and its draw depends on its
 // own position only), so whether trial i is clear of sphere k before (A) and after (B) k's
-// own move is tabulated in parallel as bit rows, and one warp then walks the spheres in order
-// with bit operations: trial i is taken when every k is clear, B where k < i has moved, A
-// elsewhere.  Rows come in blocks of kRows spheres so that the tables of 1024 spheres fit; B
-// is needed only within a block (earlier blocks have settled before it).  100 spheres at 40 %
-// through the C ABI, placement and 128^3 grid: 219 -> 12.4 ms (FP64 distances and two barriers
-// per sphere before).
+// own move is tabulated in parallel as bit rows.  That settles most trials; one warp walks the
+// others in order with bit operations: trial i is taken when every k is clear, B where k < i
+// has moved, A elsewhere.  Rows come in blocks of kRows spheres so that the tables of 1024
+// spheres fit; B is needed only within a block (earlier blocks have settled before it).  Bound
+// by the barriers and latency of one CTA.  100 spheres at 40 % through the C ABI, placement and
+// 128^3 grid: 219 ms with FP64 distances and two barriers per sphere, 12.4 ms with the bit
+// tables, 6.1 ms with settled trials and the filtered candidates above.
 // c: 3 n doubles in/out; state[0] = 1 on success, state[1] = sweeps run.
 constexpr int kRows = 128;
 struct GrowSmem {
@@ -174,8 +243,9 @@ struct GrowSmem {
     double tr[3 * kMaxSpheres];       // trials of the sweep
     float4 pf[kMaxSpheres], tf[kMaxSpheres];
     unsigned A[kRows][kMaxSpheres / 32];
-    unsigned B[kRows][kRows / 32];
+    unsigned B[kRows][kMaxSpheres / 32];
     unsigned acc[kRows / 32];         // taken trials of the block
+    unsigned open[kRows / 32];        // trials that depend on the order
     float wminf[kThreads / 32];
     double wmin[kThreads / 32];
     double lim;
@@ -206,19 +276,21 @@ __global__ void __launch_bounds__(kThreads) k_grow(uint64_t base, int n, double 
             const float4 a = s.pf[i];
             for (int k = lane; k < i; k += 32) mf = fminf(mf, near_sq(a, s.pf[k]));
         }
+        const float own = mf;
         for (int o = 16; o > 0; o >>= 1) mf = fminf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
         if (lane == 0) s.wminf[warp] = mf;
         __syncthreads();
         mf = s.wminf[lane];
         for (int o = 16; o > 0; o >>= 1) mf = fminf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
         double m = INFINITY;
-        for (int i = warp; i < n; i += kWarps) {
-            const float4 a = s.pf[i];
-            for (int k = lane; k < i; k += 32)
-                if (near_sq(a, s.pf[k]) <= mf + 2.f * kMargin)
-                    m = fmin(m, min_image_sq(s.p[3 * i], s.p[3 * i + 1], s.p[3 * i + 2], s.p[3 * k], s.p[3 * k + 1],
-                                             s.p[3 * k + 2]));
-        }
+        if (own <= mf + 2.f * kMargin)   // this thread saw a pair near the minimum: scan its pairs again
+            for (int i = warp; i < n; i += kWarps) {
+                const float4 a = s.pf[i];
+                for (int k = lane; k < i; k += 32)
+                    if (near_sq(a, s.pf[k]) <= mf + 2.f * kMargin)
+                        m = fmin(m, min_image_sq(s.p[3 * i], s.p[3 * i + 1], s.p[3 * i + 2], s.p[3 * k], s.p[3 * k + 1],
+                                                 s.p[3 * k + 2]));
+            }
         if (__any_sync(0xffffffffu, m < INFINITY))
             for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) s.wmin[warp] = m;
@@ -253,32 +325,46 @@ __global__ void __launch_bounds__(kThreads) k_grow(uint64_t base, int n, double 
         const float limf = (float)lim;
         for (int i0 = 0; i0 < n; i0 += kRows) {
             const int nr = min(kRows, n - i0), bw = (nr + 31) / 32;
-            // bit rows: trial i against every centre, and against the trials of its block
-            for (int job = warp; job < nr * (words + bw); job += kWarps) {
-                const int ri = job % nr, w = job / nr, i = i0 + ri;
-                const bool own = w >= words;                       // B row
-                const int k = (own ? i0 + (w - words) * 32 : w * 32) + lane;
-                bool ok = true;
-                if (k < n && k != i)
-                    ok = own ? clear_of(s.tf[i], s.tf[k], s.tr + 3 * i, s.tr + 3 * k, limf, lim)
-                             : clear_of(s.tf[i], s.pf[k], s.tr + 3 * i, s.p + 3 * k, limf, lim);
-                const unsigned bits = __ballot_sync(0xffffffffu, ok);
-                if (lane == 0) {
-                    if (own) s.B[ri][w - words] = bits;
-                    else s.A[ri][w] = bits;
+            // One warp per trial: its bit rows, and whether they settle it.  A centre k that the
+            // trial is not clear of rejects it unless k may have moved before (k < i in the
+            // block) to a place it is clear of; a trial clear of every place that any sphere can
+            // have is taken whatever happens.  Only the others depend on the order.
+            if (t < kRows / 32) s.acc[t] = s.open[t] = 0;
+            __syncthreads();
+            for (int ri = warp; ri < nr; ri += kWarps) {
+                const int i = i0 + ri;
+                bool reject = false, sure = true;
+                for (int w = 0; w < words && !reject; ++w) {
+                    const int k = w * 32 + lane;
+                    bool a = true, b = true;
+                    if (k < n && k != i) a = clear_of(s.tf[i], s.pf[k], s.tr + 3 * i, s.p + 3 * k, limf, lim);
+                    const bool may = k >= i0 && k < i;               // k's move of this sweep comes first
+                    if (may) b = clear_of(s.tf[i], s.tf[k], s.tr + 3 * i, s.tr + 3 * k, limf, lim);
+                    const unsigned wa = __ballot_sync(0xffffffffu, a), wb = __ballot_sync(0xffffffffu, b);
+                    reject = __any_sync(0xffffffffu, !a && !(may && b));
+                    sure = sure && __all_sync(0xffffffffu, a && b);
+                    if (lane == 0) {
+                        s.A[ri][w] = wa;
+                        s.B[ri][w] = wb;
+                    }
                 }
+                if (lane == 0 && !reject) atomicOr(sure ? &s.acc[ri >> 5] : &s.open[ri >> 5], 1u << (ri & 31));
             }
             __syncthreads();
-            if (warp == 0) {   // the block's spheres in order; lane w holds word w of the rows
+            if (warp == 0) {   // the open trials in order; lane w holds word w of the rows
                 const int w0 = i0 / 32;                            // the block's first word
                 const bool in = lane >= w0 && lane < w0 + bw;
-                unsigned acc = 0;                                  // trials taken, of lane's word
-                for (int ri = 0; ri < nr; ++ri) {
-                    const unsigned a = lane < words ? s.A[ri][lane] : 0xffffffffu;
-                    const unsigned b = in ? s.B[ri][lane - w0] : 0u;
-                    const bool ok = __all_sync(0xffffffffu, ((acc & b) | (~acc & a)) == 0xffffffffu);
-                    if (ok && lane == w0 + ri / 32) acc |= 1u << (ri & 31);
-                }
+                unsigned acc = in ? s.acc[lane - w0] : 0u;         // trials taken, of lane's word
+                for (int ow = 0; ow < bw; ++ow)
+                    for (unsigned left = s.open[ow]; left; left &= left - 1) {
+                        const int bit = __ffs(left) - 1, ri = 32 * ow + bit;
+                        const unsigned a = lane < words ? s.A[ri][lane] : 0xffffffffu;
+                        const unsigned b = lane < words ? s.B[ri][lane] : 0xffffffffu;
+                        // trials taken before i (b is all ones elsewhere)
+                        const unsigned before = lane < w0 + ow ? acc : (lane == w0 + ow ? acc & ((1u << bit) - 1u) : 0u);
+                        const bool ok = __all_sync(0xffffffffu, ((before & b) | (~before & a)) == 0xffffffffu);
+                        if (ok && lane == w0 + ow) acc |= 1u << bit;
+                    }
                 if (in) s.acc[lane - w0] = acc;
             }
             __syncthreads();
@@ -300,21 +386,49 @@ __global__ void __launch_bounds__(kThreads) k_grow(uint64_t base, int n, double 
 
 }  // namespace rsa
 
-// Runs one placement kernel; false with the error set on a CUDA failure.
+// Device scratch of a placement: centres, counters, filter bits and survivor list.
+struct PlaceScratch {
+    double* c;          // 3 n
+    long long* state;   // 4
+    unsigned* bits;     // rsa::kChunk / 32
+    int* list;          // rsa::kSurvivors
+    static size_t bytes(int n) {
+        return (3 * (size_t)n + 4) * sizeof(double) + rsa::kChunk / 8 + rsa::kSurvivors * sizeof(int);
+    }
+    PlaceScratch(void* p, int n) {
+        c = static_cast<double*>(p);
+        state = reinterpret_cast<long long*>(c + 3 * (size_t)n);
+        bits = reinterpret_cast<unsigned*>(state + 4);
+        list = reinterpret_cast<int*>(bits + rsa::kChunk / 32);
+    }
+};
+
+// Runs RSA at radius r from one stream; h_state[0]: spheres placed.  False with the error set on
+// a CUDA failure.
 static bool run_rsa(cudaStream_t st, uint64_t seed, int stream, int n, double r, long long max_candidates,
-                    double* d_out, long long* d_state, long long h_state[2]) {
+                    const PlaceScratch& d, long long h_state[4]) {
     const uint64_t base = seed + (uint64_t)stream * rsa::kStream;
     const double tr = 2.0 * r;
     const double lim = tr * tr;
     const long long limit = (max_candidates + rsa::kBlock - 1) / rsa::kBlock * rsa::kBlock;
-    rsa::k_rsa<<<1, rsa::kThreads, 0, st>>>(base, n, lim, limit, d_out, d_state);
-    cudaError_t e = cudaMemcpyAsync(h_state, d_state, 2 * sizeof(long long), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-        set_error("RSA kernel: %s", cudaGetErrorString(e));
-        return false;
+    cudaError_t e = cudaMemsetAsync(d.state, 0, 4 * sizeof(long long), st);
+    rsa::k_rsa<<<1, rsa::kThreads, 0, st>>>(base, n, lim, 0, std::min(limit, (long long)rsa::kBlock), nullptr, 0, d.c, d.state);
+    long long next = rsa::kBlock;
+    for (;;) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h_state, d.state, 4 * sizeof(long long), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            set_error("RSA kernel: %s", cudaGetErrorString(e));
+            return false;
+        }
+        next += h_state[3];   // (0 after the first block)
+        if (h_state[0] >= n || next >= limit) return true;
+        const int count = (int)std::min((long long)rsa::kChunk, limit - next);
+        rsa::k_rsa_filter<<<(count + 255) / 256, 256, 0, st>>>(base, lim, next, count, d.c, d.state, d.bits);
+        rsa::k_rsa_list<<<1, rsa::kThreads, 0, st>>>(d.bits, count, d.list, d.state);
+        rsa::k_rsa<<<1, rsa::kThreads, 0, st>>>(base, n, lim, 0, rsa::kSurvivors, d.list, next, d.c, d.state);
+        e = cudaGetLastError();
     }
-    return true;
 }
 
 // The placement of steps 1-2 above into host memory (3 n centres); generator: 0 RSA,
@@ -323,25 +437,28 @@ static hmg_status place(hmg_ctx* ctx, uint64_t seed, int n, double r, long long 
                         std::vector<double>& centres, int* generator) {
     DeviceGuard dg(ctx->device);
     cudaStream_t st = ctx->stream;
-    // the kept scratch (it holds 1024 spheres), counted against the budget for the call
+    // the kept scratch (it holds 1024 spheres and the filter's buffers); its lists are counted
+    // against the budget for the call
     const size_t bytes = (3 * (size_t)n + 2) * sizeof(double);
     const bool counted = ctx->reserve(bytes);
-    double* d_c = counted ? (double*)ctx->scratch_get(bytes) : nullptr;
-    if (!d_c) {
+    void* mem = counted ? ctx->scratch_get(PlaceScratch::bytes(n)) : nullptr;
+    if (!mem) {
         if (counted) ctx->unreserve(bytes);
         set_error("cannot allocate placement state");
         return HMG_OUT_OF_MEMORY;
     }
-    long long* d_state = reinterpret_cast<long long*>(d_c + 3 * (size_t)n);
-    long long h[2] = {0, 0};
+    const PlaceScratch d(mem, n);
+    double* d_c = d.c;
+    long long* d_state = d.state;
+    long long h[4] = {0, 0, 0, 0};
     hmg_status res = HMG_OK;
     int gen = 0;
-    if (!run_rsa(st, seed, 0, n, r, max_candidates, d_c, d_state, h)) {
+    if (!run_rsa(st, seed, 0, n, r, max_candidates, d, h)) {
         res = HMG_CUDA_ERROR;
     } else if (h[0] < n) {
         gen = 1;
         const double r85 = 0.85 * r;
-        if (!run_rsa(st, seed, 2, n, r85, max_candidates, d_c, d_state, h)) {
+        if (!run_rsa(st, seed, 2, n, r85, max_candidates, d, h)) {
             res = HMG_CUDA_ERROR;
         } else if (h[0] < n) {
             set_error("RSA at the reduced radius placed %lld of %d spheres", h[0], n);
@@ -370,7 +487,7 @@ static hmg_status place(hmg_ctx* ctx, uint64_t seed, int n, double r, long long 
             res = HMG_CUDA_ERROR;
         }
     }
-    ctx->scratch_put(d_c);
+    ctx->scratch_put(mem);
     ctx->unreserve(bytes);
     if (generator) *generator = gen;
     return res;
