@@ -858,7 +858,8 @@ def run_serve(args) -> None:
 
 # the sources of the sweep kernels (device code and the headers it includes); host-side
 # driver, engine and request-loop files do not change what a kernel moves
-KERNEL_SOURCES = ("hmg_fast.cu", "hmg_kernels.cu", "hmg_fused.cu", "hmg_internal.h")
+KERNEL_SOURCES = ("hmg_fast.cu", "hmg_kernels.cu", "hmg_fused.cu", "hmg_gen32.cu", "hmg_fixed_x.cu",
+                  "hmg_fixed_col.cu", "hmg_fixed_z.cu", "hmg_internal.h")
 
 
 def _kernel_sha() -> str:

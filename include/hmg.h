@@ -360,6 +360,7 @@ hmg_status hmg_poll(hmg_ctx* ctx, uint64_t ticket, double K_out[9], hmg_info* in
  *          (0, the default: the x inverse of one sweep and the x forward of the next
  *          are one kernel and the field is stored only before the residual sweep) or
  *          not (1).  Chained and unchained sweeps give bit-identical results.
+ *          (This bit also applies to the grid sizes without other variants.)
  *   bit 3: with chained sweeps, the x round trip runs as one launch per CTA of each
  *          row block (0) or as a persistent kernel (1) whose CTAs stage the spectrum
  *          and phase rows of their next row block in shared memory with bulk copies

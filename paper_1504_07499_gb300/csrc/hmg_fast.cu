@@ -14,7 +14,9 @@
 // Loads and stores go between HBM and registers with the pencil index fastest across
 // threads, so every warp access is a run of contiguous bytes.
 // Within a block of FP32 sweeps the x inverse of one sweep and the x forward of the next
-// are one kernel (k_fx_round); the y and z passes are the same in every sweep.
+// are one kernel (k_fx_round, k_px_round); the y and z passes are the same in every sweep.
+// The x passes of 64, 128, 192 and 256 take two real rows through one complex transform
+// (k_px_*); 96 and 512 a packed half-length transform per row (k_fx_*).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
