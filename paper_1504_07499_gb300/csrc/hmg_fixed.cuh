@@ -95,15 +95,23 @@ HMG_HD float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y 
 #endif
 HMG_HD float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }
 HMG_HD float2 swap_ri(float2 a) { return make_float2(a.y, a.x); }
-HMG_HD float mul_r2(float x) { return x * 0.70710678118654752f; }
-HMG_HD float mul_h3(float x) { return x * 0.86602540378443865f; }
+// Constants in two parts: rounded to FP32 they would scale every transform alike, and the error
+// of the six passes of a sweep would add up with one sign (relative gain of a radix-9 DFT
+// -1.6e-8 with rounded constants, below 1e-10 so; its rounding error 6.8e-8 and 6.3e-8).
+HMG_HD float mul_r2(float x) {
+    return fmaf(x, 0.70710678118654752f, x * (float)(0.70710678118654752 - 0.70710678118654752f));
+}
+HMG_HD float mul_h3(float x) {
+    return fmaf(x, 0.86602540378443865f, x * (float)(0.86602540378443865 - 0.86602540378443865f));
+}
 HMG_HD float half(float x) { return 0.5f * x; }
 template <long long C, bool CM, long long S, bool SM>
 HMG_HD float2 rot(float2 a) {
     constexpr double u = 1.0 / 18446744073709551616.0;   // 2^-64
-    constexpr float c = (float)(CM ? 1.0 - (double)C * u : (double)C * u);
-    constexpr float s = (float)(SM ? 1.0 - (double)S * u : (double)S * u);
-    return make_float2(c * a.x + s * a.y, c * a.y - s * a.x);
+    constexpr double cd = CM ? 1.0 - (double)C * u : (double)C * u, sd = SM ? 1.0 - (double)S * u : (double)S * u;
+    constexpr float c = (float)cd, cl = (float)(cd - c), s = (float)sd, sl = (float)(sd - s);
+    return make_float2(fmaf(c, a.x, fmaf(s, a.y, fmaf(cl, a.x, sl * a.y))),
+                       fmaf(c, a.y, -fmaf(s, a.x, fmaf(sl, a.x, -cl * a.y))));
 }
 template <class T>
 HMG_HD T neg(T a) { return mkc(-a.x, -a.y); }
