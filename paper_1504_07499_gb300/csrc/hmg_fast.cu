@@ -104,7 +104,7 @@ __device__ __forceinline__ void mode_parts(int kx, int ky, int kz, int N, int c,
 
 template <int L, int P, int MODE>
 __global__ void __launch_bounds__(P * Split<L>::TP, 3)
-k_fz3(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__ partial) {
+k_fz3(GridDesc g, unsigned mask, float2* spec, double* __restrict__ partial) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
     constexpr int NS = xslots<L>() * P;
     grid_begin();
@@ -291,7 +291,7 @@ k_fz3_p(const __grid_constant__ CUtensorMap zmap, GridDesc g, unsigned mask, flo
 // through shared memory (more threads, fewer registers per thread).
 template <int L, int P, int MODE>
 __global__ void __launch_bounds__(3 * P * Split<L>::TP, col_min_ctas<L, 2>())
-k_fzs(GridDesc g, unsigned mask, float2* __restrict__ spec, double* __restrict__ partial) {
+k_fzs(GridDesc g, unsigned mask, float2* spec, double* __restrict__ partial) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
     constexpr int NS = xslots<L>() * P;
     grid_begin();
@@ -423,7 +423,7 @@ __device__ __forceinline__ void stage_twiddles(float2* tws, const GridDesc& g) {
 // at v[i TP + m].  With KPT even, positions t KPT + i (i even) are 16-byte aligned pairs,
 // loaded and stored as float4 (and their phase ids as one uchar4).
 template <int M>
-__device__ __forceinline__ void s2_load(float2* v, const float2* __restrict__ row, int t) {
+__device__ __forceinline__ void s2_load(float2* v, const float2* row, int t) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, KPT = E / TP;
     if constexpr (KPT % 2 == 0) {
         const float4* r4 = reinterpret_cast<const float4*>(row);
@@ -462,7 +462,7 @@ __device__ __forceinline__ void s2_store(float2* __restrict__ row, const float2*
     }
 }
 template <int M>
-__device__ __forceinline__ void s2_load_phase(uchar2* q, const uchar2* __restrict__ row, int t) {
+__device__ __forceinline__ void s2_load_phase(uchar2* q, const uchar2* row, int t) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, KPT = E / TP;
     if constexpr (KPT % 2 == 0) {
         const uchar4* r4 = reinterpret_cast<const uchar4*>(row);
@@ -540,7 +540,7 @@ __device__ __forceinline__ void row_forward_split(float2* v, int t, float2* rs, 
 
 template <int M, int RW, int MODE>
 __global__ void __launch_bounds__(RW * Split<M>::TP, 1024 / (RW * Split<M>::TP))
-k_fx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* __restrict__ spec,
+k_fx_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ spec,
              double* __restrict__ partial) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
     __shared__ float2 tws[2 * M];
@@ -612,7 +612,7 @@ __device__ __forceinline__ void c2r_merge_shfl(float2* v, const float2* xk, cons
 // stage 1, exchange, stage 2; leaves v in the stage-2 layout (v[i TP + m] =
 // x[(t KPT + i) + E m]).  The caller has synchronized the CTA after staging twN / twM.
 template <int M, int TP, int E>
-__device__ __forceinline__ void row_inverse(float2* v, int t, float2* rs, const float2* __restrict__ src,
+__device__ __forceinline__ void row_inverse(float2* v, int t, float2* rs, const float2* src,
                                             const float2* __restrict__ twM, const float2* __restrict__ twN) {
     float2 xk[E];
 #pragma unroll
@@ -632,8 +632,8 @@ constexpr int fx_inverse_min_threads() {
 
 template <int M, int RW, int MODE>
 __global__ void __launch_bounds__(RW * Split<M>::TP, fx_inverse_min_threads<M, MODE>() / (RW * Split<M>::TP))
-k_fx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* __restrict__ tau,
-             const float* __restrict__ r32, double* __restrict__ partial) {
+k_fx_inverse(GridDesc g, unsigned mask, const float2* spec, float* __restrict__ tau,
+             const float* r32, double* __restrict__ partial) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
     __shared__ float2 tws[2 * M];
     stage_twiddles<M>(tws, g);
@@ -686,7 +686,7 @@ k_fx_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
 template <int M, int RW, bool ADDR, bool WTAU>
 __global__ void __launch_bounds__(RW * Split<M>::TP, 512 / (RW * Split<M>::TP))
 k_fx_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau,
-           const float* __restrict__ r32) {
+           const float* r32) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
     __shared__ float2 lut[16];
     __shared__ float2 tws[2 * M];
@@ -753,7 +753,7 @@ struct RoundSmem {
 template <int M, int RW, bool ADDR, bool WTAU>
 __global__ void __launch_bounds__(RW * Split<M>::TP, 512 / (RW * Split<M>::TP))
 k_fx_round_p(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau,
-             const float* __restrict__ r32, int nblk) {
+             const float* r32, int nblk) {
     constexpr int E = Split<M>::E, TP = Split<M>::TP, RS = row_stride<M>();
     using L = RoundSmem<M, RW>;
     constexpr int N = 2 * M;
@@ -893,7 +893,7 @@ __device__ __forceinline__ void pair_split(const float2* v, int t, float2* __res
 
 // The pair's values in the stage-2 layout: v[i TP + m] = (a, b) at p = t KPT + i + E m.
 template <int L>
-__device__ __forceinline__ void pair_load(float2* v, const float* __restrict__ ra, const float* __restrict__ rb, int t) {
+__device__ __forceinline__ void pair_load(float2* v, const float* ra, const float* rb, int t) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
 #pragma unroll
     for (int m = 0; m < TP; ++m) {
@@ -934,7 +934,7 @@ __device__ __forceinline__ void pair_store(float* __restrict__ ra, float* __rest
     }
 }
 template <int L>
-__device__ __forceinline__ void pair_load_phase(uchar2* q, const uint8_t* __restrict__ pa, const uint8_t* __restrict__ pb,
+__device__ __forceinline__ void pair_load_phase(uchar2* q, const uint8_t* pa, const uint8_t* pb,
                                                 int t) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP, KPT = E / TP;
 #pragma unroll
@@ -1035,7 +1035,7 @@ struct PairShape {
 
 template <int L, int MODE>
 __global__ void __launch_bounds__(128, 8)
-k_px_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* __restrict__ spec,
+k_px_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ spec,
              double* __restrict__ partial) {
     using S = PairShape<L>;
     constexpr int E = S::E, TP = S::TP, M = S::M;
@@ -1089,8 +1089,8 @@ constexpr int px_inverse_ctas() {
 
 template <int L, int MODE>
 __global__ void __launch_bounds__(128, px_inverse_ctas<L, MODE>())
-k_px_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* __restrict__ tau,
-             const float* __restrict__ r32, double* __restrict__ partial) {
+k_px_inverse(GridDesc g, unsigned mask, const float2* spec, float* __restrict__ tau,
+             const float* r32, double* __restrict__ partial) {
     using S = PairShape<L>;
     constexpr int E = S::E, TP = S::TP, M = S::M;
     __shared__ float2 tws[L];
@@ -1140,7 +1140,7 @@ k_px_inverse(GridDesc g, unsigned mask, const float2* __restrict__ spec, float* 
 // is compared with the stored one before it replaces it (sweeps that report every residual).
 template <int L, bool ADDR, bool WTAU, bool RES = false>
 __global__ void __launch_bounds__(128, 4)
-k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau, const float* __restrict__ r32,
+k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau, const float* r32,
            double* __restrict__ partial) {
     using S = PairShape<L>;
     constexpr int E = S::E, TP = S::TP, M = S::M;
@@ -1206,7 +1206,7 @@ struct PairSmem {
 template <int L, bool ADDR, bool WTAU>
 __global__ void __launch_bounds__(128, 4)
 k_px_round_p(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restrict__ tau,
-             const float* __restrict__ r32, int nblk) {
+             const float* r32, int nblk) {
     using S = PairShape<L>;
     using D = PairSmem<L>;
     constexpr int E = S::E, TP = S::TP, M = S::M, RW = S::RW;
@@ -1342,7 +1342,7 @@ __device__ __forceinline__ void y_columns(const GridDesc& g, float2* base, int t
 
 template <int L, bool ADDR, bool WTAU>
 __global__ void __launch_bounds__(256, 2)
-k_yxy(GridDesc g, unsigned mask, float2* spec, float* __restrict__ tau, const float* __restrict__ r32, int nper) {
+k_yxy(GridDesc g, unsigned mask, float2* spec, float* __restrict__ tau, const float* r32, int nper) {
     using S = YxyShape<L>;
     constexpr int M = S::M, P = S::P, RW = S::RW;
     constexpr int N = L;

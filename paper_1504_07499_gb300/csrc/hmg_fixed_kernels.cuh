@@ -132,7 +132,7 @@ __device__ __forceinline__ bool load_merge(const GridDesc& g, c64 (&v)[Plan<M>::
 #pragma unroll
             for (int q = 0; q < P::R0; ++q) {
                 v[it][q] = src[j + q * J];
-                mk = max(mk, __ldg(&ein[j + q * J]) + bits_of(mag(v[it][q])));
+                mk = max(mk, ein[j + q * J] + bits_of(mag(v[it][q])));
             }
         }
     }
@@ -148,8 +148,8 @@ __device__ __forceinline__ bool load_merge(const GridDesc& g, c64 (&v)[Plan<M>::
 #pragma unroll
             for (int q = 0; q < P::R0; ++q) {
                 const int k = j + q * J, km = k ? M - k : 0;
-                c64 a = shift(v[it][q], __ldg(&ein[k]) - e);
-                c64 b = shift(src[km], __ldg(&ein[km]) - e);
+                c64 a = shift(v[it][q], ein[k] - e);
+                c64 b = shift(src[km], ein[km] - e);
                 if (k == 0) {   // packed X(0) + i X(N/2)
                     b = mkc(a.y, 0);
                     a = mkc(a.x, 0);
@@ -166,7 +166,7 @@ __device__ __forceinline__ bool load_merge(const GridDesc& g, c64 (&v)[Plan<M>::
 
 template <int M>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
-k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ tau, c64* __restrict__ spec,
+k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* tau, c64* __restrict__ spec,
               double* __restrict__ partial) {
     using X = XShape<M>;
     using P = Plan<M>;
@@ -239,7 +239,7 @@ k_fxx_forward(GridDesc g, unsigned mask, int mode, const double* __restrict__ ta
 // ---------------------------------------------------------------------------
 template <int M>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas(XShape<M>::T, 896))
-k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* __restrict__ spec, double* __restrict__ tau,
+k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* spec, double* __restrict__ tau,
               float* __restrict__ d32, float* __restrict__ r32, double* __restrict__ partial) {
     using X = XShape<M>;
     using P = Plan<M>;
@@ -436,7 +436,7 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
                 if (a.fp64_in)
                     mk = max(mk, max(key_of(__longlong_as_double(v[it][q].x)), key_of(__longlong_as_double(v[it][q].y))));
                 else
-                    mk = max(mk, __ldg(&ein[i * estep]) + bits_of(mag(v[it][q])));
+                    mk = max(mk, ein[i * estep] + bits_of(mag(v[it][q])));
             }
         }
     }
@@ -452,7 +452,7 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
             for (int q = 0; q < P::R0; ++q) {
                 c64 z = v[it][q];
                 if (a.fp64_in) z = mkc(to_fixed(__longlong_as_double(z.x), e), to_fixed(__longlong_as_double(z.y), e));
-                else z = shift(z, __ldg(&ein[(j + q * J) * estep]) - e);
+                else z = shift(z, ein[(j + q * J) * estep] - e);
                 v[it][q] = a.inverse ? swap_ri(z) : z;
             }
         }
@@ -543,7 +543,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
 #pragma unroll
                 for (int q = 0; q < P::R0; ++q) {
                     v[it][q] = base[(j + q * J) * step];
-                    mk = max(mk, __ldg(&ein[(j + q * J) * M]) + bits_of(mag(v[it][q])));
+                    mk = max(mk, ein[(j + q * J) * M] + bits_of(mag(v[it][q])));
                 }
             }
         }
@@ -555,7 +555,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
             const int j = t + it * TPP;
             if (J % TPP == 0 || j < J) {
 #pragma unroll
-                for (int q = 0; q < P::R0; ++q) v[it][q] = shift(v[it][q], __ldg(&ein[(j + q * J) * M]) - e);
+                for (int q = 0; q < P::R0; ++q) v[it][q] = shift(v[it][q], ein[(j + q * J) * M] - e);
             }
         }
         transform<L, S>(v, o, t, cp, sm, orm, P3, e, g.twf);

@@ -255,7 +255,7 @@ __device__ __forceinline__ double widen(float f) {
 
 template <int M, int MODE>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas<M>(XShape<M>::T))
-k_gx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* __restrict__ spec,
+k_gx_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ spec,
              double* __restrict__ partial) {
     using X = XShape<M>;
     using P = Plan<M>;
@@ -293,8 +293,8 @@ k_gx_forward(GridDesc g, unsigned mask, const float* __restrict__ tau, float2* _
 
 template <int M, bool RES>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas<M>(XShape<M>::T))
-k_gx_inverse(GridDesc g, unsigned mask, int mode, const float2* __restrict__ spec, float* __restrict__ tau,
-             const float* __restrict__ r32, double* __restrict__ partial) {
+k_gx_inverse(GridDesc g, unsigned mask, int mode, const float2* spec, float* __restrict__ tau,
+             const float* r32, double* __restrict__ partial) {
     using X = XShape<M>;
     using P = Plan<M>;
     constexpr int N = X::N, RW = X::RW, T = X::T;
@@ -344,7 +344,7 @@ k_gx_inverse(GridDesc g, unsigned mask, int mode, const float2* __restrict__ spe
 template <int M>
 __global__ void __launch_bounds__(XShape<M>::T, min_ctas<M>(XShape<M>::T))
 k_gx_round(GridDesc g, unsigned mask, int add, int wtau, float2* __restrict__ spec, float* __restrict__ tau,
-           const float* __restrict__ r32) {
+           const float* r32) {
     using X = XShape<M>;
     using P = Plan<M>;
     using S = typename X::S;

@@ -57,7 +57,7 @@ __device__ double block_sum(double v, double* sh) {
 // cleared once the sum is below stop.least or not finite, and a slot that has stopped writes -1.
 template <int T>
 __global__ void __launch_bounds__(T)
-k_reduce(const double* __restrict__ partial, int count, int groups, double* __restrict__ out, StopRule stop) {
+k_reduce(const double* partial, int count, int groups, double* __restrict__ out, StopRule stop) {
     __shared__ double red[T];
     grid_begin();
     const int slot = blockIdx.x / groups, grp = blockIdx.x % groups;

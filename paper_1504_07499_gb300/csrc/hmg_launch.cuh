@@ -9,7 +9,10 @@
 // still holds it with a smaller split between cache and shared memory.
 // Every kernel launched this way calls grid_begin() in every thread before it touches memory
 // that another kernel writes (and before any early exit, so that a kernel never finishes
-// ahead of its predecessors); tables that no kernel writes may be read earlier.
+// ahead of its predecessors); tables that no kernel writes may be read earlier.  Its lifetime begins
+// while the kernel before still writes, and the read-only path (__ldg, or a restrict pointer that
+// the kernel only reads) is defined only for data that nothing writes in that time: what another
+// kernel writes is read through plain pointers, only the tables by __ldg.
 #pragma once
 
 #include <cuda_runtime.h>
