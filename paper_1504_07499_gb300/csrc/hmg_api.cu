@@ -725,7 +725,6 @@ bool Solver::check_eq(unsigned mask, const R* field, void* spec, double eps_eq[3
 // number), and the sweeps behind it skip that gradient.  Every gradient goes through the
 // sequence of sweeps and tests that one look per sweep would give.
 hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9]) {
-    if (!s->pinned()) return HMG_OUT_OF_MEMORY;
     host = s->pin;
     const unsigned all = (1u << g.nslots) - 1u;
     HMG_TRACED(HMG_K_OTHER, 0.0, launch_init_tau<double>(g, all, s->tau64, st));
@@ -841,7 +840,6 @@ hmg_status Solver::run_bulk(int max_iter, double tol, hmg_info* info, double K[9
             if (state[sl] == ph) m |= 1u << sl;
         return m;
     };
-    if (!s->pinned()) return HMG_OUT_OF_MEMORY;
     host = s->pin;
     Solver s64{g, s, st64, tr, s->partial3, s->partial3, s->pin};
     cudaEvent_t ready;

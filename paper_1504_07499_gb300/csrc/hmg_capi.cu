@@ -397,6 +397,7 @@ hmg_status solve_impl(hmg_ctx* ctx, const uint8_t* phase, int N, double km, doub
     GridDesc g;
     st = prepare(ctx, phase, N, k, fp64, 3, &g, scheme, beta);
     if (st != HMG_OK) return st;
+    if (!ctx->solve.pinned()) return HMG_OUT_OF_MEMORY;   // before any output is written
     Solver sv{g, &ctx->solve, ctx->stream, ctx->tracer.on ? &ctx->tracer : nullptr};
     hmg_info local;
     memset(&local, 0, sizeof(local));

@@ -69,7 +69,7 @@ struct SolveState {
                              // [64,96): its sweep sums
     double* pin = nullptr;   // pinned host memory in the layout of red, written by the reductions of
                              // a solve (no copy between a block and the host's look at it), and room
-                             // for flags; made by the first solve
+                             // for flags; made by pinned() before a solve's driver runs
     bool pinned();
     bool ensure(::hmg_ctx* c, int N, bool fp64, int nslots);
     void free_all(::hmg_ctx* c);
