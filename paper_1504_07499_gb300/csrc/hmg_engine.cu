@@ -11,11 +11,6 @@ namespace hmg {
 
 namespace {
 enum { PH_A = 0, PH_OUTER = 1, PH_EQ = 2, PH_INNER = 3, PH_DONE = 4 };
-// RVEs advanced at once within a tick.  Three fill the GPU with small grids and keep each one's
-// fields in L2 through its block of four sweeps; more evict each other (ms per batch at 1, 2, 3, 4,
-// 8, 16 streams: 5 x 64^3 + 4 x 96^3 + 3 x 128^3 418, 392, 390, 404, 419, 443; 12 x 64^3 157, 117, 109,
-// 109, 114, 129).
-constexpr int kSideStreams = 3;
 constexpr double kEta = 1e-4;       // correction sweeps reduce the FP64 residual by this factor
 constexpr int kStall = 24;          // sweeps without a new best FP32 residual = FP32 floor
 
@@ -26,13 +21,9 @@ hmg_status cerr(cudaError_t e, const char* what) {
 }
 }  // namespace
 
-Engine::Engine(hmg_ctx* c, cudaStream_t s, cudaStream_t s64, bool graph, int priority)
-    : ctx(c), st(s), st64(s64), use_graph(graph) {
+Engine::Engine(hmg_ctx* c, cudaStream_t s, cudaStream_t s64, bool graph, int prio)
+    : ctx(c), st(s), st64(s64), use_graph(graph), priority(prio) {
     cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
-    for (int i = 0; i < kSideStreams; ++i) {
-        cudaStream_t x;
-        if (cudaStreamCreateWithPriority(&x, cudaStreamNonBlocking, priority) == cudaSuccess) side.push_back(x);
-    }
 }
 
 Engine::~Engine() {
@@ -199,24 +190,41 @@ hmg_status Engine::capture() {
         cudaGraphExecDestroy(exec);
         exec = nullptr;
     }
+    size_t live = 0, bytes = 0;
+    for (const auto& up : entries)
+        if (!up->finished) {
+            ++live;
+            bytes += 2 * sizeof(float) * 9 * (size_t)up->g.N3;   // field and spectrum, three gradients
+        }
+    const size_t branches = side_branches(live, bytes);
+    while (side.size() < branches) {
+        cudaStream_t x;
+        if (cudaStreamCreateWithPriority(&x, cudaStreamNonBlocking, priority) != cudaSuccess) {
+            if (side.empty()) return cerr(cudaGetLastError(), "engine streams");
+            cudaGetLastError();
+            break;
+        }
+        side.push_back(x);
+    }
+    const size_t nb = std::min(branches, side.size());
     cudaEvent_t fork;
     if (cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) != cudaSuccess) return cerr(cudaGetLastError(), "event");
-    std::vector<cudaEvent_t> joins(side.size());
+    std::vector<cudaEvent_t> joins(nb);
     for (auto& j : joins) cudaEventCreateWithFlags(&j, cudaEventDisableTiming);
     cudaGraph_t graph = nullptr;
     cudaError_t ce = cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed);
     if (ce == cudaSuccess) {
         cudaEventRecord(fork, st);
-        std::vector<bool> used(side.size(), false);
+        std::vector<bool> used(nb, false);
         for (auto& up : entries) {
-            const size_t k = up->index % side.size();
+            const size_t k = up->index % nb;
             if (!used[k]) {
                 cudaStreamWaitEvent(side[k], fork, 0);
                 used[k] = true;
             }
             block_launches(up.get(), dflags, side[k]);
         }
-        for (size_t k = 0; k < side.size(); ++k)
+        for (size_t k = 0; k < nb; ++k)
             if (used[k]) {
                 cudaEventRecord(joins[k], side[k]);
                 cudaStreamWaitEvent(st, joins[k], 0);

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/hmg.h"
+#include "hmg_branches.h"
 #include "hmg_internal.h"
 #include "hmg_runtime.h"
 
@@ -83,8 +84,9 @@ class Engine {
     cudaStream_t st64;     // FP64 work, overlapped with the FP32 block
     cudaEvent_t ready;
     bool use_graph;
+    int priority;
     std::vector<std::unique_ptr<Entry>> entries;
-    std::vector<cudaStream_t> side;
+    std::vector<cudaStream_t> side;   // made as branches need them
     int* dflags = nullptr;      // 4 ints per entry
     int* hflags = nullptr;      // pinned
     double* hred = nullptr;     // pinned, 64 doubles per entry (the entry's residual sums)
