@@ -16,12 +16,12 @@ from paper_1504_07499_gb300 import build, hmg, inputs as I
 WRAP = r"""
 #include <stddef.h>
 int wrap_fail, wrap_made, wrap_freed;
-int __real_cudaMallocHost(void** p, size_t n);
+int __real_cudaHostAlloc(void** p, size_t n, unsigned flags);   /* what C++'s cudaMallocHost calls */
 int __real_cudaFreeHost(void* p);
-int __wrap_cudaMallocHost(void** p, size_t n) {
+int __wrap_cudaHostAlloc(void** p, size_t n, unsigned flags) {
     if (wrap_fail) return 2;   /* cudaErrorMemoryAllocation */
     ++wrap_made;
-    return __real_cudaMallocHost(p, n);
+    return __real_cudaHostAlloc(p, n, flags);
 }
 int __wrap_cudaFreeHost(void* p) {
     ++wrap_freed;
@@ -42,7 +42,7 @@ def wrapped(tmp_path_factory):
     subprocess.run(["gcc", "-c", "-fPIC", str(d / "wrap.c"), "-o", str(d / "wrap.o")], check=True)
     so = str(d / "libhmg_wrapped.so")
     subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-o", so, *objs, str(d / "wrap.o"), "-lcudart",
-                    "-Xlinker", "--wrap=cudaMallocHost", "-Xlinker", "--wrap=cudaFreeHost"], check=True)
+                    "-Xlinker", "--wrap=cudaHostAlloc", "-Xlinker", "--wrap=cudaFreeHost"], check=True)
     return so
 
 
