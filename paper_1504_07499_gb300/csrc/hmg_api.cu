@@ -431,9 +431,12 @@ void SolveState::free_all(Context* c) {
         c->release(*p);
         *p = nullptr;
     }
+    N = 0;
+}
+
+void SolveState::free_pinned() {
     if (pin) cudaFreeHost(pin);
     pin = nullptr;
-    N = 0;
 }
 
 bool SolveState::pinned() {

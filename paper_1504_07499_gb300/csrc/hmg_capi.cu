@@ -150,6 +150,7 @@ hmg_status hmg_destroy(hmg_ctx* ctx) {
         }
         cudaStreamSynchronize(ctx->stream);
         ctx->solve.free_all(ctx);
+        ctx->solve.free_pinned();
         if (ctx->scratch) cudaFree(ctx->scratch);
         ctx->plans.clear();
         cudaStreamSynchronize(ctx->stream64);

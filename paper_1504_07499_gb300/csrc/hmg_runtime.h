@@ -69,8 +69,10 @@ struct SolveState {
                              // [64,96): its sweep sums
     double* pin = nullptr;   // pinned host memory in the layout of red, written by the reductions of
                              // a solve (no copy between a block and the host's look at it), and room
-                             // for flags; made by pinned() before a solve's driver runs
+                             // for flags; made by pinned() before a solve's driver runs and kept over
+                             // changes of the grid size (its own does not depend on it)
     bool pinned();
+    void free_pinned();
     bool ensure(::hmg_ctx* c, int N, bool fp64, int nslots);
     void free_all(::hmg_ctx* c);
 };

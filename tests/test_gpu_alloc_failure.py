@@ -71,3 +71,14 @@ def test_no_pinned_memory_is_an_error_and_writes_nothing(lib, prec):
         assert (e == 7.0).all() and (K == 7.0).all() and info.status[0] == 7
         ok, _, _ = hmg.hmg_solve_fields(ctx.handle, ph, N, (0.2, 0.25, 2.0), 1e-8, prec, e)   # and the context goes on
     assert np.isfinite(ok).all() and not (e == 7.0).any()
+
+
+def test_pinned_memory_is_made_once_per_context(lib):
+    made, freed = lib("wrap_made"), lib("wrap_freed")
+    m0, f0 = made.value, freed.value
+    with hmg.Context(0) as ctx:
+        for N in (16, 24, 16, 32):
+            for prec in (hmg.HMG_FP64, hmg.HMG_FP32_BULK):
+                hmg.hmg_solve(ctx.handle, I.random_phase_grid(1, N), N, (0.2, 0.25, 2.0), 1e-6, prec)
+        assert (made.value - m0, freed.value - f0) == (1, 0)
+    assert (made.value - m0, freed.value - f0) == (1, 1)
