@@ -1061,7 +1061,7 @@ k_px_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ s
     __syncthreads();
     float2 v[E];
     pair_load<L>(v, src, src + L, t);
-    float acc = 0.f;
+    float2 acc = make_float2(0.f, 0.f);   // one sum per row of the pair
     if (MODE != XF_PLAIN) {
         uchar2 q[E];
         const uint8_t* ph = g.phase + (row % g.NN) * L;
@@ -1070,11 +1070,11 @@ k_px_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ s
         for (int j = 0; j < E; ++j) {
             // rounded products (never contracted into the transform's adds), as in the round trip
             v[j] = __fmul2_rn(v[j], lut[pair_index(q[j])]);
-            if (MODE == XF_FLUX) acc += v[j].x + v[j].y;
+            if (MODE == XF_FLUX) acc = cadd(acc, v[j]);
         }
     }
     if (MODE == XF_FLUX) {
-        const double s = block_sum_d((double)acc, red);
+        const double s = block_sum_d((double)acc.x + (double)acc.y, red);
         if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + pidx] = s;
     }
     float2* dst = spec + (long long)slot * 3 * g.NNM + row * M;
@@ -1117,7 +1117,7 @@ k_px_inverse(GridDesc g, unsigned mask, const float2* spec, float* __restrict__ 
     float2 v[E];
     const float2* src = spec + (long long)slot * 3 * g.NNM + row * M;
     pair_inverse<L>(v, t, sh + r * S::RS, src, src + M, PairTwSmem<L>{tws});
-    float acc = 0.f;
+    float2 acc = make_float2(0.f, 0.f);   // one sum per row of the pair
     const float wn = (float)(1.0 - g.relax), wo = (float)g.relax;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
@@ -1125,12 +1125,13 @@ k_px_inverse(GridDesc g, unsigned mask, const float2* spec, float* __restrict__ 
         if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
         if (res) {
             const float da = v[j].x - old[j].x, db = v[j].y - old[j].y;
-            acc += da * da + db * db;
+            acc.x += da * da;
+            acc.y += db * db;
         }
     }
     pair_store<L>(out, out + L, v, t);
     if (kRes) {   // uniform across the CTA (kernel argument and per-slot flag)
-        const double s = block_sum_d((double)acc, red);
+        const double s = block_sum_d((double)acc.x + (double)acc.y, red);
         if (threadIdx.x == 0 && res) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
     }
 }
@@ -1169,13 +1170,14 @@ k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     __syncthreads();   // tables and coefficient pairs
     float2 v[E];
     pair_inverse<L>(v, t, rs, sp, sp + M, PairTwSmem<L>{tws});
-    float acc = 0.f;
+    float2 acc = make_float2(0.f, 0.f);   // one sum per row of the pair
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         if (addr) v[j] = make_float2(__fadd_rn(v[j].x, radd[j].x), __fadd_rn(v[j].y, radd[j].y));
         if (RES) {
             const float da = v[j].x - radd[j].x, db = v[j].y - radd[j].y;
-            acc += da * da + db * db;
+            acc.x += da * da;
+            acc.y += db * db;
         }
     }
     if (WTAU) pair_store<L>(tau + fbase, tau + fbase + L, v, t);
@@ -1185,7 +1187,7 @@ k_px_round(GridDesc g, unsigned mask, float2* __restrict__ spec, float* __restri
     pair_forward<L>(v, t, rs, PairTwSmem<L>{tws}, sp, sp + M);
     if (RES) {   // partials in the order of k_px_inverse
         __shared__ double red[128];
-        const double s = block_sum_d((double)acc, red);
+        const double s = block_sum_d((double)acc.x + (double)acc.y, red);
         if (threadIdx.x == 0)
             partial[(long long)slot * gridDim.x + (blockIdx.x % 3) * (g.NN / S::RW) + blockIdx.x / 3] = s;
     }
