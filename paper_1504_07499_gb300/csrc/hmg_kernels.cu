@@ -100,22 +100,33 @@ __global__ void k_e_to_tau(GridDesc g, int slot, const double* __restrict__ e, R
 }
 
 // e = tau / (k + k0).  The three divisors are known, so each quotient is a product with the
-// rounded reciprocal corrected by one residual step (Brisebarre, Muller & Raina, "Accelerating
-// correctly rounded floating-point division when the divisor is known in advance", 2004):
-// three FP64 operations instead of a divide's ten or so, which bound this kernel.
+// reciprocal in two parts (Brisebarre, Muller & Raina, "Accelerating correctly rounded
+// floating-point division when the divisor is known in advance", 2004), which is within one unit
+// in the last place, and one residual step with the rounded reciprocal, which then rounds
+// correctly for every divisor (Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", 1990): four FP64 operations instead of a divide's ten or so, which bound
+// this kernel.  Operands whose residual could leave the normal range are divided.
 template <typename R>
 __global__ void k_tau_to_e(GridDesc g, int slot, const R* __restrict__ tau, double* __restrict__ e) {
-    const double rc[3] = {1.0 / g.KP[0], 1.0 / g.KP[1], 1.0 / g.KP[2]};
+    double rc[3], rl[3];   // 1 / KP = rc + rl
+    for (int p = 0; p < 3; ++p) {
+        rc[p] = 1.0 / g.KP[p];
+        rl[p] = fma(-rc[p], g.KP[p], 1.0) * rc[p];
+    }
+    auto in_range = [](double d) {   // 2^-823 <= |d| < 2^777, without the FP64 pipe
+        return ((unsigned)__double2hiint(d) >> 20 & 0x7ffu) - 200u < 1600u;
+    };
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N3; i += (long long)gridDim.x * blockDim.x) {
         const int ph = g.phase[i];
         const double kp = ph == 0 ? g.KP[0] : (ph == 1 ? g.KP[1] : g.KP[2]);
         const double r = ph == 0 ? rc[0] : (ph == 1 ? rc[1] : rc[2]);
+        const double l = ph == 0 ? rl[0] : (ph == 1 ? rl[1] : rl[2]);
         for (int c = 0; c < 3; ++c) {
             const double t = (double)tau[((long long)slot * 3 + c) * g.N3 + i];
-            const double q = t * r;
-            const double rem = fma(-q, kp, t);
-            // (an infinite or overflowing quotient has no residual)
-            e[c * g.N3 + i] = isfinite(rem) ? fma(rem, r, q) : t / kp;
+            const double q = fma(t, r, t * l);
+            double v = fma(fma(-q, kp, t), r, q);
+            if (!(in_range(t) && in_range(q))) v = t == 0.0 ? t : t / kp;
+            e[c * g.N3 + i] = v;
         }
     }
 }
