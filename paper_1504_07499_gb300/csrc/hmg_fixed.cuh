@@ -16,12 +16,15 @@
 //
 // Between passes the spectrum stays in integers, with the exponent of the pencil that wrote
 // each value in a side array, so only the field side of the x passes converts to and from
-// FP64.  Zero pencils carry a very small exponent, pencils with an infinity or a NaN a very
-// large one that marks everything computed from them as NaN.
+// FP64.  Zeros and subnormals count as 2^-1021 when a pencil's scale is chosen, so subnormals keep
+// their bits and zero pencils get a quantum below every double; pencils with an infinity or a NaN
+// carry a very large exponent that marks everything computed from them as NaN.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "hmg_internal.h"
 
@@ -32,7 +35,7 @@ struct __align__(16) c64 {
     long long x, y;
 };
 
-constexpr int kExpZero = -(1 << 20);   // exponent of a pencil that is zero
+constexpr int kExpZero = -(1 << 20);   // below every key: where a maximum starts
 constexpr int kExpNan = 1 << 20;       // exponent of a pencil that holds an infinity or a NaN
 #define HMG_HD __host__ __device__ __forceinline__
 
@@ -184,23 +187,30 @@ HMG_HD double bitsd(unsigned long long u) {
     return d;
 #endif
 }
-// smallest E with |d| < 2^E (subnormals count as zero)
+// E with |d| < 2^E, the smallest for normal numbers; zeros and subnormals share -1021
 HMG_HD int key_of(double d) {
-    const int ex = (int)((dbits(d) >> 52) & 0x7ff);
-    return ex == 0 ? kExpZero : ex == 2047 ? kExpNan : ex - 1022;
+    const unsigned long long u = dbits(d);
+    const int ex = (int)((u >> 52) & 0x7ff);
+    return ex == 2047 ? kExpNan : (ex ? ex : 1) - 1022;
 }
 // round(d 2^-e) for |d| < 2^(e + 61)
 HMG_HD long long to_fixed(double d, int e) {
     const unsigned long long u = dbits(d);
     const int ex = (int)((u >> 52) & 0x7ff);
-    const unsigned long long m = ex ? ((u << 10) & 0x3ffffffffffffc00ull) | (1ull << 62) : 0ull;   // 1.f at bit 62
-    int r = e + 1084 - ex;                     // one less than the right shift
+    // 1.f (0.f) at bit 62
+    const unsigned long long m = ((u << 10) & 0x3ffffffffffffc00ull) | ((unsigned long long)(ex ? 1u << 30 : 0u) << 32);
+    int r = e + 1084 - (ex ? ex : 1);          // one less than the right shift
     r = r < 0 ? 0 : (r > 63 ? 63 : r);
     const long long v = (long long)(((m >> r) + 1) >> 1);
     const long long s = (long long)u >> 63;
     return (v ^ s) - s;
 }
+// Values of a pencil with quantum 2^e may be subnormal where is_low(e).  LOW: with subnormals, else they
+// count as zero.  (A template parameter and a branch per pencil: tested per value they cost
+// every pass, a sweep at 256^3 10 %.)
+HMG_HD bool is_low(int e) { return e < -1022; }
 // v 2^e as a double, rounded to nearest
+template <bool LOW = false>
 HMG_HD double from_fixed(long long v, int e) {
     const long long s = v >> 63;
     const unsigned long long a = (unsigned long long)((v ^ s) - s);
@@ -209,9 +219,13 @@ HMG_HD double from_fixed(long long v, int e) {
     const int ex = e + 1085 - lz;              // biased exponent, less one (the leading bit adds it)
     unsigned long long b = (n >> 11) + ((n >> 10) & 1) + ((unsigned long long)(unsigned)ex << 52);
     if (ex >= 2046) b = 0x7ff0000000000000ull;
-    if (ex < 0 || a == 0) b = 0;
+    if (ex < 0 || a == 0) b = LOW ? (unsigned long long)shift((long long)a, e + 1074) : 0;
     return bitsd(b | ((unsigned long long)s & 0x8000000000000000ull));
 }
+template <bool LOW = false>
+HMG_HD double2 from_fixed(c64 v, int e) { return make_double2(from_fixed<LOW>(v.x, e), from_fixed<LOW>(v.y, e)); }
+using Low = std::true_type;
+using NotLow = std::false_type;
 
 // ---------------------------------------------------------------------------
 // forward DFTs of small length in registers, natural order in and out

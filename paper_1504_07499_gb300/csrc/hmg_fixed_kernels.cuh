@@ -265,6 +265,7 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* spec, double* __re
     const bool bad = load_merge<M>(g, v, t, r, row, spec + row * M, key, e);
     c64 o[P::IL][P::RL];
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
+    if (mode != XI_PLAIN) e -= g.sn;
     // output step in FP64
     double2* out = reinterpret_cast<double2*>(tau) + row * M;
     float2* dout = reinterpret_cast<float2*>(d32) + row * M;
@@ -272,23 +273,27 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* spec, double* __re
     const bool relax = g.relax != 0.0, res = mode == XI_INPLACE_RES || mode == XI_DIFF;
     const double wn = 1.0 - g.relax, wo = g.relax;
     double acc = 0.0;
-    last_emit<M>(o, t, [&](int k, c64 z) {
-        double2 n = make_double2(from_fixed(z.y, e), from_fixed(z.x, e));
-        if (bad) n = make_double2(nan(""), nan(""));
-        double2 old = make_double2(0.0, 0.0);
-        if (res || relax) old = out[k];
-        if (relax) n = make_double2(wn * n.x + wo * old.x, wn * n.y + wo * old.y);
-        if (res) {
-            const double da = n.x - old.x, db = n.y - old.y;
-            acc += da * da + db * db;
-            if (mode == XI_DIFF) {
-                const float2 f = make_float2((float)da, (float)db);
-                dout[k] = f;
-                rout[k] = f;
+    auto emit = [&](auto low) {
+        last_emit<M>(o, t, [&](int k, c64 z) {
+            double2 n = from_fixed<low>(swap_ri(z), e);
+            if (bad) n = make_double2(nan(""), nan(""));
+            double2 old = make_double2(0.0, 0.0);
+            if (res || relax) old = out[k];
+            if (relax) n = make_double2(wn * n.x + wo * old.x, wn * n.y + wo * old.y);
+            if (res) {
+                const double da = n.x - old.x, db = n.y - old.y;
+                acc += da * da + db * db;
+                if (mode == XI_DIFF) {
+                    const float2 f = make_float2((float)da, (float)db);
+                    dout[k] = f;
+                    rout[k] = f;
+                }
             }
-        }
-        if (mode != XI_DIFF) out[k] = n;
-    });
+            if (mode != XI_DIFF) out[k] = n;
+        });
+    };
+    if (is_low(e)) emit(Low());
+    else emit(NotLow());
     if (res) {
         const double s = cta_sum<T>(acc, red);
         if (threadIdx.x == 0) partial[(long long)slot * gridDim.x + blockIdx.x] = s;
@@ -327,6 +332,7 @@ k_fxx_round(GridDesc g, unsigned mask, c64* spec, double* __restrict__ tau, doub
     int e;
     const bool bad = load_merge<M>(g, v, t, r, row, sp, key, e);
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
+    e -= g.sn;
     if (P::NS > 1) __syncthreads();   // the last stage has been read by every thread
     double2* out = reinterpret_cast<double2*>(tau) + row * M;
     const double cf[3] = {g.YN[0], g.YN[1], g.YN[2]};
@@ -340,9 +346,10 @@ k_fxx_round(GridDesc g, unsigned mask, c64* spec, double* __restrict__ tau, doub
         old[it][q] = out[k];
         pq[it][q] = ph[k];
     });
+    const bool low = is_low(e);
     last_places<M>(t, [&](int k, int it, int q) {
         const c64 z = o[it][q];
-        double2 n = make_double2(from_fixed(z.y, e), from_fixed(z.x, e));
+        double2 n = low ? from_fixed<true>(swap_ri(z), e) : from_fixed(swap_ri(z), e);
         if (bad) n = make_double2(nan(""), nan(""));
         const double da = n.x - old[it][q].x, db = n.y - old[it][q].y;
         acc += da * da + db * db;
@@ -460,14 +467,14 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
     c64 o[P::IL][P::RL];
     transform<L, S>(v, o, t, p, sm, orm, NP, e, g.twf);
     const bool bad = exp_is_nan(E);
-    last_emit<L>(o, t, [&](int k, c64 z) {
-        if (a.inverse) z = swap_ri(z);
-        if (a.fp64_out) {
-            const double qn = bad ? nan("") : 0.0;
-            z = mkc(__double_as_longlong(from_fixed(z.x, e) + qn), __double_as_longlong(from_fixed(z.y, e) + qn));
-        }
-        base[k * step] = z;
-    });
+    const double qn = bad ? nan("") : 0.0;
+    auto emit = [&](auto f) {
+        last_emit<L>(o, t, [&](int k, c64 z) { base[k * step] = f(a.inverse ? swap_ri(z) : z); });
+    };
+    auto bits = [&](double2 d) { return mkc(__double_as_longlong(d.x + qn), __double_as_longlong(d.y + qn)); };
+    if (!a.fp64_out) emit([](c64 z) { return z; });
+    else if (is_low(e)) emit([&](c64 z) { return bits(from_fixed<true>(z, e)); });
+    else emit([&](c64 z) { return bits(from_fixed(z, e)); });
     if (t == 0 && !a.fp64_out) a.eout[plane * M + kx] = bad ? kExpNan : e;
 }
 
@@ -580,7 +587,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
         for (int c = 0; c < 3; ++c) top = max(top, ez[c * NP + p] + bits_of(orm[2 * P3 + c * NP + p]));
         if (kx0 + p == 0 && ky == 0 && addb)   // room for the mean added at DC
             for (int c = 0; c < 3; ++c)
-                if (g.E[slot][c] != 0.0) top = max(top, ilogb(g.gc * g.E[slot][c]) + 1);
+                if (g.E[slot][c] != 0.0) top = max(top, ilogb(g.gcn * g.E[slot][c]) + 1);
         return kx0 + p == 0 ? top + 1 : top;
     };
     auto column_bad = [&](int p) {
@@ -596,11 +603,11 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
         const bool special = kx == 0 && (ky == 0 || ky == N / 2) && (kz == 0 || kz == N / 2);
         if (special) {   // four self-conjugate modes of the packed column, in FP64
             double2 f[3];
-            for (int c = 0; c < 3; ++c) f[c] = make_double2(from_fixed(s[c].x, eg), from_fixed(s[c].y, eg));
+            for (int c = 0; c < 3; ++c) f[c] = from_fixed<true>(s[c], eg);
             if (mode == Z_EQ) {
                 acc += eq_mode(kx, ky, kz, N, f[0], f[1], f[2]);
             } else {
-                const double cE[3] = {g.gc * g.E[slot][0], g.gc * g.E[slot][1], g.gc * g.E[slot][2]};
+                const double cE[3] = {g.gcn * g.E[slot][0], g.gcn * g.E[slot][1], g.gcn * g.E[slot][2]};
                 green_mode<double>(kx, ky, kz, N, 1.0, g.ga, g.gb, addb, cE, f[0], f[1], f[2]);
                 for (int c = 0; c < 3; ++c) s[c] = mkc(to_fixed(f[c].x, eg), to_fixed(f[c].y, eg));
             }
@@ -610,6 +617,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
             const int b = proj_bits(n2);
             long long re[3] = {s[0].x, s[1].x, s[2].x}, im[3] = {s[0].y, s[1].y, s[2].y};
             if (mode == Z_EQ) {
+                // (squares of subnormals are zero)
                 const double dr = from_fixed(dir_dot(re, d, b), eg + b), di = from_fixed(dir_dot(im, d, b), eg + b);
                 acc += (kx == 0 ? 1.0 : 2.0) * (dr * dr + di * di);
             } else {

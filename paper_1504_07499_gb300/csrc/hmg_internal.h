@@ -30,7 +30,12 @@ struct GridDesc {
     int* expB;
     // per-phase coefficients, k0 = sqrt(min k * max k):
     double Y[3];           // (k - k0)/(k + k0): polarization factor of the sweep
-    double YN[3];          // Y / N^3 (FP64 sweeps: the scale of the inverse transform)
+    // FP64 sweeps: the scale 1 / N^3 of the inverse transform, as a factor in (1/2, 1] on the way
+    // into the spectrum, YN = Y 2^sn / N^3, and 2^-sn on the way out (a change of exponent), so
+    // that small fields lose no bits to it
+    double YN[3];
+    double gcn;            // gc 2^sn
+    int sn;                // floor(log2(N^3))
     double W[3];           // k/(k + k0): flux factor, phi = W tau
     double KP[3];          // k + k0: tau = (k + k0) e
     double k0;
