@@ -122,7 +122,7 @@ const char* hmg_last_error(void);
 
 /* Create a context on CUDA device `device`.  `hbm_budget_bytes` caps the device
  * memory the context may hold for solve state (0 = 90 % of the free memory at
- * creation).  *ctx receives the handle; destroy it with hmg_destroy. */
+ * creation); the tables of the grid sizes in use and 64 KB of scratch come on top.  *ctx receives the handle; destroy it with hmg_destroy. */
 hmg_status hmg_create(hmg_ctx** ctx, int device, size_t hbm_budget_bytes);
 
 /* Release every resource of the context (waits for in-flight work). */

@@ -437,8 +437,9 @@ static hmg_status place(hmg_ctx* ctx, uint64_t seed, int n, double r, long long 
                         std::vector<double>& centres, int* generator) {
     DeviceGuard dg(ctx->device);
     cudaStream_t st = ctx->stream;
-    // the kept scratch (it holds 1024 spheres and the filter's buffers); its lists are counted
-    // against the budget for the call
+    // The kept scratch holds 1024 spheres and the filter's bits and survivor list.  Like the tables of
+    // the grid sizes it is a fixed part of a context, outside the budget, which is for state that grows
+    // with the work: of a placement the centres and counters, counted for the call.
     const size_t bytes = (3 * (size_t)n + 2) * sizeof(double);
     const bool counted = ctx->reserve(bytes);
     void* mem = counted ? ctx->scratch_get(PlaceScratch::bytes(n)) : nullptr;

@@ -207,8 +207,9 @@ struct hmg_ctx {
     std::mutex server_mu;              // guards the creation of `server`
     hmg::Tracer tracer;
     std::map<int, int> ztune;   // autotuned z-pass variant per grid size (FP32 path)
-    // Device scratch of the placement and voxelization calls (sphere lists), kept for the
-    // life of the context; a larger need allocates for the call.
+    // Device scratch of the placement, voxelization and sweep calls (sphere lists, residual sums),
+    // kept for the life of the context outside the budget, as the tables of `plans` are; a larger
+    // need allocates for the call.
     static constexpr size_t kScratchBytes = 64 * 1024;
     void* scratch = nullptr;
     void* scratch_get(size_t bytes);   // nullptr: out of device memory
