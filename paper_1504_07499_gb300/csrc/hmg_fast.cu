@@ -48,7 +48,10 @@ __device__ unsigned g_wait_fail;
 template <int L, int base>
 constexpr int col_min_ctas() { return Split<L>::E > 24 ? base - 1 : base; }
 
-template <int L, int P, bool FWD>
+// Columns along y of each (component, z) plane, or with ZDIR along z of each (component, ky) plane
+// (plain transforms, of the grids there are; the sweeps' z passes below take three together.  Both
+// directions of one grid through the C ABI, us, before and now: 256^3 460 and 342, 512^3 3872 and 2465).
+template <int L, int P, bool FWD, bool ZDIR = false>
 __global__ void __launch_bounds__(P * Split<L>::TP, col_min_ctas<L, 3>())
 k_fy(GridDesc g, unsigned mask, float2* __restrict__ spec) {
     constexpr int E = Split<L>::E, TP = Split<L>::TP;
@@ -61,10 +64,12 @@ k_fy(GridDesc g, unsigned mask, float2* __restrict__ spec) {
     const int nkb = M / P;
     const int kb = blockIdx.x % nkb;
     const long long cz = blockIdx.x / nkb;
-    float2* base = spec + (long long)slot * 3 * g.NNM + cz * (long long)L * M + kb * P + p;
+    const long long step = ZDIR ? (long long)L * M : M;
+    float2* base = spec + (long long)slot * 3 * g.NNM +
+                   (ZDIR ? cz / L * g.NNM + cz % L * M : cz * (long long)L * M) + kb * P + p;
     float2 v[E];
 #pragma unroll
-    for (int n1 = 0; n1 < E; ++n1) v[n1] = base[(long long)(TP * n1 + t) * M];
+    for (int n1 = 0; n1 < E; ++n1) v[n1] = base[(TP * n1 + t) * step];
     const float2* twL = g.tw32;
     stage1_write<L, FWD>(v, t, twL, sh + p, P);
     __syncthreads();
@@ -73,7 +78,7 @@ k_fy(GridDesc g, unsigned mask, float2* __restrict__ spec) {
 #pragma unroll
     for (int i = 0; i < KPT; ++i)
 #pragma unroll
-        for (int k2 = 0; k2 < TP; ++k2) base[(long long)(t * KPT + i + E * k2) * M] = v[i * TP + k2];
+        for (int k2 = 0; k2 < TP; ++k2) base[(t * KPT + i + E * k2) * step] = v[i * TP + k2];
 }
 
 // ---------------------------------------------------------------------------
@@ -128,30 +133,11 @@ k_fz3(GridDesc g, unsigned mask, float2* spec, double* __restrict__ partial) {
 #pragma unroll
         for (int n1 = 0; n1 < E; ++n1) v[c][n1] = base[c * NNM + (long long)(TP * n1 + t) * rowz];
 
-    if (MODE == Z_INV) {
-        // plain inverse transform of each component (natural order in and out)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) stage1_write<L, false>(v[c], t, twL, sh + c * NS + p, P);
-        __syncthreads();
+    for (int c = 0; c < 3; ++c) stage1_write<L, true>(v[c], t, twL, sh + c * NS + p, P);
+    __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 3; ++c) stage2_read<L, false>(v[c], t, sh + c * NS + p, P);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) stage1_write<L, true>(v[c], t, twL, sh + c * NS + p, P);
-        __syncthreads();
-#pragma unroll
-        for (int c = 0; c < 3; ++c) stage2_read<L, true>(v[c], t, sh + c * NS + p, P);
-    }
-    if (MODE == Z_FWD || MODE == Z_INV) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int i = 0; i < KPT; ++i)
-#pragma unroll
-                for (int k2 = 0; k2 < TP; ++k2)
-                    base[c * NNM + (long long)(t * KPT + i + E * k2) * rowz] = v[c][i * TP + k2];
-        return;
-    }
+    for (int c = 0; c < 3; ++c) stage2_read<L, true>(v[c], t, sh + c * NS + p, P);
     if (MODE == Z_EQ) {
         double acc = 0.0;
 #pragma unroll
@@ -315,22 +301,9 @@ k_fzs(GridDesc g, unsigned mask, float2* spec, double* __restrict__ partial) {
 #pragma unroll
     for (int n1 = 0; n1 < E; ++n1) v[n1] = base[(long long)(TP * n1 + t) * rowz];
 
-    if (MODE == Z_INV) {
-        stage1_write<L, false>(v, t, twL, shc, P);
-        __syncthreads();
-        stage2_read<L, false>(v, t, shc, P);
-    } else {
-        stage1_write<L, true>(v, t, twL, shc, P);
-        __syncthreads();
-        stage2_read<L, true>(v, t, shc, P);
-    }
-    if (MODE == Z_FWD || MODE == Z_INV) {
-#pragma unroll
-        for (int i = 0; i < KPT; ++i)
-#pragma unroll
-            for (int k2 = 0; k2 < TP; ++k2) base[(long long)(t * KPT + i + E * k2) * rowz] = v[i * TP + k2];
-        return;
-    }
+    stage1_write<L, true>(v, t, twL, shc, P);
+    __syncthreads();
+    stage2_read<L, true>(v, t, shc, P);
     // share of d . s of this component, one slot per (t, value) of the thread group
     __syncthreads();   // every thread has read the forward exchange
 #pragma unroll
@@ -1483,16 +1456,18 @@ constexpr bool pair_rows(int N) { return N == 64 || N == 128 || N == 192 || N ==
 #define HMG_FAST_LEN(L, X) \
     case L: X(L); return true;
 
-bool fast_y(const GridDesc& g, bool fwd, unsigned mask, void* spec, cudaStream_t st) {
+namespace {
+template <bool ZDIR>
+bool fast_col(const GridDesc& g, bool fwd, unsigned mask, void* spec, cudaStream_t st) {
     float2* sp = reinterpret_cast<float2*>(spec);
 #define FY(L)                                                                                     \
     {                                                                                             \
         constexpr int P = fy_cols<L>();                                                           \
         if (g.M % P) return false;                                                                \
-        dim3 grid(g.comps * g.N * (g.M / P), g.nslots);                                                 \
+        dim3 grid(g.comps * g.N * (g.M / P), g.nslots);                                           \
         const size_t sm = sizeof(float2) * fast::xslots<L>() * P;                                 \
-        if (fwd) launch_dyn(fast::k_fy<L, P, true>, grid, P * fast::Split<L>::TP, sm, st, g, mask, sp);  \
-        else launch_dyn(fast::k_fy<L, P, false>, grid, P * fast::Split<L>::TP, sm, st, g, mask, sp);     \
+        auto k = fwd ? fast::k_fy<L, P, true, ZDIR> : fast::k_fy<L, P, false, ZDIR>;              \
+        launch_dyn(k, grid, P * fast::Split<L>::TP, sm, st, g, mask, sp);                         \
     }
     switch (g.N) {
         HMG_FAST_LEN(64, FY)
@@ -1504,6 +1479,11 @@ bool fast_y(const GridDesc& g, bool fwd, unsigned mask, void* spec, cudaStream_t
         default: return false;
     }
 #undef FY
+}
+}  // namespace
+
+bool fast_y(const GridDesc& g, bool fwd, unsigned mask, void* spec, cudaStream_t st) {
+    return fast_col<false>(g, fwd, mask, spec, st);
 }
 
 int fast_z_ctas(const GridDesc& g) {
@@ -1527,8 +1507,6 @@ void launch_fzs(int mode, dim3 grid, size_t sm, cudaStream_t st, const GridDesc&
                 double* partial) {
     constexpr int T = 3 * P * fast::Split<L>::TP;
     switch (mode) {
-        case Z_FWD: launch_dyn(fast::k_fzs<L, P, Z_FWD>, grid, T, sm, st, g, mask, sp, partial); break;
-        case Z_INV: launch_dyn(fast::k_fzs<L, P, Z_INV>, grid, T, sm, st, g, mask, sp, partial); break;
         case Z_ITER: launch_dyn(fast::k_fzs<L, P, Z_ITER>, grid, T, sm, st, g, mask, sp, partial); break;
         case Z_ITER_NOB: launch_dyn(fast::k_fzs<L, P, Z_ITER_NOB>, grid, T, sm, st, g, mask, sp, partial); break;
         default: launch_dyn(fast::k_fzs<L, P, Z_EQ>, grid, T, sm, st, g, mask, sp, partial); break;
@@ -1557,8 +1535,6 @@ void launch_fz3(int mode, dim3 grid, size_t sm, cudaStream_t st, const GridDesc&
                 double* partial) {
     constexpr int T = P * fast::Split<L>::TP;
     switch (mode) {
-        case Z_FWD: launch_dyn(fast::k_fz3<L, P, Z_FWD>, grid, T, sm, st, g, mask, sp, partial); break;
-        case Z_INV: launch_dyn(fast::k_fz3<L, P, Z_INV>, grid, T, sm, st, g, mask, sp, partial); break;
         case Z_ITER: launch_dyn(fast::k_fz3<L, P, Z_ITER>, grid, T, sm, st, g, mask, sp, partial); break;
         case Z_ITER_NOB: launch_dyn(fast::k_fz3<L, P, Z_ITER_NOB>, grid, T, sm, st, g, mask, sp, partial); break;
         default: launch_dyn(fast::k_fz3<L, P, Z_EQ>, grid, T, sm, st, g, mask, sp, partial); break;
@@ -1585,6 +1561,7 @@ bool fast_z_len(const GridDesc& g, int mode, unsigned mask, float2* sp, double* 
 }  // namespace
 
 bool fast_z(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st) {
+    if (mode == Z_FWD || mode == Z_INV) return fast_col<true>(g, mode == Z_FWD, mask, spec, st);
     float2* sp = reinterpret_cast<float2*>(spec);
     switch (g.N) {
         case 64: return fast_z_len<64>(g, mode, mask, sp, partial, st);
