@@ -1,4 +1,4 @@
-// libhmg host runtime: contexts, FFT schedules, device buffers, the solve driver of
+// libhmg host runtime: contexts, transform tables, device buffers, the solve driver of
 // §3's Algorithm (FP64 and FP32-bulk with FP64 defect correction), and the C ABI.
 #include <cuda_runtime.h>
 

@@ -8,10 +8,7 @@
 namespace hmg {
 
 __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
 
-template <typename T2> __device__ __forceinline__ T2 cadd(T2 a, T2 b) { return mk(a.x + b.x, a.y + b.y); }
-template <typename T2> __device__ __forceinline__ T2 csub(T2 a, T2 b) { return mk(a.x - b.x, a.y - b.y); }
 template <typename T2> __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
     return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -27,7 +24,6 @@ template <bool FWD, typename T2> __device__ __forceinline__ T2 mul_mi(T2 a) {
 
 // FP32 complex adds and subtracts as single packed two-lane FP32 instructions (sm_100
 // and later); a - b is b * (-1) + a, exact product, one rounding, as the scalar form.
-// Overloads of the templates above, chosen for float2.
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 

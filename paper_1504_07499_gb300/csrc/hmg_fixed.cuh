@@ -365,8 +365,8 @@ template <> struct Dft<24> : CoprimeDft<8, 3> {};
 
 // Component bits a radix may start from: R 2^(b + 1/2) < 2^63 without twiddles (`first`),
 // R 2^(b + 1/2) / 4 < 2^63 and b <= 62 behind the /4 of the twiddle product (`later`).
-constexpr int first_bits(int R) { return R >= 12 ? 58 : R >= 6 ? 59 : R >= 3 ? 60 : 61; }
-constexpr int later_bits(int R) { return R >= 12 ? 60 : R >= 6 ? 61 : 62; }
+constexpr int first_bits(int R) { return R >= 6 ? 59 : R >= 3 ? 60 : 61; }   // (R <= 9 in every plan)
+constexpr int later_bits(int R) { return R >= 6 ? 61 : 62; }
 
 // Radices of a length (first stage first, 1 = no stage) and threads per pencil: every
 // thread takes whole radix butterflies, one to three per stage.  Three stages of at most 8

@@ -13,6 +13,7 @@
 // at 256^3 through the C ABI went 9.7 -> 2.2 ms (copies and conversions of the field included).
 #pragma once
 
+#include "hmg_cta.cuh"
 #include "hmg_fft.cuh"
 #include "hmg_fixed.cuh"
 #include "hmg_green.cuh"
@@ -21,13 +22,6 @@
 namespace hmg {
 namespace fx {
 
-// largest divisor of n that is at most lim
-constexpr int divisor_upto(long long n, int lim) {
-    int d = 1;
-    for (int i = 1; i <= lim; ++i)
-        if (n % i == 0) d = i;
-    return d;
-}
 // rows per CTA of an x pass of length M, columns per CTA of a column / z pass of length L:
 // about 128 to 256 threads; columns in runs of at least 64 bytes where N/2 allows it
 template <int M> constexpr int x_rows() { return divisor_upto(4LL * M * M, 192 / Plan<M>::TPP > 1 ? 192 / Plan<M>::TPP : 1); }
@@ -46,25 +40,6 @@ template <int L> constexpr int z_cols() {
 constexpr int min_ctas(int threads, int per_sm) {
     const int t = (threads + 31) / 32 * 32;
     return t >= per_sm ? 1 : per_sm / t;
-}
-constexpr int pow2_at_least(int n) {
-    int p = 1;
-    while (p < n) p *= 2;
-    return p;
-}
-
-// fixed-order sum over the CTA's T threads, valid in thread 0; sh: pow2_at_least(T) doubles
-template <int T>
-__device__ double cta_sum(double v, double* sh) {
-    constexpr int P = pow2_at_least(T);
-    sh[threadIdx.x] = v;
-    if (threadIdx.x + T < P) sh[threadIdx.x + T] = 0.0;
-    __syncthreads();
-    for (int s = P / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    return sh[0];
 }
 
 __device__ __forceinline__ double coef3(int ph, const double* c) { return ph == 0 ? c[0] : (ph == 1 ? c[1] : c[2]); }

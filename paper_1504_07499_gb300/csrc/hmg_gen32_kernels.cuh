@@ -12,6 +12,7 @@
 // the chained x round trip is that of hmg_fast.cu.
 #pragma once
 
+#include "hmg_cta.cuh"
 #include "hmg_fft.cuh"
 #include "hmg_fixed.cuh"
 #include "hmg_green.cuh"
@@ -57,12 +58,6 @@ template <> struct Plan<384> : PlanOf<24, 16, 1, 24> {};
 template <> struct Plan<432> : PlanOf<24, 18, 1, 24> {};
 template <> struct Plan<486> : PlanOf<9, 9, 6, 54> {};
 
-constexpr int divisor_upto(long long n, int lim) {
-    int d = 1;
-    for (int i = 1; i <= lim; ++i)
-        if (n % i == 0) d = i;
-    return d;
-}
 // CTAs of about 128 to 256 threads; columns in runs of up to 16 (128 bytes)
 template <int M> constexpr int x_rows() { return divisor_upto(4LL * M * M, 160 / Plan<M>::TPP > 1 ? 160 / Plan<M>::TPP : 1); }
 template <int L> constexpr int col_cols() {
@@ -77,24 +72,6 @@ template <int L> constexpr int z_cols() {
 template <int L> constexpr int min_ctas(int threads) {
     const int t = (threads + 31) / 32 * 32, per = Plan<L>::R0 > 18 ? 768 : 1024;
     return t >= per ? 1 : per / t;
-}
-constexpr int pow2_at_least(int n) {
-    int p = 1;
-    while (p < n) p *= 2;
-    return p;
-}
-// fixed-order sum over the CTA's T threads, valid in thread 0; sh: pow2_at_least(T) doubles
-template <int T>
-__device__ double cta_sum(double v, double* sh) {
-    constexpr int P = pow2_at_least(T);
-    sh[threadIdx.x] = v;
-    if (threadIdx.x + T < P) sh[threadIdx.x + T] = 0.0;
-    __syncthreads();
-    for (int s = P / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    return sh[0];
 }
 
 // ---------------------------------------------------------------------------

@@ -15,7 +15,7 @@ constexpr int kMaxSlots = 3;       // right-hand sides (unit gradients) per RVE
     X(8) X(12) X(16) X(18) X(24) X(32) X(36) X(48) X(54) X(64) X(72) X(96) X(108) X(128) X(144) X(162) \
     X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
 
-// Everything a pass kernel needs about one RVE: sizes, FFT schedules, the
+// Everything a pass kernel needs about one RVE: sizes, transform tables, the
 // per-phase coefficient table, and the device fields (FP32 or FP64 copies).
 struct GridDesc {
     int N, M;              // grid size and N/2 (complex length of an x row)
@@ -96,7 +96,7 @@ void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, c
 template <typename R>
 void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial,
                    cudaStream_t st);
-// FP64 Z_INV of a plain transform from another buffer
+// the inverse of launch_z_pass<double>'s Z_FWD, from another buffer
 void launch_z_inverse_from(const GridDesc& g, unsigned mask, const void* src, void* spec, cudaStream_t st);
 // x inverse: writes tau (INPLACE*), adds r (ADD_R, ADD_R_RES), or writes d = new - old to
 // d32 and r32 without touching tau (DIFF).  Residual modes add (new-old)^2 per CTA.

@@ -198,7 +198,7 @@ void launch_y_pass(const GridDesc& g, bool forward, unsigned mask, void* spec, c
 template <typename R>
 void launch_z_pass(const GridDesc& g, int mode, unsigned mask, void* spec, double* partial, cudaStream_t st) {
     if constexpr (std::is_same<R, double>::value) {
-        if (mode == Z_FWD || mode == Z_INV) fx_z_plain(g, mode == Z_FWD, mask, spec, spec, st);
+        if (mode == Z_FWD) fx_z_plain(g, true, mask, spec, spec, st);
         else fx_z(g, mode, mask, spec, partial, st);
     } else if (!fast_z(g, mode, mask, spec, partial, st)) {
         gen_z(g, mode, mask, spec, partial, st);

@@ -86,8 +86,7 @@ __device__ __forceinline__ bool clear_of(float4 a, float4 b, const double* p, co
 // accepted and the later ones are re-examined against it only.  The candidates are items
 // begin .. limit - 1, or, with a list, the candidates list[0 .. limit - 1], which the filter has
 // found clear of the first `known` centres.
-// out: 3 n doubles, the first state[0] of them placed before; state[0] = spheres placed,
-// state[1] = 1 + the last candidate examined.
+// out: 3 n doubles, the first state[0] centres placed before; state[0] = spheres placed.
 __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double lim, long long begin, long long limit,
                                                   const int* __restrict__ list, long long list_base,
                                                   double* __restrict__ out, long long* __restrict__ state) {
@@ -104,7 +103,6 @@ __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double l
     __syncthreads();
     for (int i = t; i < known; i += kThreads) accf[i] = narrow(acc[3 * i], acc[3 * i + 1], acc[3 * i + 2]);
     __syncthreads();
-    long long used = begin;
     for (long long j0 = begin; j0 < limit && s_count < n; j0 += kThreads) {
         const bool valid = j0 + t < limit;
         const long long j = !valid ? 0 : list ? list_base + list[j0 + t] : j0 + t;
@@ -145,18 +143,13 @@ __global__ void __launch_bounds__(kThreads) k_rsa(uint64_t base, int n, double l
                 start = f + 1;
                 if (s_count >= n) {
                     round_done = true;
-                    used = j0 + f + 1;
                 }
             }
             __syncthreads();
         }
-        if (s_count < n) used = min(j0 + kThreads, limit);
     }
     for (int i = t; i < 3 * s_count; i += kThreads) out[i] = acc[i];
-    if (t == 0) {
-        state[0] = s_count;
-        state[1] = used;
-    }
+    if (t == 0) state[0] = s_count;
 }
 
 // After the first block most spheres are placed and nearly every candidate is rejected by one of
