@@ -11,8 +11,9 @@
 // most 2^-58 of the pencil's largest value where FP64 arithmetic rounds each operation to
 // 2^-53 of its own size.  Before each later radix the largest magnitude actually reached
 // decides how far the values are shifted down (mostly not at all), so no bits are given up
-// to worst-case growth.  Data twiddles carry 62 fractional bits.  Errors against 80-bit
-// references are below those of the FP64 passes these replace (see the tests).
+// to worst-case growth.  Data twiddles carry 62 fractional bits.  A forward
+// transform of N = 8 .. 72 errs by 3 to 7e-17 of its norm against long double, its rounding to
+// FP64 included (test_gpu_fixed_accuracy.py bounds it by 1.1e-16 and 1.7e-16).
 //
 // Between passes the spectrum stays in integers, with the exponent of the pencil that wrote
 // each value in a side array, so only the field side of the x passes converts to and from
