@@ -498,16 +498,16 @@ int Tracer::begin(cudaStream_t st) {
 void Tracer::end(int ev, int kind, double b, cudaStream_t st) {
     if (ev < 0) return;
     cudaEventRecord(events[2 * ev + 1], st);
-    pending.push_back({kind, ev, b});
+    pending.push_back({kind, ev, b, sweep});
 }
 
-void Tracer::collect() {
+void Tracer::collect(const double* share) {
     for (const Pending& p : pending) {
         float t = 0.f;
         if (cudaEventElapsedTime(&t, events[2 * p.ev], events[2 * p.ev + 1]) == cudaSuccess) {
             ms[p.kind] += t;
             launches[p.kind] += 1;
-            bytes[p.kind] += p.bytes;
+            bytes[p.kind] += share && p.sweep >= 0 ? share[p.sweep] * p.bytes : p.bytes;
         } else {
             cudaGetLastError();
         }
@@ -586,13 +586,17 @@ void Solver::sweeps(unsigned mask, R* field, void* spec, int n, double* sums, in
     // 192^3 357 and 360, 256^3 709 and 974).
     const bool in_l2 = g.nslots * 3 * (double)g.N3 * sizeof(double) <= 56e6;
     if (g.relax != 0.0 || (f64 ? !in_l2 : !fast_x_round_res_available(g))) {
-        for (int b = 0; b < n; ++b)
+        for (int b = 0; b < n; ++b) {
+            if (tr) tr->sweep = b;
             sweep<R>(mask, field, spec, Z_ITER, XI_INPLACE_RES, nullptr, nullptr, nullptr, sums + b * stride, stop);
+        }
+        if (tr) tr->sweep = -1;
         return;
     }
     const double f = (double)popc(mask) * 3.0 * (double)g.N3, F = sizeof(R);   // field elements moved per array
     double* pb = psweep ? psweep : s->partial;
     for (int b = 0; b < n; ++b) {
+        if (tr) tr->sweep = b;
         if (b == 0)
             HMG_TRACED(kind_of<R>(HMG_K_X_FORWARD), f * 2 * F + (double)g.N3,
                        launch_x_forward<R>(g, XF_POLARIZE, mask, field, spec, nullptr, st));
@@ -610,6 +614,7 @@ void Solver::sweeps(unsigned mask, R* field, void* spec, int n, double* sums, in
         HMG_TRACED(kind_of<R>(HMG_K_OTHER), 0.0,
                    launch_reduce(pb, g.nslots, x_ctas_for<R>(g), 1, sums + b * stride, st, stop));
     }
+    if (tr) tr->sweep = -1;
 }
 
 bool Solver::chained() const { return chain_sweeps(g); }
@@ -777,7 +782,13 @@ hmg_status Solver::run_fp64(int max_iter, double tol, hmg_info* info, double K[9
             set_error("CUDA error: %s", cudaGetErrorString(ce));
             return HMG_CUDA_ERROR;
         }
-        if (tr) tr->collect();
+        if (tr) {   // bytes of the gradients whose sweep was not skipped
+            double share[kAhead64] = {};
+            for (int b = 0; b < blk; ++b)
+                for (int sl = 0; sl < g.nslots; ++sl)
+                    if (((active >> sl) & 1u) && !(h[3 * b + sl] < 0.0)) share[b] += 1.0 / popc(active);
+            tr->collect(share);
+        }
         for (int sl = 0; sl < g.nslots; ++sl) {
             if (!((active >> sl) & 1u)) continue;
             for (int b = 0; b < blk; ++b) {

@@ -7,7 +7,7 @@
 //
 // Numbers.  A pencil (one 1D transform) holds complex integers v with a common exponent e,
 // value v 2^e.  On load every pencil is scaled so that its largest component fills `first`
-// bits (58 to 60, what the first radix can grow without overflow), so the quantum is at
+// bits (59 or 60, what the first radix can grow without overflow), so the quantum is at
 // most 2^-58 of the pencil's largest value where FP64 arithmetic rounds each operation to
 // 2^-53 of its own size.  Before each later radix the largest magnitude actually reached
 // decides how far the values are shifted down (mostly not at all), so no bits are given up

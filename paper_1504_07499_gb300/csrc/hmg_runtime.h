@@ -95,13 +95,16 @@ struct Tracer {
         int kind;
         int ev;
         double bytes;
+        int sweep;
     };
+    int sweep = -1;                    // sweep of a block that may be skipped, or -1
     std::vector<cudaEvent_t> events;   // pairs (start, stop)
     std::vector<int> free_pairs;
     std::vector<Pending> pending;
     int begin(cudaStream_t st);
     void end(int ev, int kind, double bytes, cudaStream_t st);
-    void collect();                    // after a stream synchronize
+    // after a stream synchronize; share[b]: part of the gradients for which sweep b was not skipped
+    void collect(const double* share = nullptr);
     void reset();
     ~Tracer();
 };
