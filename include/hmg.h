@@ -417,9 +417,10 @@ hmg_status hmg_trace_read(hmg_ctx* ctx, int kind, double* total_ms, long long* l
                           double* algo_bytes);
 
 /* Measured FP64 fused-multiply-add rate of the context's GPU (flop/s, 2 per FMA): long
- * register-only chains over the whole device, best of five timed launches.  The plain
- * FP64 form of the solver is bound by this rate rather than by HBM bandwidth; the
- * paper has no counterpart (a measurement aid for the roofline of that form). */
+ * register-only chains over the whole device, best of five timed launches.  FP64
+ * butterflies would be bound by this rate rather than by HBM bandwidth; the FP64 form of the
+ * solver therefore runs its transforms on 64-bit integers.  The paper has no counterpart (a
+ * measurement aid for the roofline of that form). */
 hmg_status hmg_fp64_rate(hmg_ctx* ctx, double* flops_out);
 
 /* Request-loop counters (zeros before the first hmg_submit): out[0] submitted,

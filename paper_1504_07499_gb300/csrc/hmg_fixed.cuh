@@ -1,7 +1,7 @@
 // FP64 transforms in block fixed point: 64-bit integers with one exponent per pencil.
 //
 // GB300 issues 2 FP64 operations per clock and SM, against 128 32-bit integer adds and 16
-// 32x32+64 multiply-adds (IMAD.WIDE): measured, 0.50 T DFMA/s and 15.8 T 64-bit adds/s.  An
+// 32x32+64 multiply-adds (IMAD.WIDE): measured, 0.63 T DFMA/s and 15.8 T 64-bit adds/s.  An
 // FP64 pass is therefore bound by the FP64 pipe (97 % of a sweep; 9.7 ms per gradient at
 // 256^3), and the same butterflies on 64-bit integers cost a tenth of that.
 //

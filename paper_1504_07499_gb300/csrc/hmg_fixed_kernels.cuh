@@ -10,7 +10,7 @@
 // value in a column pass, 59 in the z pass, whose 0.54 ms it could do in 0.32), then latency;
 // FP64 is left for the coefficient product, the flux sum and the residual (1 to 2 operations
 // per real value).  Against the FP64 butterflies these replace, one sweep of one gradient
-// at 256^3 through the C ABI went 9.7 -> 2.2 ms (copies and conversions of the field included).
+// at 256^3 through the C ABI went 9.7 -> 1.9 ms (copies and conversions of the field included).
 #pragma once
 
 #include "hmg_cta.cuh"

@@ -1,5 +1,5 @@
-// FP64 arithmetic rate of the device: the ceiling of the plain FP64 form of the solver,
-// whose passes are bound by the FP64 pipe rather than by HBM.  A grid of threads runs
+// FP64 arithmetic rate of the device: the ceiling of transforms in FP64 arithmetic, and why the
+// FP64 passes are in block fixed point (hmg_fixed.cuh).  A grid of threads runs
 // long chains of dependent fused multiply-adds on eight independent accumulators each (no
 // memory traffic in the loop); the rate is 2 flops per FMA over the CUDA-event time.
 #include <cuda_runtime.h>
