@@ -4,14 +4,15 @@
 namespace hmg {
 
 namespace {
+template <bool PLAIN>
 void col(const GridDesc& g, unsigned mask, const void* src, void* spec, const fx::ColArgs& a, cudaStream_t st) {
     const fx::c64* in = reinterpret_cast<const fx::c64*>(src);
     fx::c64* sp = reinterpret_cast<fx::c64*>(spec);
     switch (g.N) {
 #define X(N_)                                                                                          \
     case N_:                                                                                           \
-        fx::launch(fx::k_fxx_col<N_>, dim3(g.comps * N_ * (N_ / 2 / fx::ColShape<N_>::NP), g.nslots),   \
-                   fx::ColShape<N_>::T, fx::ColShape<N_>::smem, st, g, mask, in, sp, a);                    \
+        fx::launch(fx::k_fxx_col<N_, PLAIN>, dim3(g.comps * N_ * (N_ / 2 / fx::ColShape<N_>::NP), g.nslots), \
+                   fx::ColShape<N_>::T, fx::ColShape<N_>::smem, st, g, mask, in, sp, a);                 \
         break;
         HMG_ALL_SIZES(X)
 #undef X
@@ -20,11 +21,11 @@ void col(const GridDesc& g, unsigned mask, const void* src, void* spec, const fx
 }  // namespace
 
 void fx_y(const GridDesc& g, bool forward, unsigned mask, void* spec, cudaStream_t st) {
-    col(g, mask, spec, spec, fx::ColArgs{0, forward ? 0 : 1, 0, 0, g.expA, g.expB}, st);
+    col<false>(g, mask, spec, spec, fx::ColArgs{forward ? 0 : 1, g.expA, g.expB}, st);
 }
 
 void fx_z_plain(const GridDesc& g, bool forward, unsigned mask, const void* src, void* spec, cudaStream_t st) {
-    col(g, mask, src, spec, fx::ColArgs{1, forward ? 0 : 1, forward ? 0 : 1, forward ? 1 : 0, g.expB, g.expA}, st);
+    col<true>(g, mask, src, spec, fx::ColArgs{forward ? 0 : 1, g.expB, g.expA}, st);
 }
 
 }  // namespace hmg

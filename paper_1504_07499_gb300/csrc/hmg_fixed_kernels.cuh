@@ -10,7 +10,7 @@
 // value in a column pass, 59 in the z pass, whose 0.54 ms it could do in 0.32), then latency;
 // FP64 is left for the coefficient product, the flux sum and the residual (1 to 2 operations
 // per real value).  Against the FP64 butterflies these replace, one sweep of one gradient
-// at 256^3 through the C ABI went 9.7 -> 1.9 ms (copies and conversions of the field included).
+// at 256^3 through the C ABI went 9.7 -> 1.8 ms (copies and conversions of the field included).
 #pragma once
 
 #include "hmg_cta.cuh"
@@ -360,9 +360,7 @@ k_fxx_round(GridDesc g, unsigned mask, c64* spec, double* __restrict__ tau, doub
 // passes of a plain 3D transform, which read or write FP64 on their far side)
 // ---------------------------------------------------------------------------
 struct ColArgs {
-    int zdir;       // 0: columns along y of each (component, z) plane, 1: along z of each (component, ky)
     int inverse;
-    int fp64_in, fp64_out;
     const int* ein;
     int* eout;
 };
@@ -374,7 +372,10 @@ struct ColShape {
     static constexpr size_t smem = sizeof(c64) * S::TOTAL;
 };
 
-template <int L>
+// PLAIN: along z of each (component, ky) plane, from FP64 (inverse) or to FP64 (forward); else along y of
+// each (component, z) plane, integers both ways (chosen at run time the FP64 side cost the y passes
+// registers and code: a sweep of one gradient 29.1 us against 28.3 at 32^3, 1790 against 1712 at 256^3).
+template <int L, bool PLAIN>
 __global__ void __launch_bounds__(ColShape<L>::T, min_ctas(ColShape<L>::T, 1024))
 k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
     using C = ColShape<L>;
@@ -384,6 +385,7 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
     grid_begin();
     const int slot = blockIdx.y;
     if (!slot_active(g, mask, slot)) return;
+    const bool fp64_in = PLAIN && a.inverse, fp64_out = PLAIN && !a.inverse;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     c64* sm = reinterpret_cast<c64*>(smem_raw);
     __shared__ int key[NP];
@@ -397,13 +399,13 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
     const int cw = blockIdx.x / (M / NP);                        // c L + z (y columns) or c L + ky (z columns)
     const long long plane = (long long)slot * 3 * L + cw;        // (slot, c, z) or (slot, c, ky)
     const long long comp = (long long)slot * 3 + cw / L;         // (slot, c)
-    const long long first = a.zdir ? comp * L * L * M + (long long)(cw % L) * M + kx : plane * L * M + kx;
-    const long long step = a.zdir ? (long long)L * M : M;
+    const long long first = PLAIN ? comp * L * L * M + (long long)(cw % L) * M + kx : plane * L * M + kx;
+    const long long step = PLAIN ? (long long)L * M : M;
     const c64* in = src + first;   // the same buffer, or the FP64 spectrum of a plain inverse
     c64* base = spec + first;
     // exponent of element i: per (plane, y) for the y forward, per (component, i, kx) otherwise
-    const int* ein = a.ein + (!a.zdir && !a.inverse ? plane * L : comp * L * M + kx);
-    const int estep = !a.zdir && !a.inverse ? 1 : M;
+    const int* ein = a.ein + (!PLAIN && !a.inverse ? plane * L : comp * L * M + kx);
+    const int estep = !PLAIN && !a.inverse ? 1 : M;
     __syncthreads();
     c64 v[P::I0][P::R0];
     int mk = kExpZero;
@@ -415,7 +417,7 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
             for (int q = 0; q < P::R0; ++q) {
                 const int i = j + q * J;
                 v[it][q] = in[i * step];
-                if (a.fp64_in)
+                if (fp64_in)
                     mk = max(mk, max(key_of(__longlong_as_double(v[it][q].x)), key_of(__longlong_as_double(v[it][q].y))));
                 else
                     mk = max(mk, ein[i * estep] + bits_of(mag(v[it][q])));
@@ -433,7 +435,7 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
 #pragma unroll
             for (int q = 0; q < P::R0; ++q) {
                 c64 z = v[it][q];
-                if (a.fp64_in) z = mkc(to_fixed(__longlong_as_double(z.x), e), to_fixed(__longlong_as_double(z.y), e));
+                if (fp64_in) z = mkc(to_fixed(__longlong_as_double(z.x), e), to_fixed(__longlong_as_double(z.y), e));
                 else z = shift(z, ein[(j + q * J) * estep] - e);
                 v[it][q] = a.inverse ? swap_ri(z) : z;
             }
@@ -447,10 +449,10 @@ k_fxx_col(GridDesc g, unsigned mask, const c64* src, c64* spec, ColArgs a) {
         last_emit<L>(o, t, [&](int k, c64 z) { base[k * step] = f(a.inverse ? swap_ri(z) : z); });
     };
     auto bits = [&](double2 d) { return mkc(__double_as_longlong(d.x + qn), __double_as_longlong(d.y + qn)); };
-    if (!a.fp64_out) emit([](c64 z) { return z; });
+    if (!fp64_out) emit([](c64 z) { return z; });
     else if (is_low(e)) emit([&](c64 z) { return bits(from_fixed<true>(z, e)); });
     else emit([&](c64 z) { return bits(from_fixed(z, e)); });
-    if (t == 0 && !a.fp64_out) a.eout[plane * M + kx] = bad ? kExpNan : e;
+    if (t == 0 && !fp64_out) a.eout[plane * M + kx] = bad ? kExpNan : e;
 }
 
 // ---------------------------------------------------------------------------
