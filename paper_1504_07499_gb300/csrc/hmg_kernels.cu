@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "hmg_internal.h"
@@ -105,22 +106,23 @@ __global__ void k_e_to_tau(GridDesc g, int slot, const double* __restrict__ e, R
 // in the last place, and one residual step with the rounded reciprocal, which then rounds
 // correctly for every divisor (Markstein, "Computation of elementary functions on the IBM RISC
 // System/6000 processor", 1990): four FP64 operations instead of a divide's ten or so, which bound
-// this kernel.  Operands whose residual could leave the normal range are divided.
-template <typename R>
-__global__ void k_tau_to_e(GridDesc g, int slot, const R* __restrict__ tau, double* __restrict__ e) {
+// this kernel.  Operands whose residual could leave the normal range are divided.  The reciprocals
+// come from the host: formed in every thread they cost more FP64 operations than the one or two
+// voxels that a thread of a grid up to 96^3 has (a call of one FP32 sweep at 96^3 142 -> 117 us).
+struct Reciprocals {
     double rc[3], rl[3];   // 1 / KP = rc + rl
-    for (int p = 0; p < 3; ++p) {
-        rc[p] = 1.0 / g.KP[p];
-        rl[p] = fma(-rc[p], g.KP[p], 1.0) * rc[p];
-    }
+};
+
+template <typename R>
+__global__ void k_tau_to_e(GridDesc g, Reciprocals kr, int slot, const R* __restrict__ tau, double* __restrict__ e) {
     auto in_range = [](double d) {   // 2^-823 <= |d| < 2^777, without the FP64 pipe
         return ((unsigned)__double2hiint(d) >> 20 & 0x7ffu) - 200u < 1600u;
     };
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N3; i += (long long)gridDim.x * blockDim.x) {
         const int ph = g.phase[i];
         const double kp = ph == 0 ? g.KP[0] : (ph == 1 ? g.KP[1] : g.KP[2]);
-        const double r = ph == 0 ? rc[0] : (ph == 1 ? rc[1] : rc[2]);
-        const double l = ph == 0 ? rl[0] : (ph == 1 ? rl[1] : rl[2]);
+        const double r = ph == 0 ? kr.rc[0] : (ph == 1 ? kr.rc[1] : kr.rc[2]);
+        const double l = ph == 0 ? kr.rl[0] : (ph == 1 ? kr.rl[1] : kr.rl[2]);
         for (int c = 0; c < 3; ++c) {
             const double t = (double)tau[((long long)slot * 3 + c) * g.N3 + i];
             const double q = fma(t, r, t * l);
@@ -255,7 +257,12 @@ void launch_e_to_tau(const GridDesc& g, int slot, const double* e, R* tau, cudaS
 }
 template <typename R>
 void launch_tau_to_e(const GridDesc& g, int slot, const R* tau, double* e, cudaStream_t st) {
-    k_tau_to_e<R><<<pointwise_blocks(g.N3), kThreads, 0, st>>>(g, slot, tau, e);
+    Reciprocals kr;
+    for (int p = 0; p < 3; ++p) {
+        kr.rc[p] = 1.0 / g.KP[p];
+        kr.rl[p] = std::fma(-kr.rc[p], g.KP[p], 1.0) * kr.rc[p];
+    }
+    k_tau_to_e<R><<<pointwise_blocks(g.N3), kThreads, 0, st>>>(g, kr, slot, tau, e);
 }
 void launch_widen(const GridDesc& g, unsigned mask, const float* src, double* dst, cudaStream_t st) {
     k_widen<<<dim3(pointwise_blocks(3 * g.N3), g.nslots), kThreads, 0, st>>>(g, mask, src, dst);
