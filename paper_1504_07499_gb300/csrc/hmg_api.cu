@@ -171,9 +171,7 @@ GridDesc make_desc(const GridPlan& gp, const double k[3], const uint8_t* phase_d
         g.relax = 1.0 - 0.5 * beta;
         g.epsf = 1.0 / (beta * k0);
     }
-    g.sn = std::ilogb((double)g.N3);
-    for (int p = 0; p < 3; ++p) g.YN[p] = std::ldexp(g.Y[p] * (1.0 / (double)g.N3), g.sn);
-    g.gcn = std::ldexp(g.gc, g.sn);
+    for (int p = 0; p < 3; ++p) g.YN[p] = std::ldexp(g.Y[p] * (1.0 / (double)g.N3), scale_bits(N));
     for (int s = 0; s < kMaxSlots; ++s)
         for (int c = 0; c < 3; ++c) g.E[s][c] = (s == c) ? 1.0 : 0.0;
     g.nslots = nslots;

@@ -240,7 +240,7 @@ k_fxx_inverse(GridDesc g, unsigned mask, int mode, const c64* spec, double* __re
     const bool bad = load_merge<M>(g, v, t, r, row, spec + row * M, key, e);
     c64 o[P::IL][P::RL];
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
-    if (mode != XI_PLAIN) e -= g.sn;
+    if (mode != XI_PLAIN) e -= scale_bits(N);
     // output step in FP64
     double2* out = reinterpret_cast<double2*>(tau) + row * M;
     float2* dout = reinterpret_cast<float2*>(d32) + row * M;
@@ -307,7 +307,7 @@ k_fxx_round(GridDesc g, unsigned mask, c64* spec, double* __restrict__ tau, doub
     int e;
     const bool bad = load_merge<M>(g, v, t, r, row, sp, key, e);
     transform<M, S>(v, o, t, r, sm, orm, RW, e, g.twf + N);
-    e -= g.sn;
+    e -= scale_bits(N);
     if (P::NS > 1) __syncthreads();   // the last stage has been read by every thread
     double2* out = reinterpret_cast<double2*>(tau) + row * M;
     const double cf[3] = {g.YN[0], g.YN[1], g.YN[2]};
@@ -564,7 +564,7 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
         for (int c = 0; c < 3; ++c) top = max(top, ez[c * NP + p] + bits_of(orm[2 * P3 + c * NP + p]));
         if (kx0 + p == 0 && ky == 0 && addb)   // room for the mean added at DC
             for (int c = 0; c < 3; ++c)
-                if (g.E[slot][c] != 0.0) top = max(top, ilogb(g.gcn * g.E[slot][c]) + 1);
+                if (g.E[slot][c] != 0.0) top = max(top, ilogb(g.gc * g.E[slot][c]) + scale_bits(N) + 1);
         return kx0 + p == 0 ? top + 1 : top;
     };
     auto column_bad = [&](int p) {
@@ -584,7 +584,8 @@ k_fxx_z(GridDesc g, unsigned mask, int mode, c64* __restrict__ spec, double* __r
             if (mode == Z_EQ) {
                 acc += eq_mode(kx, ky, kz, N, f[0], f[1], f[2]);
             } else {
-                const double cE[3] = {g.gcn * g.E[slot][0], g.gcn * g.E[slot][1], g.gcn * g.E[slot][2]};
+                constexpr double up = (double)(1LL << scale_bits(N));   // gc E in the spectrum's scale
+                const double cE[3] = {up * (g.gc * g.E[slot][0]), up * (g.gc * g.E[slot][1]), up * (g.gc * g.E[slot][2])};
                 green_mode<double>(kx, ky, kz, N, 1.0, g.ga, g.gb, addb, cE, f[0], f[1], f[2]);
                 for (int c = 0; c < 3; ++c) s[c] = mkc(to_fixed(f[c].x, eg), to_fixed(f[c].y, eg));
             }

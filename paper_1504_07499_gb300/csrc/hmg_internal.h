@@ -15,6 +15,13 @@ constexpr int kMaxSlots = 3;       // right-hand sides (unit gradients) per RVE
     X(8) X(12) X(16) X(18) X(24) X(32) X(36) X(48) X(54) X(64) X(72) X(96) X(108) X(128) X(144) X(162) \
     X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
 
+// floor(log2(N^3))
+constexpr int scale_bits(int N) {
+    int b = 0;
+    while ((long long)N * N * N >> (b + 1)) ++b;
+    return b;
+}
+
 // Everything a pass kernel needs about one RVE: sizes, transform tables, the
 // per-phase coefficient table, and the device fields (FP32 or FP64 copies).
 struct GridDesc {
@@ -31,11 +38,9 @@ struct GridDesc {
     // per-phase coefficients, k0 = sqrt(min k * max k):
     double Y[3];           // (k - k0)/(k + k0): polarization factor of the sweep
     // FP64 sweeps: the scale 1 / N^3 of the inverse transform, as a factor in (1/2, 1] on the way
-    // into the spectrum, YN = Y 2^sn / N^3, and 2^-sn on the way out (a change of exponent), so
-    // that small fields lose no bits to it
+    // into the spectrum, YN = Y 2^sn / N^3 with sn = scale_bits(N), and 2^-sn on the way out (a change
+    // of exponent), so that small fields lose no bits to it
     double YN[3];
-    double gcn;            // gc 2^sn
-    int sn;                // floor(log2(N^3))
     double W[3];           // k/(k + k0): flux factor, phi = W tau
     double KP[3];          // k + k0: tau = (k + k0) e
     double k0;
