@@ -1007,7 +1007,7 @@ struct PairShape {
 };
 
 template <int L, int MODE>
-__global__ void __launch_bounds__(128, 8)
+__global__ void __launch_bounds__(128, Split<L>::E > 8 ? 8 : 10)
 k_px_forward(GridDesc g, unsigned mask, const float* tau, float2* __restrict__ spec,
              double* __restrict__ partial) {
     using S = PairShape<L>;
